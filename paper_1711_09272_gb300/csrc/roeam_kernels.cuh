@@ -85,6 +85,10 @@ __device__ __forceinline__ float setle(float a, float b) { float r; asm("set.le.
 __device__ __forceinline__ float vabs(float a) { return fabsf(a); }
 __device__ __forceinline__ double vabs(double a) { return fabs(a); }
 __device__ __forceinline__ V2 vabs(V2 a) { return mk2(fabsf(a.v.x), fabsf(a.v.y)); }
+// -|a|
+__device__ __forceinline__ float vnabs(float a) { return -fabsf(a); }
+__device__ __forceinline__ double vnabs(double a) { return -fabs(a); }
+__device__ __forceinline__ V2 vnabs(V2 a) { return mk2(-fabsf(a.v.x), -fabsf(a.v.y)); }
 
 template <typename T> __device__ __forceinline__ bool lt(T a, T b) { return a < b; }
 template <typename T> __device__ __forceinline__ bool gt(T a, T b) { return a > b; }
@@ -164,31 +168,31 @@ template <typename V> __device__ __forceinline__ V sgnv(V a)
 }
 template <typename V> __device__ __forceinline__ V pow8(V a) { V a2 = a * a, a4 = a2 * a2; return a4 * a4; }
 
-// Eq. 98: f(phi) = min(phi sqrt(4 + (1 - phi^2)^2) / (1 + phi^2), 1). The argument is clamped
-// at 2 (f = 1 for every phi >= 1, and the clamp keeps the powers below in range), and the
-// square root and the division share one reciprocal square root:
-// sqrt(s) / q = s / sqrt(s q^2) with s = 4 + (1 - phi^2)^2, q = 1 + phi^2.
+// Eq. 98: f(phi) = min(phi sqrt(4 + (1 - phi^2)^2) / (1 + phi^2), 1). f(1) = 1 and f = 1 for every
+// phi >= 1, so the argument is clamped at 1 (and stays in range); the square root and the
+// division share one reciprocal square root: sqrt(s) / q = s / sqrt(s q^2) with
+// s = 4 + (phi^2 - 1)^2, q = 1 + phi^2.
 template <typename V> __device__ __forceinline__ V fmach(V phi)
 {
     const V one = splat<V>(1);
-    const V p = vmn(phi, splat<V>(2));
-    const V t = vfnma(p, p, one);
+    const V p = vmn(phi, one);
+    const V t = vfma(p, p, splat<V>(-1));
     const V s = vfma(t, t, splat<V>(4));
     const V q = vfma(p, p, one);
-    return vmn(p * s * rsq(s * q * q), one);
+    return (p * s) * rsq(s * q * q);
 }
 
-// Eq. 95 (with P values of Eq. 97 already reduced to their minimum a by Eq. 96). The
-// argument is a ratio of positive values (at most 1, plus the rounding of a reciprocal), so
-// Eq. 98 needs no clamp of its argument here; its result is still clamped at 1.
+// Eq. 95 (with P values of Eq. 97 already reduced to their minimum a by Eq. 96): f(a)^8. The
+// argument is a ratio of positive values (at most 1, plus the rounding of a reciprocal), so Eq. 98
+// needs no clamp here, and only even powers of f are wanted, so the square root drops out:
+// f^2 = x (x^2 - 2 x + 5) / (1 + x)^2 with x = a^2 (4 + (1 - x)^2 = x^2 - 2 x + 5).
 template <typename V> __device__ __forceinline__ V detector_of(V a)
 {
-    const V one = splat<V>(1);
-    const V t = vfnma(a, a, one);
-    const V s = vfma(t, t, splat<V>(4));
-    const V q = vfma(a, a, one);
-    const V f = vmn(a * s * rsq(s * q * q), one);
-    return sel(ge(a, one), one, pow8(f));
+    const V x = a * a;
+    const V n = x * vfma(x, x + splat<V>(-2), splat<V>(5));
+    const V r = rcp(x + splat<V>(1));
+    const V f2 = (n * r) * r, f4 = f2 * f2;
+    return f4 * f4;
 }
 
 // Mirror image of a velocity about a unit normal (wall ghost state).
@@ -241,21 +245,29 @@ struct Variant { int scheme = 0, dup_mode = 0, ufix = 1, xi_roe = 0; };
 // floor with Eqs. 102-109), delta p_p + delta p_u (Eqs. 87-88), rho delta U_p (Eq. 89 with
 // Eqs. 99-101), delta U_u (Eqs. 90-91), assembled as Eq. 85 with the energy convention of
 // Eq. 49. With ABL the Variant switches apply (scalar V only).
+// The FP32 kernels that evaluate it are bound by instruction issue, so the terms share their
+// parts: normalised Roe weights (one operation fewer per average), c~ and |U~| by way of
+// h = (1 - theta) |U| / 2, one reciprocal for 1 / (theta c^2), Eq. 98 clamped once, Eq. 95
+// without the square root; about 30 of 400 instructions per lane and row. 512-grid batch, 8 steps
+// with the state loaded and read back: 9159 -> 8840 us; 4096^2 warped step, 4 steps: 8109 -> 7968
+// us; FP64 64^2 vortex, 20 steps: 3931 -> 3701 us.
 template <bool ABL = false, typename V, typename S>
 __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1, const GridCoef<S> &K, int eps1,
                                             int xi_form, V F[4], const Variant &var = Variant())
 {
     const V zero = splat<V>(0), one = splat<V>(1), half = splat<V>(S(0.5));
 
-    // Roe averages; c^2 in the sum-of-positives form (no cancellation at high Mach).
+    // Roe averages with normalised weights, each one product and one fused multiply-add; c^2 in
+    // the sum-of-positives form (no cancellation at high Mach or across large jumps).
     const V w = rcp(L.sr + R.sr);
+    const V wl = L.sr * w, wr = R.sr * w;
     const V rh = L.sr * R.sr;
-    const V uh = vfma(L.sr, L.un, R.sr * R.un) * w;
-    const V vh = vfma(L.sr, L.ut, R.sr * R.ut) * w;
-    const V Hh = vfma(L.sr, L.H, R.sr * R.H) * w;
+    const V uh = vfma(wl, L.un, wr * R.un);
+    const V vh = vfma(wl, L.ut, wr * R.ut);
+    const V Hh = vfma(wl, L.H, wr * R.H);
     const V du = R.un - L.un, dv = R.ut - L.ut;
     const V dq2 = vfma(du, du, dv * dv);
-    const V c2h = vfma(splat<V>(K.hgm1) * rh * w, dq2, vfma(L.sr, L.c2, R.sr * R.c2)) * w;
+    const V c2h = vfma(splat<V>(K.hgm1) * wl * wr, dq2, vfma(wl, L.c2, wr * R.c2));
     const V chi = rsq(c2h);
     const V ch = c2h * chi;
     const V aU = vabs(uh);
@@ -309,7 +321,7 @@ __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1
 
     // xi's factor [1 - f^8(Mbar)] / 2 on dU (1/2 with xi_form = 1)
     const V xfh = xi_form ? half : vfma(splat<V>(S(-0.5)), fMb8, half);
-    V xi = vmx(vfma(xfh, du, vabs(half * (L.un + R.un))), zero);
+    V xi = vmx(vfma(xfh, du, vabs(vfma(half, du, L.un))), zero);
     if (eps1) {
         // Rotated-Riemann estimate in the face frame (n = (1, 0)): n1 = dq / |dq| unless
         // |dq| < 1e-5 U_ref; |alpha1 U1| + |alpha2 U2| with the unit n2 perpendicular to n1.
@@ -330,17 +342,18 @@ __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1
     const V smc = vcopysign(mn, uh) * chi;
     const V pp = vfma(smc, dp, vfma(s1, fM, one - s1) * vmx(ch - Up, zero) * rh * du);
     const V th = vmn(vmx(splat<V>(K.mr2), M * M), one);
+    // Eqs. 89, 99-101: c~ = sqrt(((1 - theta) U / 2)^2 + theta c^2) =: sqrt(X) and
+    // |U~| = (1 + theta) |U| / 2 = |U| - h with h = (1 - theta) |U| / 2. U~ has the sign of U, so
+    // U sgn(U~) min(|U~|, c~) = |U| min(|U~|, c~), and (1 - theta) |U| / (2 c~) = h / sqrt(X).
     const V om = one - th;
-    const V ou = om * uh;
-    const V X = vfma(ou, ou, (splat<V>(4) * c2h) * th);
-    const V rX = rsq(X);           // 1 / (2 c~)
-    const V ct = half * X * rX;    // c~
-    // |U~| = (1 + theta) |U| / 2, and U sgn(U~) min(|U~|, c~) = |U| min(|U~|, c~): U~ has the
-    // sign of U
-    const V aUt = vfma(half, th, half) * aU;
-    const V term = vfma(om, vfnma(aU * rX, vmn(aUt, ct), Up), vmx(ct - Up, zero));
+    const V nh = vnabs(half * om * uh);   // -h
+    const V Z = c2h * th;
+    const V X = vfma(nh, nh, Z);
+    const V rX = rsq(X);           // 1 / c~
+    const V ct = X * rX;           // c~
+    const V term = vfma(nh, rX * vmn(aU + nh, ct), vfma(om, Up, vmx(ct - Up, zero)));
     // -rho delta U_p (the sign is taken into the factor 1 - f^8(M))
-    V nA = s1 * (fM8 - one) * term * dp * chi * chi * rcp(th);
+    V nA = s1 * (fM8 - one) * term * dp * rcp(Z);
     if constexpr (ABL) {
         if (var.dup_mode == 1) nA = zero;
         else if (var.dup_mode == 2) nA = -(vmx(ch - aU, zero) * dp * chi * chi);   // rho x Eq. 17
@@ -1040,7 +1053,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                 for (int k = 0; k < 4; ++k) {
                     const V2 A2 = mk2(Ax[k], Ay[k]), B2 = mk2(Bc[k], Bc[k]);
                     const V2 sg = limiter(vanleer, B2 - A2, mk2(Px_[k], Py_[k]) - B2);
-                    WRp[k] = B2 - half * sg;
+                    WRp[k] = vfma(mk2(-0.5f, -0.5f), sg, B2);
                     WLp[k] = vfma(half, mk2(shup(sg.v.x, 1), sy_prev[k]), A2);
                     sy_prev[k] = sg.v.y;
                 }
@@ -1125,11 +1138,11 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                         const WC<T> &self = Wn[H - 1];
                         const T Uw[4] = {self.r, self.q1, self.q2, self.q3};
                         for (int k = 0; k < 4; ++k) {
-                            // U^(k) of this cell: kept in the window (FP32 first order without
-                            // walls, +1.2 % on the benchmark batch; the walls and FP64 kernels then
-                            // spill), loaded above (reconstructing curvilinear), or loaded again
+                            // U^(k) of this cell: kept in the window (FP32 first-order Cartesian
+                            // without walls, +1.2 % on the benchmark batch; the curvilinear, walls
+                            // and FP64 kernels then spill), loaded above (reconstructing curvilinear), or loaded again
                             // (mostly an L1 hit)
-                            const T uk = (!MUSCL && !WALLS && sizeof(T) == 4) ? Uw[k]
+                            const T uk = (!MUSCL && !WALLS && !CURV && sizeof(T) == 4) ? Uw[k]
                                                             : ((MUSCL && CURV) ? Uk[k] : __ldg(DBG_LD(R, DB_SRC, R.src + x + k * R.plane)));
                             const T upd = vfma(dt * sc, D[k], uk);
                             out[k] = combine ? vfma(a.alpha, Un[k], a.beta * upd) : upd;
