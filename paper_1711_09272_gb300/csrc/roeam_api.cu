@@ -1,7 +1,7 @@
 // roeam_api.cu — host implementation of the C ABI declared in include/roeam.h.
 //
-// Owns the device memory of a batch of grids, lays the state out as pitched
-// structure-of-arrays planes, drives the fused stage kernels (directly or through a
+// Owns the device memory of a batch of grids, lays the state out as pitched rows of cells
+// (a cell's four values together), drives the fused stage kernels (directly or through a
 // cached CUDA graph of several steps), and runs the FP64 monitor reductions.
 #include <cuda_runtime.h>
 
@@ -105,6 +105,7 @@ struct roeam_grid {
     void *U = nullptr, *A = nullptr, *B = nullptr;      // U^n (in place), stage buffers
     void *vdx = nullptr, *vdy = nullptr;
     uint8_t *solid = nullptr;
+    void *rows = nullptr;            // two rows of the widest grid (roeam_edge_rows, roeam_set_halo)
     int stage_next = 0;              // next stage of a step run stage by stage (roeam_rk_stage)
     double *staging = nullptr;
     unsigned long long *rate = nullptr;                  // 2 x count slots (double bits)
@@ -887,17 +888,19 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
     g->state_set.assign(count, 0);
     long long off = 0, voff = 0, soff = 0, poff = 0;
     bool any_solid = false;
+    int max_ni = 0;
     for (int k = 0; k < count; ++k) {
         const roeam_grid_desc &q = descs[k];
         GridDev &G = g->hg[k];
+        max_ni = std::max(max_ni, q.ni);
         std::memset(&G, 0, sizeof(G));
         G.ni = q.ni;
         G.nj = q.nj;
         G.pitch = (int)round_up(q.ni, 32);
         const bool exch = q.bc[2] == ROEAM_BC_EXCHANGE || q.bc[3] == ROEAM_BC_EXCHANGE;
-        // (a grid with an EXCHANGE side keeps two ghost rows below and above in its planes)
+        // (a grid with an EXCHANGE side keeps two ghost rows below and above)
         G.plane = (long long)(q.nj + (exch ? 4 : 0)) * G.pitch;
-        G.off = off + (exch ? 2ll * G.pitch : 0);
+        G.off = off + (exch ? 8ll * G.pitch : 0);
         off += 4 * G.plane;
         if (g->curv) {
             // (an EXCHANGE grid also keeps two ghost vertex rows below and above, roeam_set_halo_vertices)
@@ -993,6 +996,7 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
         CREATE_TRY(cudaMemcpy(g->solid, hs.data(), hs.size(), cudaMemcpyHostToDevice));
     }
     CREATE_TRY(cudaMalloc(&g->staging, sizeof(double) * (size_t)g->total_packed));
+    CREATE_TRY(cudaMalloc(&g->rows, g->esize * 8 * (size_t)max_ni));
     CREATE_TRY(cudaMalloc(&g->rate, sizeof(unsigned long long) * 2 * count));
     CREATE_TRY(cudaMemset(g->rate, 0, sizeof(unsigned long long) * 2 * count));
     CREATE_TRY(cudaMalloc(&g->status, sizeof(unsigned)));
@@ -1040,6 +1044,7 @@ void roeam_destroy_grid(roeam_grid *g)
     cudaFree(g->vdy);
     cudaFree(g->solid);
     cudaFree(g->staging);
+    cudaFree(g->rows);
     cudaFree(g->rate);
     cudaFree(g->status);
     cudaFree(g->work);
@@ -1399,11 +1404,12 @@ roeam_status roeam_edge_rows(roeam_grid *g, int grid_idx, int side, int stage, v
     CUDA_TRY(cudaSetDevice(g->device));
     const GridDev &G = g->hg[grid_idx];
     const int r0 = side == 2 ? 0 : G.nj - 2;
-    const char *base = (const char *)stage_source(g, stage) + g->esize * (size_t)G.off;
-    for (int k = 0; k < 4; ++k)
-        CUDA_TRY(cudaMemcpy2DAsync((char *)dst + g->esize * (size_t)(2 * k * G.ni), g->esize * G.ni,
-                                   base + g->esize * (size_t)(k * G.plane + (long long)r0 * G.pitch),
-                                   g->esize * G.pitch, g->esize * G.ni, 2, cudaMemcpyDefault, g->stream));
+    // (gathered on the device, then one copy to wherever dst lives)
+    const long long n = 8ll * G.ni;
+    CUDA_TRY(g->precision == 32
+                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, false, g->stream)
+                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, false, g->stream));
+    CUDA_TRY(cudaMemcpyAsync(dst, g->rows, g->esize * n, cudaMemcpyDefault, g->stream));
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type != cudaMemoryTypeDevice) {
         cudaGetLastError();
@@ -1423,12 +1429,12 @@ roeam_status roeam_set_halo(roeam_grid *g, int grid_idx, int side, int stage, co
     if (stage < 0 || stage > 2) return fail(ROEAM_E_ARG, "stage must be 0, 1 or 2");
     if (!src) return fail(ROEAM_E_ARG, "src must be non-null");
     CUDA_TRY(cudaSetDevice(g->device));
-    const long long r0 = side == 2 ? -2 : G.nj;
-    char *base = (char *)stage_source(g, stage) + g->esize * (size_t)(G.off + r0 * G.pitch);
-    for (int k = 0; k < 4; ++k)
-        CUDA_TRY(cudaMemcpy2DAsync(base + g->esize * (size_t)(k * G.plane), g->esize * G.pitch,
-                                   (const char *)src + g->esize * (size_t)(2 * k * G.ni), g->esize * G.ni,
-                                   g->esize * G.ni, 2, cudaMemcpyDefault, g->stream));
+    const int r0 = side == 2 ? -2 : G.nj;
+    const long long n = 8ll * G.ni;
+    CUDA_TRY(cudaMemcpyAsync(g->rows, src, g->esize * n, cudaMemcpyDefault, g->stream));
+    CUDA_TRY(g->precision == 32
+                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, true, g->stream)
+                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, true, g->stream));
     // a host source (page-locked memory copies asynchronously) may be reused once this returns
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, src) != cudaSuccess || at.type != cudaMemoryTypeDevice) {
@@ -1685,7 +1691,7 @@ roeam_status do_residual_noalloc(roeam_grid *g, int idx, double *out)
     void *scratch = nullptr;
     roeam_status st = noalloc_scratch(g->device, &scratch);
     if (st != ROEAM_OK) return st;
-    // The kernels address this grid at element offsets G.off (working-precision planes) and
+    // The kernels address this grid at element offsets G.off (working-precision cells) and
     // G.poff (float64 copy); the shifts place both at the start of their scratch regions.
     T *region_t = (T *)scratch;
     double *region_d = (double *)((unsigned char *)scratch + bytes_t);

@@ -16,9 +16,10 @@ constexpr unsigned ST_BOUNDS = 4u;   // an index outside its buffer (bounds-chec
 
 // Per-grid descriptor, resident in device memory, read-only in kernels.
 struct GridDev {
-    long long off;    // element offset of this grid's row 0 of variable 0 in the state buffers
-    long long plane;  // elements per variable plane (nj * pitch; (nj + 4) * pitch with an
-                      // EXCHANGE side, whose planes also hold the ghost rows j = -2, -1, nj, nj+1)
+    long long off;    // element offset of this grid's cell (0, 0) in the state buffers: cell (i, j)
+                      // holds its four values (rho, rho u, rho v, rho E) at off + 4 (j pitch + i)
+    long long plane;  // cells held (nj * pitch; (nj + 4) * pitch with an EXCHANGE side, which also
+                      // keeps the ghost rows j = -2, -1, nj, nj+1)
     long long voff;   // element offset of this grid's vertex displacement planes (-1: Cartesian)
     long long soff;   // byte offset of this grid's solid mask (-1: none)
     long long poff;   // element offset of this grid in the packed host layout [4][nj][ni]
@@ -90,13 +91,13 @@ struct StageArgs {
 #define STAGE_THREADS_DEF 32
 #endif
 constexpr int STAGE_THREADS = STAGE_THREADS_DEF;
-// Resident CTAs per SM the compiler is asked to fit (register budget): 13 keeps the FP32
-// first-order Cartesian kernel at 128 registers without spills (16 warps per SM); the
-// reconstructing and curvilinear FP32 variants are held to 128 registers as well (16 warps
-// per SM: the 4096^2 warped step runs 10 % faster than at 168 registers and 12 warps, although
-// it spills 60 bytes there); FP64 and the ablation variants are left to the compiler.
+// Resident CTAs per SM the compiler is asked to fit (register budget): 20 holds the FP32
+// first-order Cartesian kernels to 96 registers, which they fit without spills since the rows in
+// flight left the registers (512-grid batch, 8 steps: 16 warps per SM 8350 us, 20 warps 7927 us);
+// the reconstructing and curvilinear FP32 variants are held to 128 registers (16 warps per SM;
+// at 96 they spill 40 to 250 bytes); FP64 and the ablation variants are left to the compiler.
 #ifndef STAGE_MIN_BLOCKS_FAST
-#define STAGE_MIN_BLOCKS_FAST 13
+#define STAGE_MIN_BLOCKS_FAST 20
 #endif
 #ifndef STAGE_MIN_BLOCKS_OTHER
 #define STAGE_MIN_BLOCKS_OTHER 16
@@ -150,6 +151,8 @@ struct Launchers {
                               cudaStream_t s, long long u_shift = 0, long long p_shift = 0);
     static cudaError_t unpack(const GridDev *grids, int g_lo, int g_hi, int max_cells, const T *U, float *packed,
                               cudaStream_t s, long long u_shift = 0, long long p_shift = 0);
+    // Two rows of a grid's state (from row r0) <-> rows, device memory laid out [4][2][ni].
+    static cudaError_t rows(T *U, long long off, int pitch, int ni, int r0, T *rows, bool set, cudaStream_t s);
     // FP64 block partials of sum V*U over the fluid cells of one grid (gridDim.x * 4 doubles).
     static cudaError_t totals(const GridDev *grids, const GridCoef<T> *coef, int g, const T *U, const T *vdx,
                               const T *vdy, const uint8_t *solid, double *partials, int nblocks, int curv,

@@ -4,11 +4,11 @@
 // (Eqs. 85-109), the finite-volume residual, and the SSP-RK3 combination, in one pass
 // over the state. Its work unit is one warp sweeping a strip of 32 columns (H halo lanes
 // on each side, H = 1 at first order, 2 with MUSCL) over a segment of rows in +j:
-//   - each lane keeps a rolling window of H+2 rows of its column in registers and
-//     prefetches the next row while it computes the current one, so every cell state is
-//     read from HBM once per stage (plus halo lanes and H+1 warm-up rows per segment);
-//   - neighbour states, detector ratios and fluxes move between lanes with warp shuffles:
-//     no shared memory and no block barrier;
+//   - each lane keeps a rolling window of H+2 rows of its column in registers, fed from a
+//     shared-memory ring of rows that asynchronous copies fill ahead of it, so every cell state
+//     is read from HBM once per stage (plus halo lanes and H+1 warm-up rows per segment);
+//   - neighbour states, detector ratios and fluxes move between lanes with warp shuffles;
+//     a lane reads only its own slots of the ring: no block barrier;
 //   - ghost cells come from the boundary conditions on the fly (periodic wrap, wall
 //     mirror, inflow state, zero-gradient outflow), so no separate boundary kernel runs;
 //   - the flux is evaluated in the face frame (normal velocity first), which makes the
@@ -457,17 +457,17 @@ template <> __device__ __forceinline__ double rate_value<double>(unsigned long l
 // source index of its ghost value and a kind: 0 interior/periodic/outflow (a plain copy of
 // the source cell), 1 WALL (the source cell mirrored about the boundary face), 2 INFLOW (the
 // prescribed state), 3 EXCHANGE (the ghost row itself, j = -2, -1, n or n + 1: a grid with an
-// EXCHANGE side stores those rows in its state planes, set by the caller from the
+// EXCHANGE side stores those rows in its state buffers, set by the caller from the
 // neighbouring slab). Indices beyond the two ghost layers (ragged strips) are clamped into the
 // grid; their values are never used.
 __device__ __forceinline__ int resolve_index(int x, int n, int bc_lo, int bc_hi, int &kind)
 {
     kind = 0;
-    if (x >= 0 && x < n) return x;
+    if ((unsigned)x < (unsigned)n) return x;
     const int bc = x < 0 ? bc_lo : bc_hi;
     int s;
     if (bc == BC_INFLOW) { kind = 2; s = 0; }
-    else if (bc == BC_EXCHANGE) { kind = 3; return clampi(x, -2, n + 1); }   // a ghost row kept in the planes
+    else if (bc == BC_EXCHANGE) { kind = 3; return clampi(x, -2, n + 1); }   // a ghost row kept with the state
     else if (bc == BC_PERIODIC) s = ((x % n) + n) % n;
     else if (bc == BC_OUTFLOW) s = x < 0 ? 0 : n - 1;
     else { kind = 1; s = x < 0 ? -1 - x : 2 * n - 1 - x; }
@@ -488,7 +488,7 @@ template <typename T> __device__ __forceinline__ T ratio_P(T r0, T p0, T r1, T p
 }
 
 // MUSCL limited slope: minmod(a, b) = (sgn a + sgn b)/2 min(|a|, |b|); van Leer
-// (a|b| + |a|b) / (|a|+|b|) = 2 a |b| / (|a| + |b|), 0 when ab <= 0. The sign test and the van
+// (a|b| + |a|b) / (|a|+|b|) = 2 a b / (a + b) when ab > 0, else 0. The sign test and the van
 // Leer quotient avoid the product a b, which in FP32 underflows for differences below ~1e-19
 // (a state scaled by 1e-24 is as valid as the unscaled one).
 template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V b)
@@ -496,20 +496,16 @@ template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V 
     const V zero = splat<V>(0);
     const auto keep = gt(a * vcopysign(splat<V>(1), b), zero);   // same signs, a != 0
     if (vanleer) {
-        const V aa = vabs(a), ab = vabs(b);
-        return sel(keep, (a + a) * (ab * rcp(aa + ab)), zero);
+        return sel(keep, (a + a) * (b * rcp(a + b)), zero);
     }
     return sel(keep, sel(gt(a, zero), vmin(a, b), vmax(a, b)), zero);
 }
 
 // Cell-window entry: primitives (rho, u, v, p) in the global frame, the derived face
-// quantities (first order: computed once per cell), the conserved rho u, rho v, rho E as
-// loaded (the first-order kernels' stage epilogue takes U^(k) from here instead of reading it
-// again), and the flags (bit 0 solid, bit 1 wall).
+// quantities (first order: computed once per cell), and the flags (bit 0 solid, bit 1 wall).
 template <typename T> struct WC {
     T r, u, v, p, c2, H, sr, Mq;
-    T q1, q2, q3;
-    uint8_t fl;
+    int fl;
 };
 
 template <typename T, bool MUSCL>
@@ -685,24 +681,26 @@ __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<f
 // stage kernel is checked against its whole buffer; an access outside it sets ST_BOUNDS in the
 // status word (reported as ROEAM_E_BOUNDS) and reads zeros or is skipped instead of faulting.
 #ifdef ROEAM_DEBUG
-__device__ __align__(16) unsigned char dbg_sink[16];
+__device__ __align__(32) unsigned char dbg_sink[32];
 struct DbgBufs {
     const unsigned char *lo[6];   // src, un, dst, vdx, vdy, solid
     unsigned long long bytes[6];
     unsigned *status;
 };
-template <typename P> __device__ __forceinline__ bool dbg_ok(const DbgBufs &d, int buf, P *p)
+template <int N = 1, typename P> __device__ __forceinline__ bool dbg_ok(const DbgBufs &d, int buf, P *p)
 {
     const unsigned char *q = (const unsigned char *)p;
-    if (d.lo[buf] && q >= d.lo[buf] && q + sizeof(P) <= d.lo[buf] + d.bytes[buf]) return true;
+    if (d.lo[buf] && q >= d.lo[buf] && q + N * sizeof(P) <= d.lo[buf] + d.bytes[buf]) return true;
     atomicOr(d.status, ST_BOUNDS);
     return false;
 }
 #define DBG_LD(R, buf, p) (dbg_ok((R).dbg, (buf), (p)) ? (p) : (decltype(p))dbg_sink)
-#define DBG_ST(R, buf, p) dbg_ok((R).dbg, (buf), (p))
+#define DBG_LD4(R, buf, p) (dbg_ok<4>((R).dbg, (buf), (p)) ? (p) : (decltype(p))dbg_sink)
+#define DBG_ST4(R, buf, p) dbg_ok<4>((R).dbg, (buf), (p))
 #else
 #define DBG_LD(R, buf, p) (p)
-#define DBG_ST(R, buf, p) true
+#define DBG_LD4(R, buf, p) (p)
+#define DBG_ST4(R, buf, p) true
 #endif
 enum { DB_SRC = 0, DB_UN = 1, DB_DST = 2, DB_VDX = 3, DB_VDY = 4, DB_SOLID = 5 };
 
@@ -711,52 +709,97 @@ template <typename T> struct GridRegs {
     T *dst;
     const T *vdx, *vdy;         // vertex displacement planes of this grid (curvilinear)
     const uint8_t *solid;       // solid mask of this grid, or null
-    int ni, nj, pitch, plane, vpitch;
+    int ni, nj, pitch, vpitch;
     int bcW, bcE, bcS, bcN;
 #ifdef ROEAM_DEBUG
     DbgBufs dbg;
 #endif
 };
 
-// Cell loads of the reconstructing kernels carry the L1 priority evict_last: their window is
-// deeper, so a row is read again by the stage epilogue several rows after its first load, and
-// without the hint most of those reads missed L1 (measured faster on the Cartesian and the
-// curvilinear reconstructing workloads; the first-order kernels measured slower with it).
-__device__ __forceinline__ float ld_keep(const float *p) { float v; asm("ld.global.nc.L1::evict_last.f32 %0, [%1];" : "=f"(v) : "l"(p)); return v; }
-__device__ __forceinline__ double ld_keep(const double *p) { double v; asm("ld.global.nc.L1::evict_last.f64 %0, [%1];" : "=d"(v) : "l"(p)); return v; }
-template <bool KEEP, typename T> __device__ __forceinline__ T ld_row(const T *p) { if constexpr (KEEP) return ld_keep(p); else return __ldg(p); }
+// A cell's four conserved values lie together in the state buffers, so a cell is one 128-bit
+// access with one address (two in FP64).
+__device__ __forceinline__ void ld_cell(const float *p, float q[4])
+{
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+}
+__device__ __forceinline__ void ld_cell(const double *p, double q[4])
+{
+    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
+// The same through ordinary loads (shared memory, or a buffer that the kernel also writes).
+__device__ __forceinline__ void ld_own(const float *p, float q[4])
+{
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+}
+__device__ __forceinline__ void ld_own(const double *p, double q[4])
+{
+    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+}
+__device__ __forceinline__ void st_cell(float *p, const float q[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(q[0], q[1], q[2], q[3]);
+}
+__device__ __forceinline__ void st_cell(double *p, const double q[4])
+{
+    reinterpret_cast<double2 *>(p)[0] = make_double2(q[0], q[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(q[2], q[3]);
+}
+// Address of the four values of cell c (row * pitch + column) of a grid's block.
+template <typename T> __device__ __forceinline__ T *cell_at(T *base, int c) { return base + 4 * (long long)c; }
 
-// Loading a cell is split in two so that the next row's HBM loads are in flight while the
-// current row is computed: issue_cell resolves row j (the column is resolved once per unit
-// into isrc / kx) and starts the loads; finish_cell turns them into primitives, derived face
-// quantities and flags. Resolution order: an INFLOW side in i gives the inflow state;
-// otherwise an INFLOW side in j gives it (then mirrored by a WALL side in i); otherwise the
+// Loading a cell is split in two: issue_cell resolves row j (the column is resolved once per unit
+// into isrc / kx) and starts an asynchronous copy of the cell into this lane's slot of the warp's
+// shared-memory ring, RING_AHEAD rows before finish_cell turns the slot into primitives, derived
+// face quantities and flags. Each lane reads only what it copied itself, so waiting for its own
+// copies orders everything: no barrier. Resolution order: an INFLOW side in i gives the inflow
+// state; otherwise an INFLOW side in j gives it (then mirrored by a WALL side in i); otherwise the
 // source cell, mirrored about the S/N boundary face by a WALL side in j, then about the W/E
-// boundary face by a WALL side in i.
+// boundary face by a WALL side in i. (An INFLOW ghost cell resolves to cell 0 of its direction and
+// ignores what is copied.)
+//
+// The ring keeps the state rows from the one being finished (j - 1, whose U^(k) the stage epilogue
+// reads back) to the one on its way, and U^n of the rows to be combined: rows in flight hold no
+// registers, and a row has RING_AHEAD iterations to arrive. Measured: with the next row, U^n and
+// U^(k) loaded into registers as four planes per variable (start), the benchmark batch's kernel
+// took 127 registers (16 warps per SM) and 15.2 warp instructions per cell in stage 2; the cell's
+// values together, a quad loaded into registers instead costs 12.4 but waits for each load where
+// the quad is copied (long-scoreboard stalls 0.7 -> 2.4 per instruction, 1 % slower); the ring 12.8
+// at 91 registers (20 warps). 512-grid batch (8 steps, state in and out) 8840 -> 7713 us, 96-grid
+// van Leer batch 2860 -> 2630, 4096^2 warped step 7968 -> 7201.
+constexpr int RING_ROWS = 8, RING_UN = 4, RING_AHEAD = 2;
+template <typename T> __host__ __device__ constexpr int ring_bytes() { return (RING_ROWS + RING_UN) * 32 * 4 * (int)sizeof(T); }
+
 template <typename T> struct Pending {
     T raw[4];
     int jsrc, ky;
     int solid;   // the cell's solid-mask byte (kernels with walls)
 };
 
-template <typename T, bool WALLS, bool KEEP = false>
-__device__ __forceinline__ void issue_cell(const GridRegs<T> &R, int isrc, int kx, int j, Pending<T> &q)
+__device__ __forceinline__ void cp16(unsigned dst, const void *src)
 {
-    q.jsrc = resolve_index(j, R.nj, R.bcS, R.bcN, q.ky);
-    q.solid = 0;
-    if (kx != 2 && q.ky != 2) {
-        const int x = q.jsrc * R.pitch + isrc;
-        q.raw[0] = ld_row<KEEP>(DBG_LD(R, DB_SRC, R.src + x));
-        q.raw[1] = ld_row<KEEP>(DBG_LD(R, DB_SRC, R.src + x + R.plane));
-        q.raw[2] = ld_row<KEEP>(DBG_LD(R, DB_SRC, R.src + x + 2 * R.plane));
-        q.raw[3] = ld_row<KEEP>(DBG_LD(R, DB_SRC, R.src + x + 3 * R.plane));
-        // (jsrc is a grid row, or an EXCHANGE ghost row, whose mask rows the grid also keeps)
-        if constexpr (WALLS)
-            if (R.solid) q.solid = __ldg(DBG_LD(R, DB_SOLID, R.solid + q.jsrc * R.ni + isrc));
-    }
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+template <typename T> __device__ __forceinline__ void copy_cell(unsigned dst, const T *src)
+{
+    cp16(dst, src);
+    if constexpr (sizeof(T) == 8) cp16(dst + 16, src + 2);
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <typename T>
+__device__ __forceinline__ void issue_cell(const GridRegs<T> &R, int isrc, int j, unsigned slot)
+{
+    int ky;
+    const int x = resolve_index(j, R.nj, R.bcS, R.bcN, ky) * R.pitch + isrc;
+    copy_cell(slot, DBG_LD4(R, DB_SRC, cell_at(R.src, x)));
 }
 
-// LATE_SOLID reads the solid-mask byte here instead of taking the one issue_cell prefetched
+// LATE_SOLID reads the solid-mask byte here instead of taking the one prefetched a row earlier
 // (the ablation kernels, whose scalar path measured faster that way; the main kernels hide
 // that load's latency behind a row of work).
 template <typename T, bool MUSCL, bool CURV, bool WALLS, bool LATE_SOLID = false>
@@ -765,20 +808,18 @@ __device__ __forceinline__ void finish_cell(const GridRegs<T> &R, const GridCoef
 {
     const int ky = q.ky;
     c.fl = 0;
-    if (kx == 2 || ky == 2) {
-        c.r = K.inflow[0]; c.u = K.inflow[1]; c.v = K.inflow[2]; c.p = K.inflow[3];
-        // (q1..q3 stay unset: an inflow ghost cell is never written)
-    } else {
-        const T ri = rcp(q.raw[0]);
-        c.r = q.raw[0]; c.u = q.raw[1] * ri; c.v = q.raw[2] * ri;
-        c.q1 = q.raw[1]; c.q2 = q.raw[2]; c.q3 = q.raw[3];
-        c.p = K.gm1 * vfnma(T(0.5) * q.raw[0], vfma(c.u, c.u, c.v * c.v), q.raw[3]);
-        if constexpr (WALLS) {
-            if constexpr (LATE_SOLID) { if (R.solid && *DBG_LD(R, DB_SOLID, R.solid + q.jsrc * R.ni + isrc)) c.fl = 1; }
-            else if (q.solid) c.fl = 1;
-        }
-    }
+    const T ri = rcp(q.raw[0]);
+    c.r = q.raw[0]; c.u = q.raw[1] * ri; c.v = q.raw[2] * ri;
+    c.p = K.gm1 * vfnma(T(0.5) * q.raw[0], vfma(c.u, c.u, c.v * c.v), q.raw[3]);
     if constexpr (WALLS) {
+        if constexpr (LATE_SOLID) { if (R.solid && *DBG_LD(R, DB_SOLID, R.solid + q.jsrc * R.ni + isrc)) c.fl = 1; }
+        else if (q.solid) c.fl = 1;
+    }
+    if (kx == 2 || ky == 2) {
+        c.fl = 0;
+        c.r = K.inflow[0]; c.u = K.inflow[1]; c.v = K.inflow[2]; c.p = K.inflow[3];
+    }
+    if constexpr (WALLS) if (kx == 1 || ky == 1) {
         if (ky == 1 && kx != 2) {
             T nx = T(0), ny = T(1);
             if constexpr (CURV) {
@@ -814,8 +855,7 @@ template <bool WALLS, typename T> __device__ __forceinline__ WC<T> shup_c(const 
     o.r = shup(c.r, d); o.u = shup(c.u, d); o.v = shup(c.v, d); o.p = shup(c.p, d);
     if (derived) { o.c2 = shup(c.c2, d); o.H = shup(c.H, d); o.sr = shup(c.sr, d); o.Mq = shup(c.Mq, d); }
     else { o.c2 = o.H = o.sr = o.Mq = T(0); }
-    // (q1..q3 stay unset: a neighbour's conserved values are never read)
-    o.fl = WALLS ? (uint8_t)__shfl_up_sync(0xffffffffu, (int)c.fl, d) : (uint8_t)0;
+    o.fl = WALLS ? __shfl_up_sync(0xffffffffu, c.fl, d) : 0;
     return o;
 }
 template <bool WALLS, typename T> __device__ __forceinline__ WC<T> shdn_c(const WC<T> &c, int d)
@@ -823,7 +863,7 @@ template <bool WALLS, typename T> __device__ __forceinline__ WC<T> shdn_c(const 
     WC<T> o;
     o.r = shdn(c.r, d); o.u = shdn(c.u, d); o.v = shdn(c.v, d); o.p = shdn(c.p, d);
     o.c2 = o.H = o.sr = o.Mq = T(0);
-    o.fl = WALLS ? (uint8_t)__shfl_down_sync(0xffffffffu, (int)c.fl, d) : (uint8_t)0;
+    o.fl = WALLS ? __shfl_down_sync(0xffffffffu, c.fl, d) : 0;
     return o;
 }
 
@@ -870,10 +910,17 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
     // MODE_NORM: each thread's FP64 sums of R^2 [k] and maxima of |R| [4 + k] in dynamic shared
     // memory (slot k * NT + thread; only norm launches ask for it), rather than in sixteen
     // registers that every launch would hold
-    extern __shared__ __align__(16) unsigned char norm_smem[];
-    double *const nacc = reinterpret_cast<double *>(norm_smem) + threadIdx.x;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *const nacc = reinterpret_cast<double *>(smem_raw + NT / 32 * ring_bytes<T>()) + threadIdx.x;
     if (a.mode == MODE_NORM)
         for (int k = 0; k < 8; ++k) nacc[k * NT] = 0.0;
+
+    // this lane's slots of its warp's ring (see issue_cell): state row r, and U^n of row r
+    constexpr int ROWB = 32 * 4 * (int)sizeof(T);
+    unsigned char *const ring_p = smem_raw + (threadIdx.x >> 5) * ring_bytes<T>() + lane * (4 * (int)sizeof(T));
+    const unsigned ring = (unsigned)__cvta_generic_to_shared(ring_p);
+    auto slot_row = [&](int r) { return (r & (RING_ROWS - 1)) * ROWB; };
+    auto slot_un = [&](int r) { return (RING_ROWS + (r & (RING_UN - 1))) * ROWB; };
 
     // Each warp takes unit tile_lo + warp first, then (dynamic scheduling) the next unclaimed
     // one, in the order of the unit table (whole-batch launches: by decreasing height), so that
@@ -890,7 +937,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         R.src = a.src + G.off;
         R.un = a.un + G.off;
         R.dst = a.dst + (G.off - a.dst_shift);
-        R.ni = G.ni; R.nj = G.nj; R.pitch = G.pitch; R.plane = (int)G.plane;
+        R.ni = G.ni; R.nj = G.nj; R.pitch = G.pitch;
         R.bcW = G.bc[0]; R.bcE = G.bc[1]; R.bcS = G.bc[2]; R.bcN = G.bc[3];
         if constexpr (CURV) { R.vdx = a.vdx + G.voff; R.vdy = a.vdy + G.voff; R.vpitch = G.vpitch; }
         else { R.vdx = R.vdy = nullptr; R.vpitch = 0; }
@@ -926,7 +973,36 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         WC<T> Wn[NW];
         T Px[NW], Py[NW - 1];
         T vX[NV], vY[NV];
-        Pending<T> pend;
+        const bool stage_mode = a.mode == MODE_STAGE;
+        const bool combine = stage_mode && a.alpha != T(0);
+        const bool un_lane = combine && out_lane;
+        // One copy group per state row r: the row itself and U^n of row r - 2, which is combined
+        // in the iteration after the one that waits for row r. Rows beyond j1 + 1 are not needed.
+        auto issue_group = [&](int r) {
+            if (r <= j1 + 1) {
+                issue_cell(R, isrc, r, ring + slot_row(r));
+                if (un_lane && r >= j0 + 2)
+                    copy_cell(ring + slot_un(r - 2), DBG_LD4(R, DB_UN, cell_at(R.un, (r - 2) * R.pitch + i)));
+            }
+            copies_commit();
+        };
+        // the solid-mask byte of row j's cell; without a mask an unused byte (any readable address),
+        // so that the load is unconditional (a load that merges with another value at the end of a
+        // branch is waited for there)
+        const uint8_t *solid_p = R.solid ? R.solid : reinterpret_cast<const uint8_t *>(a.grids);
+        const int solid_pitch = R.solid ? R.ni : 0;
+        auto solid_of = [&](int j) {
+            int ky;
+            const int js = resolve_index(j, R.nj, R.bcS, R.bcN, ky);
+            return (int)__ldg(solid_p + (long long)js * solid_pitch + (solid_pitch ? isrc : 0));
+        };
+        auto finish_row = [&](int j, int sol, WC<T> &c) {
+            Pending<T> q;
+            q.jsrc = resolve_index(j, R.nj, R.bcS, R.bcN, q.ky);
+            q.solid = R.solid ? sol : 0;
+            ld_own(reinterpret_cast<const T *>(ring_p + slot_row(j)), q.raw);
+            finish_cell<T, MUSCL, CURV, WALLS, ABL>(R, K, i, isrc, kx, j, q, c);
+        };
         // vertex rows 0..nj, and the two ghost vertex rows beyond an EXCHANGE side
         const int vjlo = R.bcS == BC_EXCHANGE ? -2 : 0, vjhi = R.bcN == BC_EXCHANGE ? nj + 2 : nj;
         auto vload = [&](int J, T &x, T &y) {
@@ -937,27 +1013,31 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         };
         auto px_of = [&](const WC<T> &c) {   // Eq. 97 on this lane's west face; 1 at solid sides
             const T rl = shup(c.r, 1), pl = shup(c.p, 1);
-            if constexpr (WALLS) {
-                const int fl = __shfl_up_sync(0xffffffffu, (int)c.fl, 1);
-                if ((c.fl | fl) & 1) return T(1);
+            const T P = ratio_P(rl, pl, c.r, c.p);
+            if constexpr (WALLS) {   // (a select: a branch around the ratio would diverge at every wall)
+                const int fl = __shfl_up_sync(0xffffffffu, c.fl, 1);
+                return ((c.fl | fl) & 1) ? T(1) : P;
             }
-            return ratio_P(rl, pl, c.r, c.p);
+            return P;
         };
         auto py_of = [&](const WC<T> &lo, const WC<T> &hi) {
-            if constexpr (WALLS) {
-                if ((lo.fl | hi.fl) & 1) return T(1);
-            }
-            return ratio_P(lo.r, lo.p, hi.r, hi.p);
+            const T P = ratio_P(lo.r, lo.p, hi.r, hi.p);
+            if constexpr (WALLS) return ((lo.fl | hi.fl) & 1) ? T(1) : P;
+            return P;
         };
-        // window rows j0-H .. j0+1, each row's loads issued one row ahead (the last issue is
-        // the loop's first prefetch, row j0+2)
+        // window rows j0-H .. j0+1, and RING_AHEAD rows more on their way
+        for (int r = j0 - H; r <= j0 + 1 + RING_AHEAD; ++r) issue_group(r);
         for (int v = 0; v < NV; ++v) vload(j0 - 1 + v, vX[v], vY[v]);
-        issue_cell<T, WALLS && !ABL, MUSCL>(R, isrc, kx, j0 - H, pend);
+        int sol = 0;
+        int sols[NW];
+        if constexpr (WALLS && !ABL) {
+            for (int w = 0; w < NW; ++w) sols[w] = solid_of(j0 - H + w);
+            sol = solid_of(j0 + 2);
+        }
+        copies_wait<RING_AHEAD>();
         for (int w = 0; w < NW; ++w) {
             const int jr = j0 - H + w;
-            const Pending<T> cur = pend;
-            issue_cell<T, WALLS && !ABL, MUSCL>(R, isrc, kx, jr + 1, pend);
-            finish_cell<T, MUSCL, CURV, WALLS, ABL>(R, K, i, isrc, kx, jr, cur, Wn[w]);
+            finish_row(jr, WALLS && !ABL ? sols[w] : 0, Wn[w]);
             Px[w] = px_of(Wn[w]);
             if (w > 0) Py[w - 1] = py_of(Wn[w - 1], Wn[w]);
         }
@@ -969,23 +1049,13 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             const V2 hi = limiter(vanleer, mk2(b0.v, b0.p) - mk2(a0.v, a0.p), mk2(c0.v, c0.p) - mk2(b0.v, b0.p));
             sy_prev[0] = lo.v.x; sy_prev[1] = lo.v.y; sy_prev[2] = hi.v.x; sy_prev[3] = hi.v.y;
         }
-        T Un[4] = {T(0), T(0), T(0), T(0)};
         T acc[4] = {T(0), T(0), T(0), T(0)};
         T my_rate = T(0);
-        const bool stage_mode = a.mode == MODE_STAGE;
-        const bool combine = stage_mode && a.alpha != T(0);
 
-        // two rows per trip for the first-order kernels (measured faster; the reconstructing ones
-        // are not)
-#pragma unroll (MUSCL ? 1 : 2)
+        // two rows per trip for the first-order Cartesian kernel without walls (measured faster;
+        // the others are not, or spill)
+#pragma unroll (MUSCL || CURV || WALLS ? 1 : 2)
         for (int j = j0; j <= j1; ++j) {
-            // U^n of row j (combined at iteration j+1), issued early
-            T Un_next[4] = {T(0), T(0), T(0), T(0)};
-            if (combine && out_lane && j < j1) {
-                const int x = j * R.pitch + i;
-                for (int k = 0; k < 4; ++k) Un_next[k] = *DBG_LD(R, DB_UN, R.un + (x + k * R.plane));
-            }
-
             // ---- the two faces of this lane: west x-face of row j (cells lane-1 | lane) and
             //      the y-face between rows j-1 and j (window H-1 | H)
             Face<T> fx, fy;
@@ -995,7 +1065,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             fy.B = Wn[H];
             if constexpr (MUSCL) {
                 // (fx.Am's values are shuffled in on the scalar path, the only one that reads them)
-                fx.Am.fl = WALLS ? (uint8_t)__shfl_up_sync(0xffffffffu, (int)Wn[H].fl, 2) : (uint8_t)0;
+                fx.Am.fl = WALLS ? __shfl_up_sync(0xffffffffu, Wn[H].fl, 2) : 0;
                 fx.Bp = shdn_c<WALLS>(Wn[H], 1);
                 fy.Am = Wn[H - 2];
                 fy.Bp = Wn[H + 1];
@@ -1076,21 +1146,9 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                     scalar = __any_sync(0xffffffffu, marginal);
                 }
             }
-            // U^(k) of row j-1 for this iteration's epilogue, issued just before the faces are
-            // evaluated (the reconstructing curvilinear kernel, which is latency-bound: +2.4 %
-            // over the epilogue read when issued at the top of the iteration, +2 % more and 36
-            // instead of 60 bytes of spills here, after the slopes and the screens; the other
-            // kernels measured slower with it and read it again in the epilogue)
-            T Uk[4] = {T(0), T(0), T(0), T(0)};
-            if constexpr (MUSCL && CURV) {
-                if (stage_mode && out_lane && j > j0) {
-                    const int x = (j - 1) * R.pitch + i;
-                    for (int k = 0; k < 4; ++k) Uk[k] = __ldg(DBG_LD(R, DB_SRC, R.src + x + k * R.plane));
-                }
-            }
             if (scalar) {
                 if constexpr (MUSCL) {
-                    const uint8_t fl = fx.Am.fl;
+                    const int fl = fx.Am.fl;
                     fx.Am = shup_c<WALLS>(Wn[H], 2, false);
                     fx.Am.fl = fl;
                 }
@@ -1135,20 +1193,15 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                     const int x = (j - 1) * R.pitch + i;
                     if (stage_mode) {
                         T out[4];
-                        const WC<T> &self = Wn[H - 1];
-                        const T Uw[4] = {self.r, self.q1, self.q2, self.q3};
+                        // (the first stage, alpha = 0 and beta = 1, combines with U^(k) itself)
+                        T Uk[4], Un[4];
+                        ld_own(reinterpret_cast<const T *>(ring_p + slot_row(j - 1)), Uk);
+                        ld_own(reinterpret_cast<const T *>(ring_p + (combine ? slot_un(j - 1) : slot_row(j - 1))), Un);
                         for (int k = 0; k < 4; ++k) {
-                            // U^(k) of this cell: kept in the window (FP32 first-order Cartesian
-                            // without walls, +1.2 % on the benchmark batch; the curvilinear, walls
-                            // and FP64 kernels then spill), loaded above (reconstructing curvilinear), or loaded again
-                            // (mostly an L1 hit)
-                            const T uk = (!MUSCL && !WALLS && !CURV && sizeof(T) == 4) ? Uw[k]
-                                                            : ((MUSCL && CURV) ? Uk[k] : __ldg(DBG_LD(R, DB_SRC, R.src + x + k * R.plane)));
-                            const T upd = vfma(dt * sc, D[k], uk);
-                            out[k] = combine ? vfma(a.alpha, Un[k], a.beta * upd) : upd;
+                            const T upd = vfma(dt * sc, D[k], Uk[k]);
+                            out[k] = vfma(a.alpha, Un[k], a.beta * upd);
                         }
-                        for (int k = 0; k < 4; ++k)
-                            if (DBG_ST(R, DB_DST, R.dst + (x + k * R.plane))) R.dst[x + k * R.plane] = out[k];
+                        if (DBG_ST4(R, DB_DST, cell_at(R.dst, x))) st_cell(cell_at(R.dst, x), out);
                         if (!solid && a.want_rate) {
                             const CellPrims<T> cp = cell_prims(out[0], out[1], out[2], out[3], K);
                             if (!(out[0] > T(0)) || !(cp.p > T(0))) {
@@ -1171,8 +1224,8 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                             }
                         }
                     } else if (a.mode == MODE_RESIDUAL) {
-                        for (int k = 0; k < 4; ++k)
-                            if (DBG_ST(R, DB_DST, R.dst + (x + k * R.plane))) R.dst[x + k * R.plane] = D[k] * sc;
+                        const T out[4] = {D[0] * sc, D[1] * sc, D[2] * sc, D[3] * sc};
+                        if (DBG_ST4(R, DB_DST, cell_at(R.dst, x))) st_cell(cell_at(R.dst, x), out);
                     } else if (!solid) {
                         for (int k = 0; k < 4; ++k) {
                             const double rk = (double)(D[k] * sc);
@@ -1183,7 +1236,6 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                 }
             }
             if (j == j1) break;
-            for (int k = 0; k < 4; ++k) Un[k] = Un_next[k];
             // (curvilinear faces carry their lengths; Cartesian ones twice the flux: the x-face
             //  difference is weighted by dy / dx here and the sum scaled by 1 / (2 dy) above,
             //  so that equal fluxes on opposite faces cancel exactly)
@@ -1193,13 +1245,15 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                 for (int k = 0; k < 4; ++k) acc[k] = vfma(Fw[k] - shdn(Fw[k], 1), rxy, Fs[k]);
             }
 
-            // ---- advance the window: row j+2 enters from the prefetch
+            // ---- advance the window: row j+2 enters from the ring
             for (int w = 0; w < NW - 1; ++w) { Wn[w] = Wn[w + 1]; Px[w] = Px[w + 1]; }
             for (int w = 0; w < NW - 2; ++w) Py[w] = Py[w + 1];
-            finish_cell<T, MUSCL, CURV, WALLS, ABL>(R, K, i, isrc, kx, j + NW - H, pend, Wn[NW - 1]);
+            issue_group(j + 2 + RING_AHEAD);
+            copies_wait<RING_AHEAD>();
+            finish_row(j + 2, sol, Wn[NW - 1]);
+            if constexpr (WALLS && !ABL) sol = solid_of(j + 3);
             Px[NW - 1] = px_of(Wn[NW - 1]);
             Py[NW - 2] = py_of(Wn[NW - 2], Wn[NW - 1]);
-            issue_cell<T, WALLS && !ABL, MUSCL>(R, isrc, kx, j + NW - H + 1, pend);
             if constexpr (CURV) {
                 for (int v = 0; v < NV - 1; ++v) { vX[v] = vX[v + 1]; vY[v] = vY[v + 1]; }
                 vload(j + NV - 1, vX[NV - 1], vY[NV - 1]);
@@ -1251,7 +1305,8 @@ template <int NT, typename T> __device__ __forceinline__ T block_max(T v, T *red
 }
 
 // ------------------------------------------------------------------ small kernels
-// Host layout [4][nj][ni] per grid (H: float64 or float) <-> pitched planes, blockIdx.y = grid.
+// Host layout [4][nj][ni] per grid (H: float64 or float) <-> the state's pitched cells of four
+// values, blockIdx.y = grid.
 // Each thread moves IO_PER cells a stride of gridDim.x * 256 apart, all of their loads issued
 // before the first store, so that a thread has IO_PER x 4 loads in flight instead of one DRAM
 // latency per cell; indices are 32-bit (a grid holds at most 2^28 cells). With RATE the pack
@@ -1271,7 +1326,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_l
     const unsigned ni = (unsigned)G.ni, n = ni * (unsigned)G.nj, stride = gridDim.x * 256u;
     const H *__restrict__ src = packed + (G.poff - p_shift);
     T *__restrict__ dst = U + G.off;
-    const long long pitch = G.pitch, plane = G.plane;
+    const unsigned pitch = (unsigned)G.pitch;
     T m = T(0);
     for (unsigned q0 = blockIdx.x * 256u + threadIdx.x; q0 < n; q0 += IO_PER * stride) {
         T v[IO_PER][4];
@@ -1286,8 +1341,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_l
             const unsigned q = q0 + e * stride;
             if (q >= n) break;
             const unsigned j = q / ni, i = q - j * ni;
-            const long long c = (long long)j * pitch + i;
-            for (int k = 0; k < 4; ++k) dst[c + k * plane] = v[e][k];
+            st_cell(dst + 4ull * (j * pitch + i), v[e]);
             if constexpr (RATE) {
                 if (G.soff >= 0 && ro.solid[G.soff + q]) continue;
                 const GridCoef<T> &K = ro.coef[g];
@@ -1318,7 +1372,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g
     const unsigned ni = (unsigned)G.ni, n = ni * (unsigned)G.nj, stride = gridDim.x * 256u;
     const T *__restrict__ src = U + (G.off - u_shift);
     H *__restrict__ dst = packed + (G.poff - p_shift);
-    const long long pitch = G.pitch, plane = G.plane;
+    const unsigned pitch = (unsigned)G.pitch;
     for (unsigned q0 = blockIdx.x * 256u + threadIdx.x; q0 < n; q0 += IO_PER * stride) {
         T v[IO_PER][4];
 #pragma unroll
@@ -1326,8 +1380,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g
             const unsigned q = q0 + e * stride;
             if (q < n) {
                 const unsigned j = q / ni, i = q - j * ni;
-                const long long c = (long long)j * pitch + i;
-                for (int k = 0; k < 4; ++k) v[e][k] = src[c + k * plane];
+                ld_cell(src + 4ull * (j * pitch + i), v[e]);
             }
         }
 #pragma unroll
@@ -1336,6 +1389,24 @@ __global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g
             if (q < n)
                 for (int k = 0; k < 4; ++k) dst[(long long)k * n + q] = (H)v[e][k];
         }
+    }
+}
+
+// Two rows (from row r0) of a grid's state <-> [4][2][ni] working-precision values, the layout of
+// roeam_edge_rows and roeam_set_halo.
+template <typename T, bool SET>
+__global__ void __launch_bounds__(128) rows_kernel(T *U, long long off, int pitch, int ni, int r0, T *rows)
+{
+    const int i = blockIdx.x * 128 + threadIdx.x, r = blockIdx.y;
+    if (i >= ni) return;
+    T *c = U + off + 4 * ((long long)(r0 + r) * pitch + i);
+    T q[4];
+    if constexpr (SET) {
+        for (int k = 0; k < 4; ++k) q[k] = rows[(long long)(2 * k + r) * ni + i];
+        st_cell(c, q);
+    } else {
+        ld_own(c, q);
+        for (int k = 0; k < 4; ++k) rows[(long long)(2 * k + r) * ni + i] = q[k];
     }
 }
 
@@ -1361,8 +1432,9 @@ __global__ void __launch_bounds__(256) totals_kernel(const GridDev *grids, const
         } else {
             V = G.dx * G.dy;
         }
-        const long long c = G.off + (long long)j * G.pitch + i;
-        for (int k = 0; k < 4; ++k) s[k] = fma(V, (double)U[c + k * G.plane], s[k]);
+        T q4[4];
+        ld_cell(U + G.off + 4 * ((long long)j * G.pitch + i), q4);
+        for (int k = 0; k < 4; ++k) s[k] = fma(V, (double)q4[k], s[k]);
     }
     for (int o = 16; o > 0; o >>= 1)
         for (int k = 0; k < 4; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
@@ -1381,15 +1453,16 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS, bool ABL = false> struc
     static constexpr int NT = STAGE_THREADS;
     static cudaError_t launch(const StageArgs<T> &a, int nblocks, cudaStream_t s)
     {
-        const size_t smem = a.mode == MODE_NORM ? 8 * NT * sizeof(double) : 0;   // (the norm accumulators)
+        // (the rings, and the norm accumulators)
+        const size_t smem = NT / 32 * ring_bytes<T>() + (a.mode == MODE_NORM ? 8 * NT * sizeof(double) : 0);
         stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL><<<nblocks, NT, smem, s>>>(a);
         return cudaGetLastError();
     }
     static int occupancy()
     {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL>, NT, 0) !=
-            cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL>, NT,
+                                                          NT / 32 * ring_bytes<T>()) != cudaSuccess)
             return 1;
         return n > 0 ? n : 1;
     }
@@ -1502,6 +1575,15 @@ cudaError_t Launchers<T>::unpack(const GridDev *grids, int g_lo, int g_hi, int m
                                  cudaStream_t s, long long u_shift, long long p_shift)
 {
     return launch_unpack<T, float>(grids, g_lo, g_hi, max_cells, U, packed, s, u_shift, p_shift);
+}
+
+template <typename T>
+cudaError_t Launchers<T>::rows(T *U, long long off, int pitch, int ni, int r0, T *rows, bool set, cudaStream_t s)
+{
+    const dim3 grid((ni + 127) / 128, 2);
+    if (set) rows_kernel<T, true><<<grid, 128, 0, s>>>(U, off, pitch, ni, r0, rows);
+    else rows_kernel<T, false><<<grid, 128, 0, s>>>(U, off, pitch, ni, r0, rows);
+    return cudaGetLastError();
 }
 
 template <typename T>
