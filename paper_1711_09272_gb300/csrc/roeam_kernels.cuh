@@ -52,6 +52,14 @@ template <> struct Sc<V2> { using S = float; using M = B2; };
 template <typename V> __device__ __forceinline__ V splat(typename Sc<V>::S c) { return V(c); }
 template <> __device__ __forceinline__ V2 splat<V2>(float c) { return mk2(c, c); }
 
+// FP64 comparisons, minima and maxima through the bit patterns. The FP64 pipe takes 16 to 19
+// cycles per warp instruction and SM, comparisons included, the integer pipes about 2.5 for a
+// 64-bit minimum; the bits of doubles compare like signed integers wherever at least one operand
+// is not negative, which holds at every call below (-0 < +0, and a NaN compares as large).
+__device__ __forceinline__ long long dbits(double a) { return __double_as_longlong(a); }
+__device__ __forceinline__ double imin(double a, double b) { return dbits(a) < dbits(b) ? a : b; }
+__device__ __forceinline__ double imax(double a, double b) { return dbits(a) < dbits(b) ? b : a; }
+
 template <typename T> __device__ __forceinline__ T vmin(T a, T b) { return a < b ? a : b; }
 template <typename T> __device__ __forceinline__ T vmax(T a, T b) { return a > b ? a : b; }
 __device__ __forceinline__ V2 vmin(V2 a, V2 b) { return mk2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y)); }
@@ -61,23 +69,23 @@ __device__ __forceinline__ V2 vmax(V2 a, V2 b) { return mk2(fmaxf(a.v.x, b.v.x),
 // of the detector, whose operands are never NaN, the results are the same; the three-operand
 // minimum is one instruction on sm_100-class GPUs.
 __device__ __forceinline__ float fmn(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double fmn(double a, double b) { return fmin(a, b); }
+__device__ __forceinline__ double fmn(double a, double b) { return imin(a, b); }
 __device__ __forceinline__ float fmx(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double fmx(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ double fmx(double a, double b) { return imax(a, b); }
 __device__ __forceinline__ float fmn3(float a, float b, float c)
 {
     float r;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ double fmn3(double a, double b, double c) { return fmin(fmin(a, b), c); }
-// Minimum and maximum inside the flux, whose operands are finite: single instructions for
-// every operand type (the V2 forms above already are).
+__device__ __forceinline__ double fmn3(double a, double b, double c) { return imin(imin(a, b), c); }
+// Minimum and maximum inside the flux, whose operands are finite and at least one of them not
+// negative: single instructions in FP32 (the V2 forms above already are), integer ones in FP64.
 __device__ __forceinline__ float vmn(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double vmn(double a, double b) { return fmin(a, b); }
+__device__ __forceinline__ double vmn(double a, double b) { return imin(a, b); }
 __device__ __forceinline__ V2 vmn(V2 a, V2 b) { return vmin(a, b); }
 __device__ __forceinline__ float vmx(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double vmx(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ double vmx(double a, double b) { return imax(a, b); }
 __device__ __forceinline__ V2 vmx(V2 a, V2 b) { return vmax(a, b); }
 // 1 where a < b (a <= b), else 0, as one instruction each (PTX set).
 __device__ __forceinline__ float setlt(float a, float b) { float r; asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
@@ -91,6 +99,7 @@ __device__ __forceinline__ double vnabs(double a) { return -fabs(a); }
 __device__ __forceinline__ V2 vnabs(V2 a) { return mk2(-fabsf(a.v.x), -fabsf(a.v.y)); }
 
 template <typename T> __device__ __forceinline__ bool lt(T a, T b) { return a < b; }
+__device__ __forceinline__ bool ge(double a, double b) { return dbits(a) >= dbits(b); }   // (b >= 0)
 template <typename T> __device__ __forceinline__ bool gt(T a, T b) { return a > b; }
 template <typename T> __device__ __forceinline__ bool ge(T a, T b) { return a >= b; }
 template <typename T> __device__ __forceinline__ bool eq(T a, T b) { return a == b; }
@@ -109,11 +118,12 @@ __device__ __forceinline__ V2 sel(B2 m, V2 a, V2 b) { return mk2(m.x ? a.v.x : b
 
 // Reciprocal, reciprocal square root and square root (of a non-negative value). FP32 uses
 // the single-instruction hardware approximations (PTX rcp/rsqrt/sqrt .approx). FP64 starts
-// from the hardware approximations (PTX rcp.approx.ftz.f64, rsqrt.approx.ftz.f64) and refines
-// them by two Newton-Raphson steps, each of which squares the relative error (y <- y + y e
-// with e = 1 - x y for 1/x, y <- y + y e / 2 with e = 1 - x y^2 for 1/sqrt(x)): within two
-// ulp of the correctly rounded results for the positive normal arguments the scheme produces
-// (roeam_math_check compares them with the IEEE operations), at a fraction of their cost.
+// from the hardware approximations (PTX rcp.approx.ftz.f64, rsqrt.approx.ftz.f64, good to about
+// 20 bits) and applies one third-order step, which cubes the relative error: with e = 1 - x y,
+// 1/x = y (1 + e + e^2 + ...), and with e = 1 - x y^2, 1/sqrt(x) = y (1 + e/2 + 3 e^2/8 + ...).
+// Three and five FP64 operations, against four and eight for two Newton steps; within two ulp of
+// the correctly rounded results for the positive normal arguments the scheme produces
+// (roeam_math_check compares them with the IEEE operations).
 __device__ __forceinline__ float rcp(float x)
 {
     float r;
@@ -136,21 +146,17 @@ __device__ __forceinline__ double rcp(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double e = fma(-x, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-x, y, 1.0);
-    return fma(y, e, y);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ double rsq(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double e = fma(-x * y, y, 1.0);
-    y = fma(0.5 * y, e, y);
-    e = fma(-x * y, y, 1.0);
-    return fma(0.5 * y, e, y);
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ double sqrt0(double x) { return x > 0.0 ? x * rsq(x) : 0.0; }
+__device__ __forceinline__ double sqrt0(double x) { return dbits(x) > 0 ? x * rsq(x) : 0.0; }
 __device__ __forceinline__ V2 rcp(V2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
 __device__ __forceinline__ V2 rsq(V2 x) { return mk2(rsq(x.v.x), rsq(x.v.y)); }
 __device__ __forceinline__ V2 sqrt0(V2 x) { return mk2(sqrt0(x.v.x), sqrt0(x.v.y)); }
@@ -226,7 +232,10 @@ __device__ __forceinline__ FS<V> side_from_prims(V r, V un, V ut, V p, const Gri
 // The bracket sgn(U + c) - sgn(U - c) of Eq. 92 for |U| and c >= 0: 2 for |U| < c, 1 for
 // |U| = c, 0 above (in FP32 as the sum of two set instructions).
 __device__ __forceinline__ float bracket(float aU, float c) { return setlt(aU, c) + setle(aU, c); }
-__device__ __forceinline__ double bracket(double aU, double c) { return aU < c ? 2.0 : (aU == c ? 1.0 : 0.0); }
+__device__ __forceinline__ double bracket(double aU, double c)
+{
+    return dbits(aU) < dbits(c) ? 2.0 : (dbits(aU) == dbits(c) ? 1.0 : 0.0);
+}
 __device__ __forceinline__ V2 bracket(V2 aU, V2 c)
 {
     return mk2(setlt(aU.v.x, c.v.x), setlt(aU.v.y, c.v.y)) + mk2(setle(aU.v.x, c.v.x), setle(aU.v.y, c.v.y));
@@ -480,11 +489,8 @@ template <typename T> __device__ __forceinline__ T shdn(T v, int d) { return __s
 
 template <typename T> __device__ __forceinline__ T ratio_P(T r0, T p0, T r1, T p1)
 {
-    // Eq. 97; in FP32 each ratio is the smaller value times the reciprocal of the larger
-    if constexpr (sizeof(T) == 4)
-        return fmn(fmn(p0, p1) * rcp(fmx(p0, p1)), fmn(r0, r1) * rcp(fmx(r0, r1)));
-    else
-        return fmn(fmn(p0, p1) / fmx(p0, p1), fmn(r0, r1) / fmx(r0, r1));
+    // Eq. 97; each ratio is the smaller value times the reciprocal of the larger
+    return fmn(fmn(p0, p1) * rcp(fmx(p0, p1)), fmn(r0, r1) * rcp(fmx(r0, r1)));
 }
 
 // MUSCL limited slope: minmod(a, b) = (sgn a + sgn b)/2 min(|a|, |b|); van Leer
@@ -499,6 +505,14 @@ template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V 
         return sel(keep, (a + a) * (b * rcp(a + b)), zero);
     }
     return sel(keep, sel(gt(a, zero), vmin(a, b), vmax(a, b)), zero);
+}
+
+// The same in FP64 with its sign tests on the bit patterns.
+template <> __device__ __forceinline__ double limiter<double>(bool vanleer, double a, double b)
+{
+    const bool keep = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && ((dbits(a) << 1) != 0);
+    const double m = vanleer ? (a + a) * (b * rcp(a + b)) : copysign(imin(fabs(a), fabs(b)), a);
+    return keep ? m : 0.0;
 }
 
 // Cell-window entry: primitives (rho, u, v, p) in the global frame, the derived face
