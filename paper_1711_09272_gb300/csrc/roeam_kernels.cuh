@@ -1171,10 +1171,11 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                     // the branch is warp-uniform, so the shuffles are safe here)
                     fx.nAmx = shup(fx.nx, 1); fx.nAmy = shup(fx.ny, 1);
                     fx.nBpx = shdn(fx.nx, 1); fx.nBpy = shdn(fx.ny, 1);
-                    const T x0 = shdn(vX[0], 1), y0 = shdn(vY[0], 1), x3 = shdn(vX[3], 1), y3 = shdn(vY[3], 1);
+                    // (vertex rows j - 1 and j + 1)
+                    const T x0 = shdn(vX[0], 1), y0 = shdn(vY[0], 1), x2 = shdn(vX[2], 1), y2 = shdn(vY[2], 1);
                     T tx = -(y0 - vY[0]), ty = K.dx + (x0 - vX[0]), l = rsq(vfma(tx, tx, ty * ty));
                     fy.nAmx = tx * l; fy.nAmy = ty * l;
-                    tx = -(y3 - vY[3]); ty = K.dx + (x3 - vX[3]); l = rsq(vfma(tx, tx, ty * ty));
+                    tx = -(y2 - vY[2]); ty = K.dx + (x2 - vX[2]); l = rsq(vfma(tx, tx, ty * ty));
                     fy.nBpx = tx * l; fy.nBpy = ty * l;
                 }
                 if constexpr (!PACKED || WALLS || MUSCL) {
