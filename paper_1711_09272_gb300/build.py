@@ -1,7 +1,7 @@
 """Compiles the CUDA library libroeam.so in-tree for sm_103a (GB300).
 
 The translation units (2D host ABI, FP32 and FP64 kernels, FP32 and FP64 ablation-variant
-kernels; 3D host ABI, FP32 and FP64 3D kernels) compile in parallel with nvcc and link into
+kernels, FP32 and FP64 tile kernels; 3D host ABI, FP32 and FP64 3D kernels) compile in parallel with nvcc and link into
 paper_1711_09272_gb300/_build/libroeam.so.
 """
 from __future__ import annotations
@@ -16,15 +16,16 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libroeam.so")
-SOURCES = ["roeam_api.cu", "roeam_k32.cu", "roeam_k64.cu", "roeam_k32_abl.cu", "roeam_k64_abl.cu", "roeam3_api.cu",
-           "roeam3_k32.cu", "roeam3_k64.cu"]
+SOURCES = ["roeam_api.cu", "roeam_k32.cu", "roeam_k64.cu", "roeam_k32_abl.cu", "roeam_k64_abl.cu", "roeam_t32.cu",
+           "roeam_t64.cu", "roeam3_api.cu", "roeam3_k32.cu", "roeam3_k64.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--prec-div=false", "--prec-sqrt=false",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 # The 2D translation units write every fused multiply-add out explicitly and forbid the
 # compiler from forming others, so that results are bit-identical across work-unit layouts
 # (tile shapes, row slabs) and across the copies of an unrolled loop body.
-EXACT_FMA = {"roeam_api.cu", "roeam_k32.cu", "roeam_k64.cu", "roeam_k32_abl.cu", "roeam_k64_abl.cu"}
+EXACT_FMA = {"roeam_api.cu", "roeam_k32.cu", "roeam_k64.cu", "roeam_k32_abl.cu", "roeam_k64_abl.cu", "roeam_t32.cu",
+             "roeam_t64.cu"}
 
 
 def nvcc() -> str:

@@ -47,7 +47,10 @@ roeam_status fail(roeam_status st, const char *fmt, ...)
 
 long long round_up(long long a, long long m) { return (a + m - 1) / m * m; }
 
-constexpr int GRAPH_STEPS = 8;   // SSP-RK3 steps per captured graph (an even number)
+constexpr int GRAPH_STEPS = 8;   // SSP-RK3 steps per captured graph (a multiple of RATE_SLOTS)
+// Rate slots per grid: step n reads slot n, writes slot n + 1 and (tile kernels, which have no
+// earlier launch of the same step to do it) clears slot n + 2, all modulo RATE_SLOTS.
+constexpr int RATE_SLOTS = 4;
 
 // NVTX range around a library call (visible in a profiler's timeline; free without one).
 struct Range {
@@ -63,7 +66,11 @@ constexpr size_t MAX_GRAPHS = 8; // captured graphs kept per handle (one per (cf
 
 struct GraphKey {
     double cfl, dt_fixed;
-    bool operator<(const GraphKey &o) const { return cfl < o.cfl || (cfl == o.cfl && dt_fixed < o.dt_fixed); }
+    const void *state;   // the buffer holding U^n (whole-step tile launches alternate between two)
+    bool operator<(const GraphKey &o) const
+    {
+        return cfl != o.cfl ? cfl < o.cfl : (dt_fixed != o.dt_fixed ? dt_fixed < o.dt_fixed : state < o.state);
+    }
 };
 
 }  // namespace
@@ -108,7 +115,13 @@ struct roeam_grid {
     void *rows = nullptr;            // two rows of the widest grid (roeam_edge_rows, roeam_set_halo)
     int stage_next = 0;              // next stage of a step run stage by stage (roeam_rk_stage)
     double *staging = nullptr;
-    unsigned long long *rate = nullptr;                  // 2 x count slots (double bits)
+    unsigned long long *rate = nullptr;                  // RATE_SLOTS x count slots (see rate_slot)
+    bool rate_clean = false;        // the next step's output slot is already zero (a tile step ran last)
+    // Tile kernels (see setup_tile_kernel): whether rk_step uses them, their work list and launch
+    bool tile_on = false;
+    int4 *d_rects = nullptr;
+    int nrects = 0, rect_threads = 0;
+    size_t rect_smem = 0;
     unsigned *status = nullptr;
     unsigned *work = nullptr;                            // dynamic unit-scheduling counters (2)
     double *partials = nullptr;
@@ -271,6 +284,101 @@ roeam_status setup_tiles(roeam_grid *g, int cfg)
     return ROEAM_OK;
 }
 
+// Whether roeam_rk_step runs this handle through the tile kernels, and their rectangles.
+//
+// Every grid is cut into rectangles of at most w x h cells of nearly equal size, one CTA each, and
+// (w, h) minimises an estimate of a step's cycles in which CTAs go over the SMs in rounds.
+// FP32 (a whole step per CTA): per stage a latency and the passes its face pairs take over an SM's
+// 128 lanes. Tiles are taken where that beats the strips' three launches of about 6 us each plus
+// their arithmetic. Measured, us per step, tiles / strips: periodic first order 128^2 6.3 / 16.8,
+// 256^2 9.9 / 20.1, 400^2 15.8 / 27.5, 700^2 40.9 / 45.8, 900^2 69 / 52; van Leer 256^2 12.9 / 24.5,
+// 512^2 35.6 / 39.5, 700^2 68 / 61; the estimates follow these within about 10 %, so the line lies
+// where both sides cost about the same.
+// FP64 (a stage per CTA): FP64 operations per face and cell, 76 cycles per warp on each of the four
+// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 168 / 277, 1024^2 2313 / 2696).
+// EXCHANGE sides (the caller sets ghost rows between stages) and the ablation kernels stay with the
+// strips.
+template <typename T>
+roeam_status setup_tile_kernel(roeam_grid *g)
+{
+    g->tile_on = false;
+    if (g->kind == KIND_ABLATION) return ROEAM_OK;
+    const int stages = tile_stages<T>(), H = g->muscl ? 2 : 1, E = H * stages;
+    const bool walls = g->kind == KIND_WALLS;
+    int max_ni = 0, max_nj = 0;
+    double cells = 0;
+    for (const GridDev &G : g->hg) {
+        for (int s = 0; s < 4; ++s)
+            if (G.bc[s] == ROEAM_BC_EXCHANGE) return ROEAM_OK;
+        max_ni = std::max(max_ni, G.ni);
+        max_nj = std::max(max_nj, G.nj);
+        cells += (double)G.ni * G.nj;
+    }
+    if (stages == 3 && cells > 1.5e6) return ROEAM_OK;   // (strips win well below this)
+    const double slow = g->curv ? 1.28 : (walls ? 1.18 : 1.0);
+    const int every = 1 + (g->count - 1) / 256;           // (a sample of a large batch's grids)
+    double best = 1e300;
+    int bw = 0, bh = 0;
+    for (int w = 64; w >= 4; --w)   // (of equal estimates the widest: 32 x 14 runs the 256^2 Gresho step in
+        for (int h = 2; h <= 64; ++h) {   // 13.0 us, 16 x 32 in 14.3)
+            if (w > max_ni + 3 || h > max_nj + 1) continue;
+            const size_t smem = tile_bytes<T>(w + 2 * E, h + 2 * E, g->muscl, g->curv, walls, stages);
+            if (smem > TILE_SMEM_MAX) continue;
+            double t = 0;
+            if (stages == 3) {
+                for (int s = 0; s < stages; ++s) {
+                    const int e = H * (stages - 1 - s);
+                    const double pairs = (double)(w + 2 * e + 1) * (h + 2 * e + 1);
+                    t += 2100 + std::ceil(pairs / 128) * (g->muscl ? 1030 : 750) * slow;
+                }
+            } else {
+                const double faces = (double)(w + 1) * h + (double)w * (h + 1);
+                const double pos = (double)(w + 2 * H) * (h + 2 * H), own = (double)w * h;
+                t = 76 * ((g->muscl ? 185 : 133) * std::ceil(faces / 128) + (g->muscl ? 13 : 40) * std::ceil(pos / 128) +
+                          ((g->muscl ? 60 : 10) + 32) * std::ceil(own / 128));
+
+            }
+            if (t >= best) continue;   // (at least one round)
+            double tiles = 0;
+            for (int k = 0; k < g->count; k += every)
+                tiles += (double)every * ((g->hg[k].ni + w - 1) / w) * ((g->hg[k].nj + h - 1) / h);
+            const double cost = std::ceil(tiles / g->num_sms) * t;
+            if (cost < best * 0.999) { best = cost; bw = w; bh = h; }
+        }
+    if (bw == 0) return ROEAM_OK;
+    if (stages == 3) {
+        const double strips = 36000.0 + cells * (g->muscl ? 0.18 : 0.1) * (g->curv ? 1.35 : (walls ? 1.1 : 1.0));
+        if (best + 2500.0 > strips) return ROEAM_OK;
+    }
+    std::vector<int4> rects;
+    int mw = 0, mh = 0;
+    for (int k = 0; k < g->count; ++k) {
+        const GridDev &G = g->hg[k];
+        const int nx = (G.ni + bw - 1) / bw, ny = (G.nj + bh - 1) / bh;
+        for (int y = 0; y < ny; ++y)
+            for (int x = 0; x < nx; ++x) {
+                const int x0 = (int)((long long)x * G.ni / nx), x1 = (int)((long long)(x + 1) * G.ni / nx);
+                const int y0 = (int)((long long)y * G.nj / ny), y1 = (int)((long long)(y + 1) * G.nj / ny);
+                rects.push_back(make_int4(k, x0, y0, (x1 - x0) | ((y1 - y0) << 16)));
+                mw = std::max(mw, x1 - x0);
+                mh = std::max(mh, y1 - y0);
+            }
+    }
+    g->nrects = (int)rects.size();
+    g->rect_smem = tile_bytes<T>(mw + 2 * E, mh + 2 * E, g->muscl, g->curv, walls, stages);
+    const int positions = (mw + 2 * E) * (mh + 2 * E);
+    g->rect_threads = std::min(tile_threads<T>(), std::max(128, (positions + 31) / 32 * 32));
+    // One CTA per SM where that holds them all: with room for a second, the next launch's CTAs (which
+    // come early, and wait) pair up on the SMs that are idle now (64^2 FP64 vortex, 20 steps: 855 us,
+    // 682 us with the room taken).
+    if (g->nrects <= g->num_sms) g->rect_smem = std::max(g->rect_smem, (size_t)115 * 1024);
+    CUDA_TRY(TileLaunchers<T>::prepare(g->muscl, g->curv, walls));
+    CUDA_TRY(cudaMalloc(&g->d_rects, sizeof(int4) * rects.size()));
+    CUDA_TRY(cudaMemcpy(g->d_rects, rects.data(), sizeof(int4) * rects.size(), cudaMemcpyHostToDevice));
+    g->tile_on = true;
+    return ROEAM_OK;
+}
+
 // roeam_step_host's unit table: the units of every chunk of grids, cut with the current tile
 // shape's segment height halved (down to MIN_SEGMENT_ROWS) until the chunk alone has a unit for every
 // resident warp, ordered by decreasing height within the chunk.
@@ -420,12 +528,60 @@ StageArgs<T> base_args(roeam_grid *g)
     return a;
 }
 
+unsigned long long *rate_slot(roeam_grid *g, long long step)
+{
+    return g->rate + (size_t)(step & (RATE_SLOTS - 1)) * g->count;
+}
+
+// One SSP-RK3 step through the tile kernels. `state` is the buffer holding U^n; a whole-step launch
+// (FP32) leaves U^(n+1) in `other`, stage launches (FP64) update `state` in place.
+template <typename T>
+roeam_status launch_tile_step(roeam_grid *g, cudaStream_t s, long long step, double cfl, double dt_fixed, void *state,
+                              void *other)
+{
+    TileArgs<T> a;
+    std::memset(&a, 0, sizeof(a));
+    a.grids = g->d_grids;
+    a.coef = (const GridCoef<T> *)g->d_coef;
+    a.tiles = g->d_rects;
+    a.ngrids = g->count;
+    a.vdx = (const T *)g->vdx;
+    a.vdy = (const T *)g->vdy;
+    a.solid = g->solid;
+    a.rate_rd = rate_slot(g, step);
+    a.rate_wr = rate_slot(g, step + 1);
+    a.cfl_t = T(cfl);
+    a.dt_fixed_t = T(dt_fixed);
+    a.status = g->status;
+#ifdef ROEAM_DEBUG
+    a.n_state = g->total_elems;
+    a.n_vert = g->total_vert;
+    a.n_solid = g->total_solid;
+#endif
+    T *U = (T *)state, *A = (T *)other, *B = (T *)g->B;
+    const auto run = [&]() {
+        return TileLaunchers<T>::step(a, g->muscl, g->curv, g->kind == KIND_WALLS, g->nrects, g->rect_threads,
+                                      g->rect_smem, s);
+    };
+    a.un = U;
+    if (tile_stages<T>() == 3) {
+        a.src = U; a.dst = A; a.want_rate = 1; a.rate_zero = rate_slot(g, step + 2);
+        CUDA_TRY(run());
+        return ROEAM_OK;
+    }
+    a.src = U; a.dst = A; a.alpha = T(0); a.beta = T(1); a.rate_zero = rate_slot(g, step + 2);
+    CUDA_TRY(run());
+    a.src = A; a.dst = B; a.alpha = T(0.75); a.beta = T(0.25); a.rate_zero = nullptr;
+    CUDA_TRY(run());
+    a.src = B; a.dst = U; a.alpha = T(1.0 / 3.0); a.beta = T(2.0 / 3.0); a.want_rate = 1;
+    CUDA_TRY(run());
+    return ROEAM_OK;
+}
+
 template <typename T>
 roeam_status launch_step(roeam_grid *g, cudaStream_t s, long long step, double cfl, double dt_fixed)
 {
-    const int par = (int)(step & 1);
-    unsigned long long *rd = g->rate + (size_t)par * g->count;
-    unsigned long long *wr = g->rate + (size_t)(1 - par) * g->count;
+    unsigned long long *rd = rate_slot(g, step), *wr = rate_slot(g, step + 1);
     T *U = (T *)g->U, *A = (T *)g->A, *B = (T *)g->B;
     StageArgs<T> a = base_args<T>(g);
     a.mode = MODE_STAGE;
@@ -451,7 +607,7 @@ roeam_status launch_step(roeam_grid *g, cudaStream_t s, long long step, double c
 template <typename T>
 roeam_status rate_out(roeam_grid *g, int lo, int hi, cudaStream_t s, RateOut<T> &ro)
 {
-    unsigned long long *slot = g->rate + (size_t)(g->step & 1) * g->count;
+    unsigned long long *slot = rate_slot(g, g->step);
     CUDA_TRY(cudaMemsetAsync(slot + lo, 0, sizeof(unsigned long long) * (hi - lo), s));
     ro.coef = (const GridCoef<T> *)g->d_coef;
     ro.vdx = (const T *)g->vdx;
@@ -466,20 +622,28 @@ template <typename T>
 roeam_status rk_steps(roeam_grid *g, double cfl, double dt_fixed, int nsteps)
 {
     int left = nsteps;
+    const bool swaps = g->tile_on && tile_stages<T>() == 3;   // the state moves between U and A
+    const int per_step = swaps ? 1 : 3;                        // launches
+    if (left > 0 && g->tile_on && !g->rate_clean)
+        CUDA_TRY(cudaMemsetAsync(rate_slot(g, g->step + 1), 0, sizeof(unsigned long long) * g->count, g->stream));
+    if (left > 0) g->rate_clean = g->tile_on;
     auto direct = [&]() -> roeam_status {
-        roeam_status st = launch_step<T>(g, g->stream, g->step, cfl, dt_fixed);
+        roeam_status st = g->tile_on ? launch_tile_step<T>(g, g->stream, g->step, cfl, dt_fixed, g->U, g->A)
+                                     : launch_step<T>(g, g->stream, g->step, cfl, dt_fixed);
         if (st != ROEAM_OK) return st;
+        if (swaps) std::swap(g->U, g->A);
         g->step += 1;
-        g->launches += 3;
+        g->launches += per_step;
         left -= 1;
         return ROEAM_OK;
     };
-    if (left > 0 && (g->step & 1)) {
+    // (a graph's rate slots start at slot 0)
+    while (left >= GRAPH_STEPS && (g->step & (RATE_SLOTS - 1))) {
         roeam_status st = direct();
         if (st != ROEAM_OK) return st;
     }
     if (left >= GRAPH_STEPS) {
-        GraphKey key{cfl, dt_fixed};
+        GraphKey key{cfl, dt_fixed, g->U};
         auto it = g->graphs.find(key);
         if (it == g->graphs.end() && g->graphs.size() >= MAX_GRAPHS) {
             // keep the cache small: a caller that varies dt_fixed call by call rebuilds graphs
@@ -491,7 +655,10 @@ roeam_status rk_steps(roeam_grid *g, double cfl, double dt_fixed, int nsteps)
             cudaGraph_t graph;
             CUDA_TRY(cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeThreadLocal));
             for (int s = 0; s < GRAPH_STEPS; ++s) {
-                roeam_status st = launch_step<T>(g, g->cap_stream, s, cfl, dt_fixed);
+                roeam_status st = g->tile_on ? launch_tile_step<T>(g, g->cap_stream, s, cfl, dt_fixed,
+                                                                   swaps && (s & 1) ? g->A : g->U,
+                                                                   swaps && (s & 1) ? g->U : g->A)
+                                             : launch_step<T>(g, g->cap_stream, s, cfl, dt_fixed);
                 if (st != ROEAM_OK) {
                     graph = nullptr;
                     cudaStreamEndCapture(g->cap_stream, &graph);
@@ -509,7 +676,7 @@ roeam_status rk_steps(roeam_grid *g, double cfl, double dt_fixed, int nsteps)
         while (left >= GRAPH_STEPS) {
             CUDA_TRY(cudaGraphLaunch(it->second, g->stream));
             g->step += GRAPH_STEPS;
-            g->launches += 3 * GRAPH_STEPS;
+            g->launches += per_step * GRAPH_STEPS;
             left -= GRAPH_STEPS;
         }
     }
@@ -751,9 +918,7 @@ namespace {
 template <typename T>
 roeam_status do_stage(roeam_grid *g, int stage, double dt, int part = 0)
 {
-    const int par = (int)(g->step & 1);
-    unsigned long long *rd = g->rate + (size_t)par * g->count;
-    unsigned long long *wr = g->rate + (size_t)(1 - par) * g->count;
+    unsigned long long *rd = rate_slot(g, g->step), *wr = rate_slot(g, g->step + 1);
     T *U = (T *)g->U, *A = (T *)g->A, *B = (T *)g->B;
     StageArgs<T> a = base_args<T>(g);
     a.mode = MODE_STAGE;
@@ -773,6 +938,7 @@ roeam_status do_stage(roeam_grid *g, int stage, double dt, int part = 0)
         a.tile_lo = part == 1 ? 0 : g->part_split;
         a.tile_hi = part == 1 ? g->part_split : g->total_tiles;
     }
+    g->rate_clean = false;
     if (a.tile_hi > a.tile_lo) {
         CUDA_TRY(Launchers<T>::stage(a, g->muscl, g->curv, g->kind, g->nblocks, g->stream));
         g->launches += 1;
@@ -824,9 +990,8 @@ roeam_status pipe_chunk(roeam_grid *g, int chunk, int lo, int hi, int nsteps, do
     a.cfl_t = T(cfl);
     a.dt_fixed_t = T(dt_fixed);
     for (long long st = g->step; st < g->step + nsteps; ++st) {
-        const int par = (int)(st & 1);
-        a.rate_rd = g->rate + (size_t)par * g->count;
-        unsigned long long *wr = g->rate + (size_t)(1 - par) * g->count;
+        a.rate_rd = rate_slot(g, st);
+        unsigned long long *wr = rate_slot(g, st + 1);
         CUDA_TRY(cudaMemsetAsync(wr + lo, 0, sizeof(unsigned long long) * (hi - lo), s));
         a.rate_zero = nullptr;
         a.src = U; a.un = U; a.dst = A; a.alpha = T(0); a.beta = T(1); a.want_rate = 0; a.rate_wr = nullptr;
@@ -997,8 +1162,8 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
     }
     CREATE_TRY(cudaMalloc(&g->staging, sizeof(double) * (size_t)g->total_packed));
     CREATE_TRY(cudaMalloc(&g->rows, g->esize * 8 * (size_t)max_ni));
-    CREATE_TRY(cudaMalloc(&g->rate, sizeof(unsigned long long) * 2 * count));
-    CREATE_TRY(cudaMemset(g->rate, 0, sizeof(unsigned long long) * 2 * count));
+    CREATE_TRY(cudaMalloc(&g->rate, sizeof(unsigned long long) * RATE_SLOTS * count));
+    CREATE_TRY(cudaMemset(g->rate, 0, sizeof(unsigned long long) * RATE_SLOTS * count));
     CREATE_TRY(cudaMalloc(&g->status, sizeof(unsigned)));
     CREATE_TRY(cudaMemset(g->status, 0, sizeof(unsigned)));
     CREATE_TRY(cudaMalloc(&g->work, 2 * sizeof(unsigned)));
@@ -1013,6 +1178,8 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
     st = g->precision == 32 ? upload_coef<float>(g) : upload_coef<double>(g);
     if (st != ROEAM_OK) return cleanup(st);
     st = setup_tiles(g, 0);
+    if (st != ROEAM_OK) return cleanup(st);
+    st = g->precision == 32 ? setup_tile_kernel<float>(g) : setup_tile_kernel<double>(g);
     if (st != ROEAM_OK) return cleanup(st);
     // Load the module that holds the allocation-free residual's scratch array now (CUDA loads
     // modules lazily, and committing the array is an allocation), so that a caller which makes
@@ -1037,6 +1204,7 @@ void roeam_destroy_grid(roeam_grid *g)
     cudaFree(g->d_units_all);
     cudaFree(g->d_units_part);
     cudaFree(g->d_units_pipe);
+    cudaFree(g->d_rects);
     cudaFree(g->U);
     cudaFree(g->A);
     cudaFree(g->B);
@@ -1154,9 +1322,8 @@ roeam_status roeam_rk_step(roeam_grid *g, double cfl, double dt_fixed, int nstep
         if (nsteps == 0 || dt_fixed > 0.0) {
             for (int k = 0; k < g->count; ++k) dt_last[k] = nsteps == 0 ? 0.0 : dt_fixed;
         } else {
-            const int par = (int)((step0 + nsteps - 1) & 1);   // slot the last step read its rate from
-            CUDA_TRY(cudaMemcpyAsync(g->h_rate, g->rate + (size_t)par * g->count,
-                                     sizeof(unsigned long long) * g->count, cudaMemcpyDeviceToHost, g->stream));
+            // (the slot the last step read its rate from)
+            CUDA_TRY(cudaMemcpyAsync(g->h_rate, rate_slot(g, step0 + nsteps - 1), sizeof(unsigned long long) * g->count, cudaMemcpyDeviceToHost, g->stream));
             CUDA_TRY(cudaStreamSynchronize(g->stream));
             for (int k = 0; k < g->count; ++k) {
                 double r;
@@ -1239,7 +1406,7 @@ roeam_status roeam_autotune(roeam_grid *g, double cfl, int steps, int *best_cfg,
         if (!g->state_set[k]) return fail(ROEAM_E_STATE, "state of grid %d not set", k);
     CUDA_TRY(cudaSetDevice(g->device));
     const size_t sbytes = g->esize * (size_t)g->total_elems;
-    const size_t rbytes = sizeof(unsigned long long) * 2 * g->count;
+    const size_t rbytes = sizeof(unsigned long long) * RATE_SLOTS * g->count;
     void *save = nullptr;
     CUDA_TRY(cudaMalloc(&save, sbytes + rbytes));
     const long long step0 = g->step;
@@ -1298,6 +1465,7 @@ roeam_status roeam_autotune(roeam_grid *g, double cfl, int steps, int *best_cfg,
                 CUDA_TRY(cudaMemcpyAsync(g->U, save, sbytes, cudaMemcpyDeviceToDevice, g->stream));
                 CUDA_TRY(cudaMemcpyAsync(g->rate, (char *)save + sbytes, rbytes, cudaMemcpyDeviceToDevice, g->stream));
                 g->step = step0;
+                g->rate_clean = false;
             }
             times[cfg] = per;
             if (per < best_ms) { best_ms = per; best = cfg; }
@@ -1333,15 +1501,13 @@ long long roeam_cell_count(const roeam_grid *g, int grid_idx)
     return g->total_packed / 4;
 }
 
-
 // ---- stage-by-stage stepping and ghost rows (row slabs of one grid on several GPUs)
 
 roeam_status roeam_max_rate(roeam_grid *g, double *rate_out)
 {
     if (!g || !rate_out) return fail(ROEAM_E_ARG, "null argument");
     CUDA_TRY(cudaSetDevice(g->device));
-    const int par = (int)(g->step & 1);
-    CUDA_TRY(cudaMemcpyAsync(g->h_rate, g->rate + (size_t)par * g->count, sizeof(unsigned long long) * g->count,
+    CUDA_TRY(cudaMemcpyAsync(g->h_rate, rate_slot(g, g->step), sizeof(unsigned long long) * g->count,
                              cudaMemcpyDeviceToHost, g->stream));
     CUDA_TRY(cudaStreamSynchronize(g->stream));
     for (int k = 0; k < g->count; ++k) {
@@ -1356,7 +1522,6 @@ roeam_status roeam_max_rate(roeam_grid *g, double *rate_out)
     }
     return read_status(g);
 }
-
 
 roeam_status roeam_rk_stage(roeam_grid *g, int stage, double dt)
 {
@@ -1574,13 +1739,13 @@ static roeam_status step_host(roeam_grid *g, double cfl, double dt_fixed, int ns
     for (int k = 0; k < g->count; ++k) g->state_set[k] = 1;
     const long long step0 = g->step;
     g->step += nsteps;
+    g->rate_clean = false;
     CUDA_TRY(cudaStreamSynchronize(g->stream));
     if (dt_last) {
         if (dt_fixed > 0.0) {
             for (int k = 0; k < g->count; ++k) dt_last[k] = dt_fixed;
         } else {
-            const int par = (int)((step0 + nsteps - 1) & 1);
-            CUDA_TRY(cudaMemcpy(g->h_rate, g->rate + (size_t)par * g->count, sizeof(unsigned long long) * g->count,
+            CUDA_TRY(cudaMemcpy(g->h_rate, rate_slot(g, step0 + nsteps - 1), sizeof(unsigned long long) * g->count,
                                 cudaMemcpyDeviceToHost));
             for (int k = 0; k < g->count; ++k) {
                 if (g->precision == 32) {

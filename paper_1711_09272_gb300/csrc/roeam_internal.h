@@ -159,6 +159,51 @@ struct Launchers {
                               cudaStream_t s);
 };
 
+// ---- tile kernels (roeam_tile.cuh): a whole step per launch in FP32, a stage per launch in FP64
+template <typename T> __host__ __device__ constexpr int tile_stages() { return sizeof(T) == 4 ? 3 : 1; }
+template <typename T> __host__ __device__ constexpr int tile_threads() { return sizeof(T) == 4 ? 512 : 256; }
+constexpr size_t TILE_SMEM_MAX = 226 * 1024;   // dynamic shared memory a tile may take (227 KB per CTA in all)
+
+template <typename T>
+struct TileArgs {
+    const GridDev *grids;
+    const GridCoef<T> *coef;
+    const int4 *tiles;      // (grid, first column, first row, width | height << 16)
+    int ngrids;
+    const T *src, *un;      // U^(k) and U^n (STAGES = 3: both U^n)
+    T *dst;
+    const T *vdx, *vdy;
+    const uint8_t *solid;
+    T alpha, beta;          // STAGES = 1
+    int want_rate;
+    const unsigned long long *rate_rd;
+    unsigned long long *rate_wr, *rate_zero;
+    T cfl_t, dt_fixed_t;
+    unsigned *status;
+#ifdef ROEAM_DEBUG
+    long long n_state, n_vert, n_solid;   // buffer sizes, read by the bounds checks of debug builds
+#endif
+};
+
+// Shared memory of a tile of W x R positions (the rectangle and its halo): quads of T per position
+// (U, primitives, two fluxes, derived quantities or two slopes, U^n), the Eq. 97 ratios (one row
+// more: the pair list's unused faces past the last row read it), vertices, column and row maps,
+// flags.
+template <typename T> inline size_t tile_bytes(int W, int R, bool muscl, bool curv, bool walls, int stages)
+{
+    const size_t P = (size_t)W * R;
+    return sizeof(T) * (4 * P * (4 + (muscl ? 2 : 1) + (stages == 3 ? 1 : 0)) + 2 * (P + W + 2) +
+                        (curv ? 2 * (size_t)(W + 1) * (R + 1) : 0)) +
+           sizeof(int) * 2 * (W + 1 + R + 1) + (walls ? (P + 15) / 16 * 16 : 0);
+}
+
+template <typename T>
+struct TileLaunchers {
+    static cudaError_t step(const TileArgs<T> &a, int muscl, int curv, int walls, int ntiles, int threads, size_t smem,
+                            cudaStream_t s);
+    static cudaError_t prepare(int muscl, int curv, int walls);
+};
+
 // The ablation-variant stage kernels, instantiated in their own translation units.
 template <typename T>
 struct AblationLaunchers {

@@ -1,0 +1,6 @@
+// FP32 instantiations of the tile kernels.
+#include "roeam_tile.cuh"
+
+namespace roeam {
+template struct TileLaunchers<float>;
+}

@@ -1,0 +1,644 @@
+// roeam_tile.cuh — sm_103a kernels of the Roe-AM step for grids that the warp strips of
+// stage_kernel cannot fill the chip with, and for FP64.
+//
+// One CTA holds a rectangle of cells with its halo in shared memory and runs four phases per
+// Runge-Kutta stage, a block barrier between them: primitives and derived quantities per cell
+// (ghost cells from the boundary conditions), Eq. 97 ratios and limited slopes per cell, fluxes per
+// face, update per cell. Every phase spreads its work over all threads, so a stage takes one flux
+// evaluation's latency per few hundred faces instead of the strip's row after row.
+//
+// STAGES = 3 (FP32): the whole SSP-RK3 step in one launch. The CTA loads a halo of 3 H cells
+// (H = 1 at first order, 2 with MUSCL) and updates a margin of 2 H, H and 0 cells around its
+// rectangle in the three stages, recomputing what its neighbours also compute, so no CTA waits
+// for another and U^(1), U^(2) never leave shared memory. What bounds a step is then latency and, on
+// the larger grids, instruction issue: of 7 us for a 12 x 10 rectangle, 0.8 are descriptors and maps,
+// 0.5 the load, and a stage takes 0.45 ghost cells, 0.2 ratios, 0.7 fluxes, 0.45 update. The strips
+// take 17 to 25 us a step on these grids whatever their size (three launches of a few serial row
+// iterations each): 256^2 van Leer 24.5 -> 12.7 us a step, 400^2 corner 32 -> 19, 800 x 20 duct
+// 25 -> 7.9.
+// STAGES = 1 (FP64): one stage per launch. FP64 kernels are bound by the FP64 pipe, so recomputed
+// halos cost time; the phases evaluate each face once per CTA and keep all lanes busy where the
+// strips of a small grid evaluated three rows of faces per two rows of cells. The fluxes take 75 % of
+// a stage and run at the pipe's rate (133 operations per first-order face, about 190 reconstructed).
+// 64^2 139 -> 33 us a step, 256^2 first order 277 -> 167, van Leer 496 -> 252, 1024^2 2696 -> 2304.
+//
+// In directions that are not periodic the halo ends H cells outside the grid; in periodic ones the
+// halo cells are cells of the other side, which evolve like their originals.
+#pragma once
+
+#include "roeam_kernels.cuh"
+
+namespace roeam {
+
+// Bounds-checked debug builds: n elements at index i of a buffer of `size`, or ST_BOUNDS and no access.
+#ifdef ROEAM_DEBUG
+__device__ __forceinline__ bool tile_ok(long long i, int n, long long size, unsigned *status)
+{
+    if (i >= 0 && i + n <= size) return true;
+    atomicOr(status, ST_BOUNDS);
+    return false;
+}
+#define TILE_OK(i, n, size) tile_ok((i), (n), a.size, a.status)
+#else
+#define TILE_OK(i, n, size) true
+#endif
+
+// Asynchronous copy of one value into shared memory.
+template <typename T> __device__ __forceinline__ void copy_value(T *dst, const T *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"((int)sizeof(T)) : "memory");
+}
+
+// Largest of a warp's non-negative rates, through the bit patterns (redux: one instruction per word).
+__device__ __forceinline__ float warp_rate_max(float r)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(r)));
+}
+__device__ __forceinline__ double warp_rate_max(double r)
+{
+    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return __hiloint2double((int)mh, (int)ml);
+}
+
+template <typename T, bool MUSCL, bool CURV, bool WALLS, int STAGES>
+__global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<T> a)
+{
+    constexpr int H = MUSCL ? 2 : 1;
+    constexpr int E = H * STAGES;
+    constexpr bool PAIRS = sizeof(T) == 4;   // FP32 evaluates a cell's west and south faces as one packed pair
+    // The next launch may start; it waits below (like this one) before it touches the state.
+    asm volatile("griddepcontrol.launch_dependents;");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T red[tile_threads<T>() / 32];
+
+    const int4 tile = __ldg(a.tiles + blockIdx.x);
+    const int g = a.ngrids == 1 ? 0 : tile.x;   // (one grid: its descriptor is loaded beside the tile's)
+    const int x0 = tile.y, y0 = tile.z, w = tile.w & 0xffff, h = tile.w >> 16;
+    const GridDev &G = a.grids[g];
+    const GridCoef<T> K = a.coef[g];
+    const int ni = G.ni, nj = G.nj, pitch = G.pitch;
+    const int bcW = G.bc[0], bcE = G.bc[1], bcS = G.bc[2], bcN = G.bc[3];
+    const bool perx = bcW == BC_PERIODIC, pery = bcS == BC_PERIODIC;
+    const bool use_s1 = G.use_s1 != 0, vanleer = G.limiter == 2;
+    const int eps1 = G.eps1, xi_form = G.xi_form;
+    const int W = w + 2 * E, R = h + 2 * E, P = W * R;   // positions: column c is ix0 + c, row r is jy0 + r
+    const int ix0 = x0 - E, jy0 = y0 - E;
+
+    T *const U = reinterpret_cast<T *>(smem_raw);
+    T *const A1 = U + 4 * P;
+    T *const FX = A1 + 4 * P, *const FY = FX + 4 * P;
+    T *const A2 = FY + 4 * P;                       // derived quantities, or x-slopes
+    T *const SY = A2 + 4 * P;                       // y-slopes (MUSCL)
+    T *const Un = A2 + (MUSCL ? 8 : 4) * P;         // U^n (STAGES = 3)
+    T *const PP = A2 + ((MUSCL ? 8 : 4) + (STAGES == 3 ? 4 : 0)) * P;   // Eq. 97 ratios of the west and south faces
+    T *const VV = PP + 2 * (P + W + 2);                       // vertex displacements (CURV): (W + 1) x (R + 1) pairs
+    int *const CM = reinterpret_cast<int *>(VV + (CURV ? 2 * (W + 1) * (R + 1) : 0));   // columns, then rows: see below
+    int *const RM = CM + 2 * (W + 1);
+    uint8_t *const FL = reinterpret_cast<uint8_t *>(RM + 2 * (R + 1));
+    const int tid = threadIdx.x, nt = blockDim.x;
+
+    // The margins of the stages: stage s updates columns [lox, hix) and rows [loy, hiy) (clipped to
+    // the grid in directions that are not periodic).
+    auto margin = [&](int s, int &lox, int &hix, int &loy, int &hiy) {
+        const int e = E - H * (s + 1);
+        lox = perx ? E - e : max(E - e, -ix0); hix = perx ? E + w + e : min(E + w + e, ni - ix0);
+        loy = pery ? E - e : max(E - e, -jy0); hiy = pery ? E + h + e : min(E + h + e, nj - jy0);
+    };
+    // Per column (and row): [0] the grid column its cells are loaded from (-1: none), or the vertex
+    // column; [1] for ghost cells the position their values come from and their kind (resolve_index)
+    // in bits 16 and up. Divisions happen here once, not per position and phase: `recip` holds
+    // 2^32 / n + 1 for the width n of every rectangle that a phase covers.
+    __shared__ unsigned recip[4 * STAGES + 2];
+    if (tid < 4 * STAGES + 2) {
+        int n = tid == 4 * STAGES ? W + 1 : W;
+        if (tid < 4 * STAGES) {
+            int lox, hix, loy, hiy;
+            margin(tid >> 2, lox, hix, loy, hiy);
+            const int p = tid & 3;   // cells with ghosts, ratios, face pairs (or west faces), cells
+            n = hix - lox + (p == 0 ? 2 * H : (p == 1 ? 2 : (p == 2 ? 1 : 0)));
+        }
+        recip[tid] = 0xffffffffu / (unsigned)n + 1u;
+    }
+    for (int q = tid; q < W + 1 + R + 1; q += nt) {
+        const bool col = q < W + 1;
+        const int x = col ? q : q - (W + 1), v = (col ? ix0 : jy0) + x, n = col ? ni : nj, o = col ? ix0 : jy0;
+        const bool per = col ? perx : pery;
+        int src = v, from = x;
+        if (per) { src = v % n; src = src < 0 ? src + n : src; }
+        else if (v < 0 || v >= n) {
+            int kind;
+            from = resolve_index(v, n, col ? bcW : bcS, col ? bcE : bcN, kind) - o;
+            from = (from & 0xffff) | kind << 16;
+            src = -1;
+        }
+        (col ? CM : RM)[2 * x] = src;
+        (col ? CM : RM)[2 * x + 1] = from;
+    }
+    __syncthreads();
+
+    // every position of the rectangle [c0, c1) x [r0, r1), spread over the threads; m = recip of its width
+    auto over = [&](unsigned m, int c0, int c1, int r0, int r1, auto &&body) {
+        const int wd = c1 - c0, n = wd * (r1 - r0);
+#pragma unroll 1
+        for (int idx = tid; idx < n; idx += nt) {
+            const int q = wd == 1 ? idx : (int)__umulhi((unsigned)idx, m);   // idx / wd (idx wd < 2^32)
+            body(c0 + idx - q * wd, r0 + q);
+        }
+    };
+
+    // vertices do not depend on the launches before this one
+    if constexpr (CURV)
+        over(recip[4 * STAGES], 0, W + 1, 0, R + 1, [&](int c, int r) {
+            // (a periodic seam's last vertex column repeats the first)
+            int i = ix0 + c, j = jy0 + r;
+            i = perx && (i < 0 || i > ni) ? CM[2 * c] : clampi(i, 0, ni);
+            j = pery && (j < 0 || j > nj) ? RM[2 * r] : clampi(j, 0, nj);
+            const long long b = G.voff + (long long)j * G.vpitch + i;
+            if (TILE_OK(b, 1, n_vert)) {
+                copy_value(VV + 2 * (r * (W + 1) + c), a.vdx + b);
+                copy_value(VV + 2 * (r * (W + 1) + c) + 1, a.vdy + b);
+            }
+        });
+    auto vtx = [&](int c, int r, T &x, T &y) { x = VV[2 * (r * (W + 1) + c)]; y = VV[2 * (r * (W + 1) + c) + 1]; };
+    // unit normals and lengths of the west face and the south face of position (c, r)
+    auto geom_x = [&](int c, int r, T &nx, T &ny, T &len) {
+        if constexpr (CURV) {
+            T xa, ya, xb, yb;
+            vtx(c, r, xa, ya); vtx(c, r + 1, xb, yb);
+            const T sx = K.dy + (yb - ya), sy = -(xb - xa);
+            len = sqrt0(vfma(sx, sx, sy * sy));
+            const T li = rcp(len);
+            nx = sx * li; ny = sy * li;
+        } else { nx = T(1); ny = T(0); len = T(2); }   // (the residual applies the Cartesian lengths)
+    };
+    auto geom_y = [&](int c, int r, T &nx, T &ny, T &len) {
+        if constexpr (CURV) {
+            T xa, ya, xb, yb;
+            vtx(c, r, xa, ya); vtx(c + 1, r, xb, yb);
+            const T sx = -(yb - ya), sy = K.dx + (xb - xa);
+            len = sqrt0(vfma(sx, sx, sy * sy));
+            const T li = rcp(len);
+            nx = sx * li; ny = sy * li;
+        } else { nx = T(0); ny = T(1); len = T(2); }
+    };
+
+    // everything from here on may depend on the launch before this one
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (a.rate_zero && blockIdx.x == 0)
+        for (int q = tid; q < a.ngrids; q += nt) a.rate_zero[q] = 0ull;
+    {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(U);
+        over(recip[4 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
+            const int i = CM[2 * c], j = RM[2 * r];
+            const long long x = G.off + 4 * ((long long)j * pitch + i);
+            if ((i | j) >= 0 && TILE_OK(x, 4, n_state))
+                copy_cell(dst + (unsigned)((r * W + c) * 4 * (int)sizeof(T)), a.src + x);
+        });
+        copies_commit();
+    }
+    if constexpr (WALLS) {
+        // (solid cells are never combined with periodic sides; ghost cells are flagged below)
+        const unsigned mw = recip[4 * STAGES + 1];
+        const bool mask = G.soff >= 0;
+#pragma unroll 4
+        for (int at = tid; at < P; at += nt) {
+            const int r = (int)__umulhi((unsigned)at, mw), c = at - r * W;
+            const int i = CM[2 * c], j = RM[2 * r];
+            uint8_t f = 0;
+            const long long x = G.soff + (long long)j * ni + i;
+            if (mask && (i | j) >= 0 && TILE_OK(x, 1, n_solid)) f = __ldg(a.solid + x);
+            FL[at] = f;
+        }
+    }
+    // Primitives (and, at first order, the derived face quantities) of a cell from its state.
+    auto prims = [&](const T raw[4], WC<T> &q) {
+        const T ri = rcp(raw[0]);
+        q.r = raw[0]; q.u = raw[1] * ri; q.v = raw[2] * ri;
+        q.p = K.gm1 * vfnma(T(0.5) * raw[0], vfma(q.u, q.u, q.v * q.v), raw[3]);
+    };
+    auto put_cell = [&](int at, WC<T> &q) {
+        const T a1[4] = {q.r, q.u, q.v, q.p};
+        st_cell(A1 + 4 * at, a1);
+        if constexpr (!MUSCL) {
+            derive<T, false>(q, K);
+            const T a2[4] = {q.c2, q.H, q.sr, q.Mq};
+            st_cell(A2 + 4 * at, a2);
+        }
+    };
+    // A ghost cell (outside the grid in a direction that is not periodic) from its source cell.
+    auto ghost_cell = [&](int c, int r) {
+        const int at = r * W + c, cm = CM[2 * c + 1], rm = RM[2 * r + 1];
+        const int cs = cm & 0xffff, kx = cm >> 16, rs = rm & 0xffff, ky = rm >> 16;
+        WC<T> q;
+        if (kx == 2 || ky == 2) {
+            q.r = K.inflow[0]; q.u = K.inflow[1]; q.v = K.inflow[2]; q.p = K.inflow[3];
+        } else {
+            T raw[4];
+            ld_own(U + 4 * (rs * W + cs), raw);
+            prims(raw, q);
+        }
+        if constexpr (WALLS) {
+            const int i = ix0 + c, j = jy0 + r;
+            uint8_t f = (kx == 2 || ky == 2) ? (uint8_t)0 : (uint8_t)(FL[rs * W + cs] & 1);
+            // (the boundary face's row clamped to the grid: corner ghost cells, whose velocities are
+            //  never used)
+            if (ky == 1 && kx != 2) {
+                T nx, ny, l;
+                geom_y(cs, (j < 0 ? 0 : nj) - jy0, nx, ny, l);
+                mirror_vel(q.u, q.v, nx, ny);
+            }
+            if (kx == 1) {
+                T nx, ny, l;
+                geom_x((i < 0 ? 0 : ni) - ix0, pery ? r : clampi(j, 0, nj - 1) - jy0, nx, ny, l);
+                mirror_vel(q.u, q.v, nx, ny);
+            }
+            if ((kx == 1 || ky == 1) && kx != 2) f |= 2;
+            FL[at] = f;
+        }
+        put_cell(at, q);
+    };
+    const T dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_value<T>(__ldg(a.rate_rd + g));
+    const T rxy = K.dy / K.dx, cy = T(0.5) * K.dx * K.Vi;   // Cartesian residual weights
+    copies_wait<0>();
+    // (each thread turns the cells that it copied itself into primitives: no barrier in between)
+    over(recip[4 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
+        if ((CM[2 * c] | RM[2 * r]) >= 0) {
+            T raw[4];
+            WC<T> q;
+            ld_own(U + 4 * (r * W + c), raw);
+            prims(raw, q);
+            put_cell(r * W + c, q);
+        }
+    });
+    __syncthreads();
+
+    T my_rate = T(0);
+#pragma unroll 1
+    for (int s = 0; s < STAGES; ++s) {
+        int lox, hix, loy, hiy;
+        margin(s, lox, hix, loy, hiy);
+        const unsigned *const m = recip + 4 * s;
+        const T alpha = STAGES == 1 ? a.alpha : (s == 0 ? T(0) : (s == 1 ? T(0.75) : T(1.0 / 3.0)));
+        const T beta = STAGES == 1 ? a.beta : (s == 0 ? T(1) : (s == 1 ? T(0.25) : T(2.0 / 3.0)));
+        const bool last = s == STAGES - 1;
+
+        // ---- ghost cells, where the cells that the stage reads (H beyond its margin) leave the grid on
+        //      a side that is not periodic: columns west and east (all rows), then rows south and north
+        const int gW = perx ? 0 : max(0, -ix0 - (lox - H)), gE = perx ? 0 : max(0, hix + H - (ni - ix0));
+        const int gS = pery ? 0 : max(0, -jy0 - (loy - H)), gN = pery ? 0 : max(0, hiy + H - (nj - jy0));
+        if (gW | gE | gS | gN) {   // (0 to H columns or rows each)
+            const int rows = hiy - loy + 2 * H, cl = lox - H + gW, cols = hix + H - gE - cl;
+            const int nW = gW * rows, nE = nW + gE * rows, nS = nE + gS * cols, nN = nS + gN * cols;
+            for (int k = tid; k < nN; k += nt) {
+                int c, r;
+                if (k < nE) {
+                    const int q = k < nW ? k : k - nW, two = (k < nW ? gW : gE) - 1;
+                    c = (k < nW ? lox - H : hix + H - gE) + (two ? q & 1 : 0);
+                    r = loy - H + (q >> two);
+                } else {
+                    const int q = k < nS ? k - nE : k - nS, d = q >= cols;
+                    c = cl + q - (d ? cols : 0);
+                    r = (k < nS ? loy - H : hiy + H - gN) + d;
+                }
+                ghost_cell(c, r);
+            }
+            __syncthreads();
+        }
+
+        // ---- cells: Eq. 97 ratios of the west and south faces (1 at solid sides), limited slopes
+        // (at first order the ratios of the outermost column's west and row's south faces read outside
+        //  the stage's cells, but inside shared memory, and are not used)
+        over(m[1], lox - 1, hix + 1, loy - 1, hiy + 1, [&](int c, int r) {
+            const int at = r * W + c;
+            T q[4], qw[4], qs[4];
+            ld_own(A1 + 4 * at, q);
+            ld_own(A1 + 4 * (at - 1), qw);
+            ld_own(A1 + 4 * (at - W), qs);
+            T Px = ratio_P(qw[0], qw[3], q[0], q[3]), Py = ratio_P(qs[0], qs[3], q[0], q[3]);
+            int fl = 0, flw = 0, fls = 0;
+            if constexpr (WALLS) {
+                fl = FL[at] & 1; flw = FL[at - 1] & 1; fls = FL[at - W] & 1;
+                if (fl | flw) Px = T(1);
+                if (fl | fls) Py = T(1);
+            }
+            PP[2 * at] = Px;
+            PP[2 * at + 1] = Py;
+            if constexpr (MUSCL) {
+                T qe[4], qn[4];
+                ld_own(A1 + 4 * (at + 1), qe);
+                ld_own(A1 + 4 * (at + W), qn);
+                if constexpr (WALLS) {
+                    // a solid stencil cell is replaced by the mirror of this cell about their face
+                    const int fle = FL[at + 1] & 1, fln = FL[at + W] & 1;
+                    if (flw | fls | fle | fln) {
+                        T nx, ny, l;
+                        if (flw) { for (int k = 0; k < 4; ++k) qw[k] = q[k]; geom_x(c, r, nx, ny, l); mirror_vel(qw[1], qw[2], nx, ny); }
+                        if (fle) { for (int k = 0; k < 4; ++k) qe[k] = q[k]; geom_x(c + 1, r, nx, ny, l); mirror_vel(qe[1], qe[2], nx, ny); }
+                        if (fls) { for (int k = 0; k < 4; ++k) qs[k] = q[k]; geom_y(c, r, nx, ny, l); mirror_vel(qs[1], qs[2], nx, ny); }
+                        if (fln) { for (int k = 0; k < 4; ++k) qn[k] = q[k]; geom_y(c, r + 1, nx, ny, l); mirror_vel(qn[1], qn[2], nx, ny); }
+                    }
+                }
+                T sx[4], sy[4];
+                for (int k = 0; k < 4; ++k) {
+                    if constexpr (PAIRS) {
+                        const V2 B = mk2(q[k], q[k]);
+                        const V2 sl = limiter(vanleer, B - mk2(qw[k], qs[k]), mk2(qe[k], qn[k]) - B);
+                        sx[k] = sl.v.x; sy[k] = sl.v.y;
+                    } else {
+                        sx[k] = limiter(vanleer, q[k] - qw[k], qe[k] - q[k]);
+                        sy[k] = limiter(vanleer, q[k] - qs[k], qn[k] - q[k]);
+                    }
+                }
+                st_cell(A2 + 4 * at, sx);
+                st_cell(SY + 4 * at, sy);
+            }
+        });
+        __syncthreads();
+
+        // ---- faces. `d` = 1: the west face of position (c, r), `d` = W: its south face.
+        auto detector_min = [&](int at, int d) {
+            // Eq. 96 in 2D: the face and the transverse faces of both its cells
+            const int o = d == 1 ? 0 : 1, tr = d == 1 ? W : 1;
+            const T *q = PP + 2 * at;
+            return fmn3(fmn3(q[o], q[1 - o - 2 * d], q[1 - o - 2 * d + 2 * tr]), q[1 - o], q[1 - o + 2 * tr]);
+        };
+        // The two sides of a face in global primitives (MUSCL: reconstructed, else the cells), walls
+        // taking the fluid side's first-order state and its mirror; false where no flux passes.
+        auto sides = [&](int at, int d, T nx, T ny, T L[4], T Rr[4]) {
+            ld_own(A1 + 4 * (at - d), L);
+            ld_own(A1 + 4 * at, Rr);
+            int fA = 0, fB = 0;
+            if constexpr (WALLS) { fA = FL[at - d]; fB = FL[at]; }
+            if constexpr (MUSCL) {
+                if (!WALLS || (fA | fB) == 0) {
+                    const T *S = d == 1 ? A2 : SY;
+                    T sA[4], sB[4], rL[4], rR[4];
+                    ld_own(S + 4 * (at - d), sA);
+                    ld_own(S + 4 * at, sB);
+                    for (int k = 0; k < 4; ++k) { rL[k] = vfma(T(0.5), sA[k], L[k]); rR[k] = vfnma(T(0.5), sB[k], Rr[k]); }
+                    if (rL[0] > T(0) && rL[3] > T(0) && rR[0] > T(0) && rR[3] > T(0))
+                        for (int k = 0; k < 4; ++k) { L[k] = rL[k]; Rr[k] = rR[k]; }
+                }
+            }
+            if constexpr (WALLS) {
+                if (fA | fB) {
+                    if (fA & fB & 1) return false;
+                    if (fA) { for (int k = 0; k < 4; ++k) L[k] = Rr[k]; mirror_vel(L[1], L[2], nx, ny); }
+                    else { for (int k = 0; k < 4; ++k) Rr[k] = L[k]; mirror_vel(Rr[1], Rr[2], nx, ny); }
+                }
+            }
+            return true;
+        };
+        // The whole evaluation of one face on its own (FP64; in FP32 the faces across a jump of 1e5
+        // or more in density or pressure, whose positivity is decided in FP64): face_scalar.
+        auto marginal_face = [&](int c, int r, int d, T s1, T F[4]) {
+            const int at = r * W + c;
+            Face<T> f;
+            T l;
+            auto cell = [&](int q, WC<T> &o) {
+                T v[4];
+                ld_own(A1 + 4 * q, v);
+                o.r = v[0]; o.u = v[1]; o.v = v[2]; o.p = v[3];
+                o.c2 = o.H = o.sr = o.Mq = T(0);
+                o.fl = WALLS ? FL[q] : 0;
+            };
+            cell(at - d, f.A); cell(at, f.B);
+            if constexpr (MUSCL) {
+                cell(at - 2 * d, f.Am); cell(at + d, f.Bp);
+                if (d == 1) { geom_x(c - 1, r, f.nAmx, f.nAmy, l); geom_x(c + 1, r, f.nBpx, f.nBpy, l); }
+                else { geom_y(c, r - 1, f.nAmx, f.nAmy, l); geom_y(c, r + 1, f.nBpx, f.nBpy, l); }
+            }
+            if (d == 1) geom_x(c, r, f.nx, f.ny, f.len);
+            else geom_y(c, r, f.nx, f.ny, f.len);
+            f.s1 = s1;
+            face_scalar<T, MUSCL>(f, K, eps1, xi_form, vanleer, F);
+        };
+        if constexpr (PAIRS) {
+            over(m[2], lox, hix + 1, loy, hiy + 1, [&](int c, int r) {
+                const int at = r * W + c;
+                V2 s1 = mk2(1.f, 1.f);
+                if (use_s1) s1 = detector_of(mk2(detector_min(at, 1), detector_min(at, W)));
+                float Fx[4], Fy[4];
+                if constexpr (MUSCL) {
+                    const float eps = 1e-5f;
+                    if (PP[2 * at] < eps || PP[2 * at + 1] < eps) {
+                        marginal_face(c, r, 1, s1.v.x, Fx);
+                        marginal_face(c, r, W, s1.v.y, Fy);
+                        st_cell(FX + 4 * at, Fx);
+                        st_cell(FY + 4 * at, Fy);
+                        return;
+                    }
+                }
+                Face<float> fx, fy;
+                geom_x(c, r, fx.nx, fx.ny, fx.len);
+                geom_y(c, r, fy.nx, fy.ny, fy.len);
+                fx.s1 = s1.v.x; fy.s1 = s1.v.y;
+                float Lx[4], Rx[4], Ly[4], Ry[4];
+                const bool okx = sides(at, 1, fx.nx, fx.ny, Lx, Rx), oky = sides(at, W, fy.nx, fy.ny, Ly, Ry);
+                V2 WL[4], WR[4];
+                if constexpr (MUSCL) {
+                    for (int k = 0; k < 4; ++k) { WL[k] = mk2(Lx[k], Ly[k]); WR[k] = mk2(Rx[k], Ry[k]); }
+                } else {
+                    auto put = [&](const float v[4], int q, WC<float> &o) {
+                        float d4[4];
+                        ld_own(A2 + 4 * q, d4);
+                        o.r = v[0]; o.u = v[1]; o.v = v[2]; o.p = v[3];
+                        o.c2 = d4[0]; o.H = d4[1]; o.sr = d4[2]; o.Mq = d4[3];
+                    };
+                    // (a wall face's mirrored side has the fluid cell's derived quantities)
+                    int ax = at - 1, bx = at, ay = at - W, by = at;
+                    if constexpr (WALLS) {
+                        if (FL[ax]) ax = at; else if (FL[bx]) bx = at - 1;
+                        if (FL[ay]) ay = at; else if (FL[by]) by = at - W;
+                    }
+                    put(Lx, ax, fx.A); put(Rx, bx, fx.B); put(Ly, ay, fy.A); put(Ry, by, fy.B);
+                }
+                faces_packed<MUSCL, CURV>(fx, fy, K, eps1, xi_form, WL, WR, Fx, Fy);
+                if constexpr (WALLS) {
+                    if (!okx) Fx[0] = Fx[1] = Fx[2] = Fx[3] = 0.f;
+                    if (!oky) Fy[0] = Fy[1] = Fy[2] = Fy[3] = 0.f;
+                }
+                st_cell(FX + 4 * at, Fx);
+                st_cell(FY + 4 * at, Fy);
+            });
+        } else {
+            // west faces, then south faces, one list: every lane has a face
+            const int wx = hix + 1 - lox, hx = hiy - loy, nx_ = wx * hx, wyy = hix - lox, ny_ = wyy * (hiy + 1 - loy);
+            const unsigned mx = m[2], my = m[3];
+            for (int idx = tid; idx < nx_ + ny_; idx += nt) {
+                const bool isx = idx < nx_;
+                const int k = isx ? idx : idx - nx_, wd = isx ? wx : wyy;
+                const int q = wd == 1 ? k : (int)__umulhi((unsigned)k, isx ? mx : my);
+                const int c = lox + k - q * wd, r = loy + q, at = r * W + c, d = isx ? 1 : W;
+                T nx, ny, len;
+                if (isx) geom_x(c, r, nx, ny, len); else geom_y(c, r, nx, ny, len);
+                T L[4], Rr[4], F[4] = {T(0), T(0), T(0), T(0)};
+                if (sides(at, d, nx, ny, L, Rr)) {
+                    const T s1 = use_s1 ? detector_of(detector_min(at, d)) : T(1);
+                    FS<T> sl, sr;
+                    if constexpr (MUSCL) {
+                        if constexpr (CURV) {
+                            sl = side_rot(L[0], L[1], L[2], L[3], nx, ny, K);
+                            sr = side_rot(Rr[0], Rr[1], Rr[2], Rr[3], nx, ny, K);
+                        } else {
+                            sl = side_from_prims(L[0], isx ? L[1] : L[2], isx ? L[2] : L[1], L[3], K);
+                            sr = side_from_prims(Rr[0], isx ? Rr[1] : Rr[2], isx ? Rr[2] : Rr[1], Rr[3], K);
+                        }
+                    } else {
+                        int qa = at - d, qb = at;
+                        if constexpr (WALLS) { if (FL[qa]) qa = at; else if (FL[qb]) qb = at - d; }
+                        T da[4], db[4];
+                        ld_own(A2 + 4 * qa, da);
+                        ld_own(A2 + 4 * qb, db);
+                        if constexpr (CURV) {
+                            sl = {L[0], vfma(nx, L[1], ny * L[2]), vfma(nx, L[2], -(ny * L[1])), L[3], da[0], da[1], da[2], da[3]};
+                            sr = {Rr[0], vfma(nx, Rr[1], ny * Rr[2]), vfma(nx, Rr[2], -(ny * Rr[1])), Rr[3], db[0], db[1], db[2], db[3]};
+                        } else {
+                            sl = {L[0], isx ? L[1] : L[2], isx ? L[2] : L[1], L[3], da[0], da[1], da[2], da[3]};
+                            sr = {Rr[0], isx ? Rr[1] : Rr[2], isx ? Rr[2] : Rr[1], Rr[3], db[0], db[1], db[2], db[3]};
+                        }
+                    }
+                    T G2[4];
+                    roeam_flux2(sl, sr, s1, K, eps1, xi_form, G2);
+                    if constexpr (CURV) {
+                        const T hl = T(0.5) * len;
+                        F[0] = hl * G2[0];
+                        F[1] = hl * vfnma(ny, G2[2], nx * G2[1]);
+                        F[2] = hl * vfma(ny, G2[1], nx * G2[2]);
+                        F[3] = hl * G2[3];
+                    } else {   // (twice the flux: the residual applies the half lengths)
+                        F[0] = G2[0]; F[1] = isx ? G2[1] : G2[2]; F[2] = isx ? G2[2] : G2[1]; F[3] = G2[3];
+                    }
+                }
+                st_cell((isx ? FX : FY) + 4 * at, F);
+            }
+        }
+        __syncthreads();
+
+        // ---- cells: R = D sc, then the stage combination
+        over(m[3], lox, hix, loy, hiy, [&](int c, int r) {
+            const int at = r * W + c;
+            T fw[4], fe[4], fs[4], fn[4], uk[4], un[4], out[4];
+            ld_own(FX + 4 * at, fw);
+            ld_own(FX + 4 * (at + 1), fe);
+            ld_own(FY + 4 * at, fs);
+            ld_own(FY + 4 * (at + W), fn);
+            ld_own(U + 4 * at, uk);
+            const bool own = c >= E && c < E + w && r >= E && r < E + h;   // (others also update halo cells)
+            const long long x = G.off + 4 * ((long long)(jy0 + r) * pitch + (ix0 + c));
+            if (STAGES == 1) {
+                if (alpha != T(0)) ld_own(a.un + x, un);
+                else for (int k = 0; k < 4; ++k) un[k] = uk[k];
+            } else if (s == 0) {
+                for (int k = 0; k < 4; ++k) un[k] = uk[k];
+                st_cell(Un + 4 * at, uk);
+            } else {
+                ld_own(Un + 4 * at, un);
+            }
+            bool solid = false;
+            if constexpr (WALLS) solid = FL[at] & 1;
+            CellGeom<T> cg;
+            if constexpr (CURV) {
+                T x00, y00, x10, y10, x01, y01, x11, y11;
+                vtx(c, r, x00, y00); vtx(c + 1, r, x10, y10); vtx(c, r + 1, x01, y01); vtx(c + 1, r + 1, x11, y11);
+                cg = cell_geom(x00, x10, x01, x11, y00, y10, y01, y11, K.dx, K.dy);
+            } else {
+                cg.Xx = K.dy; cg.Xy = T(0); cg.Yx = T(0); cg.Yy = K.dx; cg.V = K.V;
+            }
+            const T sc = CURV ? rcp(cg.V) : cy;
+            for (int k = 0; k < 4; ++k) {
+                T D = CURV ? (fw[k] - fe[k] + fs[k]) - fn[k] : vfma(fw[k] - fe[k], rxy, fs[k]) - fn[k];
+                if (solid) D = T(0);
+                const T upd = vfma(dt * sc, D, uk[k]);
+                out[k] = vfma(alpha, un[k], beta * upd);
+            }
+            if (!last) {
+                st_cell(U + 4 * at, out);
+                WC<T> q;
+                prims(out, q);
+                put_cell(at, q);
+            } else if (TILE_OK(x, 4, n_state)) {
+                st_cell(a.dst + x, out);
+            }
+            if (own && !solid) {
+                if (last && a.want_rate) {
+                    const CellPrims<T> cp = cell_prims(out[0], out[1], out[2], out[3], K);
+                    if (!(out[0] > T(0)) || !(cp.p > T(0))) {
+                        const bool fin = isfinite((double)out[0]) && isfinite((double)cp.p);
+                        atomicOr(a.status, fin ? ST_NONPOSITIVE : ST_NONFINITE);
+                    } else {
+                        my_rate = vmax(my_rate, cell_rate<CURV>(cp, cg, K));
+                    }
+                } else {
+                    const T e2 = T(2) * out[0] * out[3], m2 = vfma(out[1], out[1], out[2] * out[2]);
+                    if (!(out[0] > T(0)) || !(e2 > m2)) {
+                        const CellPrims<T> cp = cell_prims(out[0], out[1], out[2], out[3], K);
+                        if (!(out[0] > T(0)) || !(cp.p > T(0))) {
+                            const bool fin = isfinite((double)out[0]) && isfinite((double)cp.p);
+                            atomicOr(a.status, fin ? ST_NONPOSITIVE : ST_NONFINITE);
+                        }
+                    }
+                }
+            }
+        });
+        if (!last) __syncthreads();
+    }
+    if (a.want_rate) {
+        my_rate = warp_rate_max(my_rate);
+        if ((tid & 31) == 0) red[tid >> 5] = my_rate;
+        __syncthreads();
+        if (tid < 32) {
+            my_rate = warp_rate_max(tid < nt / 32 ? red[tid] : T(0));
+            if (tid == 0 && my_rate > T(0)) atomicMax(a.rate_wr + g, rate_bits(my_rate));
+        }
+    }
+}
+
+// ------------------------------------------------------------------ launchers
+template <typename T, bool MUSCL, bool CURV, bool WALLS> struct TileVariant {
+    static constexpr int STAGES = tile_stages<T>();
+    static cudaError_t launch(const TileArgs<T> &a, int ntiles, int threads, size_t smem, cudaStream_t s)
+    {
+        cudaLaunchConfig_t c = {};
+        c.gridDim = dim3((unsigned)ntiles);
+        c.blockDim = dim3((unsigned)threads);
+        c.dynamicSmemBytes = smem;
+        c.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        c.attrs = at;
+        c.numAttrs = 1;
+        return cudaLaunchKernelEx(&c, tile_kernel<T, MUSCL, CURV, WALLS, STAGES>, a);
+    }
+    static cudaError_t prepare(size_t smem)
+    {
+        return cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
+};
+
+#define ROEAM_TILE_DISPATCH(CALL)                                                                              \
+    if (muscl) return curv ? (walls ? TileVariant<T, true, true, true>::CALL : TileVariant<T, true, true, false>::CALL) \
+                           : (walls ? TileVariant<T, true, false, true>::CALL : TileVariant<T, true, false, false>::CALL); \
+    return curv ? (walls ? TileVariant<T, false, true, true>::CALL : TileVariant<T, false, true, false>::CALL) \
+                : (walls ? TileVariant<T, false, false, true>::CALL : TileVariant<T, false, false, false>::CALL);
+
+template <typename T>
+cudaError_t TileLaunchers<T>::step(const TileArgs<T> &a, int muscl, int curv, int walls, int ntiles, int threads,
+                                   size_t smem, cudaStream_t s)
+{
+    ROEAM_TILE_DISPATCH(launch(a, ntiles, threads, smem, s))
+}
+
+// Allows the kernel the most shared memory that a launch may ask for (the attribute belongs to the
+// device, so every handle asks for the same).
+template <typename T>
+cudaError_t TileLaunchers<T>::prepare(int muscl, int curv, int walls)
+{
+    ROEAM_TILE_DISPATCH(prepare(TILE_SMEM_MAX))
+}
+
+}  // namespace roeam
