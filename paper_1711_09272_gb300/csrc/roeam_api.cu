@@ -603,17 +603,23 @@ roeam_status launch_step(roeam_grid *g, cudaStream_t s, long long step, double c
 }
 
 // The rate output of a pack into the current step's rate slots (grids [lo, hi) of `slot`
-// zeroed first on stream s), so that the next step takes its dt from the state just loaded.
+// zeroed first on stream s), so that the next step takes its dt from the state just loaded. Where
+// every grid is loaded and the next slot is known to be zero (a tile step or such a load came last),
+// that slot becomes the current one and the pack itself clears the one after: no launch more.
 template <typename T>
 roeam_status rate_out(roeam_grid *g, int lo, int hi, cudaStream_t s, RateOut<T> &ro)
 {
-    unsigned long long *slot = rate_slot(g, g->step);
-    CUDA_TRY(cudaMemsetAsync(slot + lo, 0, sizeof(unsigned long long) * (hi - lo), s));
+    if (g->rate_clean && lo == 0 && hi == g->count && s == g->stream) {
+        g->step += 1;
+        ro.rate_zero = rate_slot(g, g->step + 1);
+    } else {
+        CUDA_TRY(cudaMemsetAsync(rate_slot(g, g->step) + lo, 0, sizeof(unsigned long long) * (hi - lo), s));
+    }
     ro.coef = (const GridCoef<T> *)g->d_coef;
     ro.vdx = (const T *)g->vdx;
     ro.vdy = (const T *)g->vdy;
     ro.solid = g->solid;
-    ro.rate = slot;
+    ro.rate = rate_slot(g, g->step);
     ro.curv = g->curv;
     return ROEAM_OK;
 }

@@ -130,6 +130,7 @@ template <typename T> struct RateOut {
     const T *vdx = nullptr, *vdy = nullptr;
     const uint8_t *solid = nullptr;
     unsigned long long *rate = nullptr;
+    unsigned long long *rate_zero = nullptr;   // slots to reset (the next step's output), may be null
     int curv = 0;
 };
 

@@ -68,8 +68,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
     constexpr int H = MUSCL ? 2 : 1;
     constexpr int E = H * STAGES;
     constexpr bool PAIRS = sizeof(T) == 4;   // FP32 evaluates a cell's west and south faces as one packed pair
-    // The next launch may start; it waits below (like this one) before it touches the state.
-    asm volatile("griddepcontrol.launch_dependents;");
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T red[tile_threads<T>() / 32];
 
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
     };
 
     // everything from here on may depend on the launch before this one
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     if (a.rate_zero && blockIdx.x == 0)
         for (int q = tid; q < a.ngrids; q += nt) a.rate_zero[q] = 0ull;
     {
@@ -601,17 +600,7 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS> struct TileVariant {
     static constexpr int STAGES = tile_stages<T>();
     static cudaError_t launch(const TileArgs<T> &a, int ntiles, int threads, size_t smem, cudaStream_t s)
     {
-        cudaLaunchConfig_t c = {};
-        c.gridDim = dim3((unsigned)ntiles);
-        c.blockDim = dim3((unsigned)threads);
-        c.dynamicSmemBytes = smem;
-        c.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        c.attrs = at;
-        c.numAttrs = 1;
-        return cudaLaunchKernelEx(&c, tile_kernel<T, MUSCL, CURV, WALLS, STAGES>, a);
+        return launch_pdl(tile_kernel<T, MUSCL, CURV, WALLS, STAGES>, dim3((unsigned)ntiles), dim3((unsigned)threads), smem, s, a);
     }
     static cudaError_t prepare(size_t smem)
     {
