@@ -1,9 +1,9 @@
 // roeam3_api.cu — host implementation of the 3D C ABI declared in include/roeam3.h.
 //
-// Owns the device memory of a batch of 3D grids (pitched structure-of-arrays volumes, one per
-// conserved variable), builds the work units of the 3D stage kernel (30 x 14 columns of a plane
-// in FP32, 30 x 6 in FP64, by a segment of planes), and drives the three fused stage launches of each SSP-RK3 step with
-// per-grid time steps read on the device.
+// Owns the device memory of a batch of 3D grids (pitched rows of cells, each a quad and a tail of
+// values), builds the work units of the 3D stage kernel (a rectangle of columns by a segment of
+// planes), and drives the three fused stage launches of each SSP-RK3 step with per-grid time steps
+// read on the device.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -54,7 +54,8 @@ struct roeam3_grid {
     void *U = nullptr, *A = nullptr, *B = nullptr;
     long long total_elems = 0, total_packed = 0, max_cells = 0;
     int4 *d_units = nullptr;
-    int nunits = 0, nblocks = 0;
+    int nunits = 0, threads = 0;
+    size_t smem = 0;
     unsigned long long *rate = nullptr;   // 2 x count slots, alternating by step parity
     int parity = 0;
     unsigned *status = nullptr;
@@ -135,57 +136,71 @@ roeam_status upload_coef3(roeam3_grid *g, const roeam3_grid_desc *d)
     return ROEAM_OK;
 }
 
-// Work units: 30 x 14 columns of a plane in FP32, 30 x 6 in FP64 (TILE3_X x tile3_y<T>() written
-// cells) by a segment of
-// planes. The number of segments per column starts at about four units per resident CTA and is
-// then chosen, up to twice that, to fill the last round of units over the CTAs (all units cost
-// about the same): the 256^3 Taylor-Green vortex had 1548 units over 304 CTAs, a sixth round
-// 9 % full; 7 segments give 2709 units in 8.9 rounds. Each extra segment re-reads two planes,
-// which the choice weighs at half a plane of work each.
+// Work units: rectangles of at most w x h columns by segments of planes, one CTA each (one fits an SM).
+// FP32 takes 30 x 14 columns; (w, h) in FP64 and the number of segments minimise an estimate of a
+// launch's cycles, units going over the SMs in rounds: planes (a segment costs about one more) times a
+// plane's cycles, which in FP64 are its FP64 operations on an SM's four pipes and three barriers.
+// FP64 threads: one per face of a plane up to 256, also where there are fewer positions than that: two warps
+// per scheduler hide each other's latency (32^3: 398 us a step with a thread per position, 241 with 256;
+// 384 threads: 64^3 1348 us against 1332, 16^3 126 against 103, 95 x 63 x 127 3519 against 3852).
+template <typename T>
 roeam_status setup_units3(roeam3_grid *g, int num_sms)
 {
-    const int occ = g->precision == 32 ? Launchers3<float>::stage_occupancy(g->nscal)
-                                       : Launchers3<double>::stage_occupancy(g->nscal);
-    g->nblocks = std::max(1, occ * num_sms);
-    const int TILE3_Y = g->precision == 32 ? tile3_y<float>() : tile3_y<double>();
-    long long columns = 0, nk_max = 1;
+    int max_ni = 0, max_nj = 0, max_nk = 0;
     for (const GridDev3 &G : g->hg) {
-        columns += (long long)((G.ni + TILE3_X - 1) / TILE3_X) * ((G.nj + TILE3_Y - 1) / TILE3_Y);
-        nk_max = std::max<long long>(nk_max, G.nk);
+        max_ni = std::max(max_ni, G.ni);
+        max_nj = std::max(max_nj, G.nj);
+        max_nk = std::max(max_nk, G.nk);
     }
-    const long long target = 4ll * g->nblocks;
-    const long long nseg0 = std::max(1ll, (target + columns - 1) / columns);
-    long long nseg = nseg0;
-    {
-        double best = -1.0;
-        for (long long n = nseg0; n <= 2 * nseg0; ++n) {
-            long long units = 0;
-            double planes = 0.0, extra = 0.0;
-            for (const GridDev3 &G : g->hg) {
-                const long long cols = (long long)((G.ni + TILE3_X - 1) / TILE3_X) * ((G.nj + TILE3_Y - 1) / TILE3_Y);
-                const int zs = std::max(4, (int)((G.nk + n - 1) / n));
-                const long long segs = (G.nk + zs - 1) / zs;
-                units += cols * segs;
-                planes += (double)cols * G.nk;
-                extra += (double)cols * segs;   // two re-read planes per segment, at half a plane each
+    const bool f32 = sizeof(T) == 4;
+    const int every = 1 + (g->count - 1) / 16;   // (a sample of a large batch's grids)
+    double best = 1e300;
+    int bw = 0, bh = 0, bn = 1;
+    auto consider = [&](int w, int h, double plane, double segment, double planes_more) {
+        for (int n = 1; n <= std::min(max_nk, 96); ++n) {
+            double units = 0;
+            int zs = 0;
+            for (int q = 0; q < g->count; q += every) {
+                const GridDev3 &G = g->hg[q];
+                const int sn = std::min(n, G.nk);
+                units += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * sn;
+                zs = std::max(zs, (G.nk + sn - 1) / sn);
             }
-            const long long rounds = (units + g->nblocks - 1) / g->nblocks;
-            const double eff = (double)units / (double)(rounds * g->nblocks) * planes / (planes + extra);
-            if (eff > best + 1e-9) { best = eff; nseg = n; }
+            const double cost = std::ceil(units / num_sms) * (plane * (zs + planes_more) + segment);
+            if (cost < best * 0.999) { best = cost; bw = w; bh = h; bn = n; }
         }
-    }
+    };
+    if (f32) consider(MARCH3_X, MARCH3_Y, 5000, 6000, 1.0);
+    else
+        for (int w = 64; w >= 2; w -= 2)
+            for (int h = 2; h <= 64; ++h) {
+                if (w > max_ni + 1 || h > max_nj + 1 || bytes3<T>(w, h, g->nv) == 0) continue;
+                const double faces = (double)(w + 1) * h + (double)w * (h + 1) + (double)w * h;
+                const double positions = (double)(w + 2) * (h + 2);
+                consider(w, h, 2500 + 76 * (std::ceil(faces / 128) * (148 + 9 * g->nscal) +
+                                            std::ceil(positions / 128) * (75 + 7 * g->nv)), 4000, 1.3);
+            }
+    if (bw == 0) return fail3(ROEAM_E_ARG, "no work unit fits");
     std::vector<int4> units;
+    int mw = 0, mh = 0;
     for (int gi = 0; gi < g->count; ++gi) {
         const GridDev3 &G = g->hg[gi];
-        const int zs = std::max(4, (int)((G.nk + nseg - 1) / nseg));
-        for (int k0 = 0; k0 < G.nk; k0 += zs) {
-            const int k1 = std::min(G.nk, k0 + zs);
-            for (int j0 = 0; j0 < G.nj; j0 += TILE3_Y)
-                for (int i0 = 0; i0 < G.ni; i0 += TILE3_X) units.push_back(make_int4(gi, i0, j0, k0 | (k1 << 16)));
-        }
+        const int nx = (G.ni + bw - 1) / bw, ny = (G.nj + bh - 1) / bh, nz = std::min(bn, G.nk);
+        for (int z = 0; z < nz; ++z)
+            for (int y = 0; y < ny; ++y)
+                for (int x = 0; x < nx; ++x) {
+                    const int x0 = (int)((long long)x * G.ni / nx), x1 = (int)((long long)(x + 1) * G.ni / nx);
+                    const int y0 = (int)((long long)y * G.nj / ny), y1 = (int)((long long)(y + 1) * G.nj / ny);
+                    const unsigned z0 = (unsigned)((long long)z * G.nk / nz), z1 = (unsigned)((long long)(z + 1) * G.nk / nz);
+                    units.push_back(make_int4(gi, x0 | (x1 - x0) << 16, y0 | (y1 - y0) << 16, (int)(z0 | z1 << 16)));
+                    mw = std::max(mw, x1 - x0);
+                    mh = std::max(mh, y1 - y0);
+                }
     }
     g->nunits = (int)units.size();
-    g->nblocks = (int)std::min<long long>(g->nblocks, g->nunits);
+    g->smem = bytes3<T>(mw, mh, g->nv);
+    g->threads = f32 ? threads3<T>() : std::min(threads3<T>(), std::max(128, (3 * mw * mh + mw + mh + 31) / 32 * 32));
+    CUDA_TRY3(Launchers3<T>::prepare(g->nscal));
     CUDA_TRY3(cudaMalloc(&g->d_units, sizeof(int4) * units.size()));
     CUDA_TRY3(cudaMemcpy(g->d_units, units.data(), sizeof(int4) * units.size(), cudaMemcpyHostToDevice));
     return ROEAM_OK;
@@ -206,25 +221,17 @@ StageArgs3<T> base_args3(roeam3_grid *g)
 }
 
 template <typename T>
-roeam_status refresh_rate3(roeam3_grid *g)
-{
-    unsigned long long *slot = g->rate + (size_t)g->parity * g->count;
-    CUDA_TRY3(cudaMemsetAsync(slot, 0, sizeof(unsigned long long) * g->count, g->stream));
-    CUDA_TRY3(Launchers3<T>::rate(g->d_grids, (const GridCoef3<T> *)g->d_coef, 0, g->count, (const T *)g->U, g->nscal,
-                                  slot, g->stream));
-    g->launches += 1;
-    return ROEAM_OK;
-}
-
-template <typename T>
 roeam_status do_set3(roeam3_grid *g, int lo, int hi, const double *host)
 {
     const GridDev3 &a = g->hg[lo], &b = g->hg[hi - 1];
     const long long n0 = a.poff, n1 = b.poff + (long long)g->nv * b.ni * b.nj * b.nk;
     CUDA_TRY3(cudaMemcpyAsync(g->staging + n0, host, sizeof(double) * (n1 - n0), cudaMemcpyHostToDevice, g->stream));
-    CUDA_TRY3(Launchers3<T>::pack(g->d_grids, lo, hi, g->nv, g->max_cells, g->staging, (T *)g->U, g->stream));
+    unsigned long long *slot = g->rate + (size_t)g->parity * g->count;
+    CUDA_TRY3(cudaMemsetAsync(slot + lo, 0, sizeof(unsigned long long) * (hi - lo), g->stream));
+    CUDA_TRY3(Launchers3<T>::pack(g->d_grids, (const GridCoef3<T> *)g->d_coef, lo, hi, g->nscal, g->max_cells, g->staging,
+                                  (T *)g->U, slot, g->stream));
     g->launches += 1;
-    return refresh_rate3<T>(g);
+    return ROEAM_OK;
 }
 
 roeam_status sync_status3(roeam3_grid *g)
@@ -241,7 +248,7 @@ roeam_status sync_status3(roeam3_grid *g)
 template <typename T>
 roeam_status do_get3(roeam3_grid *g, int lo, int hi, double *host, const void *src)
 {
-    CUDA_TRY3(Launchers3<T>::unpack(g->d_grids, lo, hi, g->nv, g->max_cells, (const T *)src, g->staging, g->stream));
+    CUDA_TRY3(Launchers3<T>::unpack(g->d_grids, lo, hi, g->nscal, g->max_cells, (const T *)src, g->staging, g->stream));
     g->launches += 1;
     const GridDev3 &a = g->hg[lo], &b = g->hg[hi - 1];
     const long long n0 = a.poff, n1 = b.poff + (long long)g->nv * b.ni * b.nj * b.nk;
@@ -261,13 +268,13 @@ roeam_status launch_step3(roeam3_grid *g, double cfl, double dt_fixed)
     const T *U = (const T *)g->U;
     // stage 1: U1 = U + dt R(U)   (also clears the next step's rate slots)
     a.src = U; a.un = U; a.dst = (T *)g->A; a.alpha = T(0); a.beta = T(1); a.rate_zero = a.rate_wr; a.want_rate = 0;
-    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->nblocks, g->stream));
+    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->threads, g->smem, g->stream));
     // stage 2: U2 = 3/4 U + 1/4 (U1 + dt R(U1))
     a.src = (const T *)g->A; a.dst = (T *)g->B; a.alpha = T(0.75); a.beta = T(0.25); a.rate_zero = nullptr;
-    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->nblocks, g->stream));
+    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->threads, g->smem, g->stream));
     // stage 3: U = 1/3 U + 2/3 (U2 + dt R(U2)), in place; the next step's rate
     a.src = (const T *)g->B; a.dst = (T *)g->U; a.alpha = T(1.0 / 3.0); a.beta = T(2.0 / 3.0); a.want_rate = 1;
-    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->nblocks, g->stream));
+    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->threads, g->smem, g->stream));
     g->launches += 3;
     g->parity ^= 1;
     return ROEAM_OK;
@@ -281,7 +288,7 @@ roeam_status do_residual3(roeam3_grid *g, int lo, int hi, double *out)
     a.src = (const T *)g->U;
     a.un = (const T *)g->U;
     a.dst = (T *)g->A;
-    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->nblocks, g->stream));
+    CUDA_TRY3(Launchers3<T>::stage(a, g->nscal, g->threads, g->smem, g->stream));
     g->launches += 1;
     if (!out) return ROEAM_OK;
     return do_get3<T>(g, lo, hi, out, g->A);
@@ -348,7 +355,7 @@ roeam_status roeam3_create_grid(int count, const roeam3_grid_desc *descs, int de
         G.pitch = (int)round_up3(q.ni, 32);
         G.vol = (long long)q.nk * q.nj * G.pitch;
         G.off = off;
-        off += round_up3((long long)g->nv * G.vol, 64);
+        off += round_up3((long long)(4 + tail3(g->nv)) * G.vol, 64);
         G.poff = poff;
         poff += (long long)g->nv * q.ni * q.nj * q.nk;
         for (int s = 0; s < 6; ++s) G.bc[s] = q.bc[s];
@@ -388,7 +395,7 @@ roeam_status roeam3_create_grid(int count, const roeam3_grid_desc *descs, int de
 #undef CREATE3_TRY
     st = g->precision == 32 ? upload_coef3<float>(g, descs) : upload_coef3<double>(g, descs);
     if (st != ROEAM_OK) return cleanup(st);
-    st = setup_units3(g, num_sms);
+    st = g->precision == 32 ? setup_units3<float>(g, num_sms) : setup_units3<double>(g, num_sms);
     if (st != ROEAM_OK) return cleanup(st);
     *out = g;
     return ROEAM_OK;

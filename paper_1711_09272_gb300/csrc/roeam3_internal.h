@@ -12,8 +12,10 @@ constexpr int MAX_VARS3 = 5 + MAX_SCALARS;
 
 // Per-grid descriptor of a 3D grid, resident in device memory.
 struct GridDev3 {
-    long long off;     // element offset of this grid's variable-0 volume in the state buffers
-    long long vol;     // elements per variable volume (nk * nj * pitch)
+    long long off;     // element offset of this grid in the state buffers: quads (rho, rho u, rho v, rho w)
+                       // of its cells at off + 4 c, c = (k nj + j) pitch + i, then their tails
+                       // (rho E, scalars; tail3(nv) values) at off + 4 vol + tail3(nv) c
+    long long vol;     // cells held (nk * nj * pitch)
     long long poff;    // element offset of this grid in the packed host layout [nv][nk][nj][ni]
     int ni, nj, nk, pitch;
     int bc[6];         // W, E, S, N, B, T
@@ -32,26 +34,33 @@ struct GridCoef3 {
     T inflow[MAX_VARS3];
 };
 
-// Work-unit shape of the 3D stage kernel: a CTA of ty3<T>() warps covers 32 columns (30
-// written) by ty3<T>() rows (two fewer written) and marches along z over a segment of planes.
-// FP32 takes 16-row tiles, one 512-thread CTA per SM at 128 registers (30 x 14 of its 32 x 16
-// cells written; 8-row tiles, two CTAs per SM, write 30 x 6 of 32 x 8 and measured 3.4 % slower
-// on the 256^3 Taylor-Green vortex); FP64, which needs up to 255 registers, 8-row tiles.
-#ifndef ROEAM_TY3_F32
-#define ROEAM_TY3_F32 16
-#endif
-#ifndef ROEAM_TY3_F64
-#define ROEAM_TY3_F64 8
-#endif
-template <typename T> __host__ __device__ constexpr int ty3() { return sizeof(T) == 4 ? ROEAM_TY3_F32 : ROEAM_TY3_F64; }
-template <typename T> __host__ __device__ constexpr int tile3_y() { return ty3<T>() - 2; }
-constexpr int TILE3_X = 30;
+// Values beyond the first four of a cell of nv variables (three are stored as four, so that a tail is
+// one aligned access).
+__host__ __device__ constexpr int tail3(int nv) { return nv - 4 == 3 ? 4 : nv - 4; }
+
+// Threads per CTA of the 3D stage kernel (FP64: at most), and the cells of an FP32 unit: 32 columns by a
+// row per warp, less the halo.
+template <typename T> __host__ __device__ constexpr int threads3() { return sizeof(T) == 4 ? 512 : 256; }
+constexpr int MARCH3_X = 30, MARCH3_Y = threads3<float>() / 32 - 2;
+
+// Shared memory of the 3D stage kernel for a rectangle of w x h cells, or 0 if it does not fit.
+// FP32 (whatever the rectangle): per thread two buffers of exchanged fields (9 + scalars cell values, 3
+// ratios, nv fluxes), four raw cells and two of U^n. FP64: a record of rec3 values per position (cells and
+// a halo of one), at most two positions per thread.
+__host__ __device__ constexpr int rec3(int nv) { return ((56 + 12 * tail3(nv) + 6 + 3) / 4 | 1) * 4; }
+template <typename T> inline size_t bytes3(int w, int h, int nv)
+{
+    if (sizeof(T) == 4)
+        return w <= MARCH3_X && h <= MARCH3_Y ? sizeof(T) * threads3<T>() * (2 * (4 + nv + 3 + nv) + 6 * (4 + tail3(nv))) : 0;
+    const size_t b = sizeof(T) * (size_t)(w + 2) * (h + 2) * rec3(nv);
+    return b <= TILE_SMEM_MAX && (w + 2) * (h + 2) <= 2 * threads3<T>() ? b : 0;
+}
 
 template <typename T>
 struct StageArgs3 {
     const GridDev3 *grids;
     const GridCoef3<T> *coef;
-    const int4 *units;       // (grid, column of lane 0 + 1, row of warp 0 + 1, k0 | k1 << 16)
+    const int4 *units;       // (grid, first column | width << 16, first row | height << 16, k0 | k1 << 16)
     int ngrids, nunits;
     const T *src, *un;
     T *dst;
@@ -66,13 +75,12 @@ struct StageArgs3 {
 
 template <typename T>
 struct Launchers3 {
-    static cudaError_t stage(const StageArgs3<T> &a, int nscal, int nblocks, cudaStream_t s);
-    static int stage_occupancy(int nscal);
-    static cudaError_t rate(const GridDev3 *grids, const GridCoef3<T> *coef, int g_lo, int g_hi, const T *U, int nscal,
-                            unsigned long long *rate, cudaStream_t s);
-    static cudaError_t pack(const GridDev3 *grids, int g_lo, int g_hi, int nv, long long max_cells,
-                            const double *packed, T *U, cudaStream_t s);
-    static cudaError_t unpack(const GridDev3 *grids, int g_lo, int g_hi, int nv, long long max_cells, const T *U,
+    static cudaError_t stage(const StageArgs3<T> &a, int nscal, int threads, size_t smem, cudaStream_t s);
+    static cudaError_t prepare(int nscal);   // lets the stage kernel take the shared memory it may ask for
+    // Packed float64 host layout <-> state; the pack raises rate[g] (zeroed by the caller).
+    static cudaError_t pack(const GridDev3 *grids, const GridCoef3<T> *coef, int g_lo, int g_hi, int nscal,
+                            long long max_cells, const double *packed, T *U, unsigned long long *rate, cudaStream_t s);
+    static cudaError_t unpack(const GridDev3 *grids, int g_lo, int g_hi, int nscal, long long max_cells, const T *U,
                               double *packed, cudaStream_t s);
     static cudaError_t totals(const GridDev3 *grids, int g, const T *U, int nv, double *partials, int nblocks,
                               cudaStream_t s);

@@ -487,6 +487,19 @@ template <typename T> __device__ __forceinline__ T rate_value(unsigned long long
 template <> __device__ __forceinline__ float rate_value<float>(unsigned long long b) { return __uint_as_float((unsigned)b); }
 template <> __device__ __forceinline__ double rate_value<double>(unsigned long long b) { return __longlong_as_double((long long)b); }
 
+// Largest of a warp's non-negative rates, through the bit patterns (redux: one instruction per word).
+__device__ __forceinline__ float warp_rate_max(float r)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(r)));
+}
+__device__ __forceinline__ double warp_rate_max(double r)
+{
+    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return __hiloint2double((int)mh, (int)ml);
+}
+
 // Boundary resolution of one index direction: a cell index outside [0, n) maps to the
 // source index of its ghost value and a kind: 0 interior/periodic/outflow (a plain copy of
 // the source cell), 1 WALL (the source cell mirrored about the boundary face), 2 INFLOW (the

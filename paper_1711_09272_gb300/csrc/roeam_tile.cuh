@@ -49,19 +49,6 @@ template <typename T> __device__ __forceinline__ void copy_value(T *dst, const T
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"((int)sizeof(T)) : "memory");
 }
 
-// Largest of a warp's non-negative rates, through the bit patterns (redux: one instruction per word).
-__device__ __forceinline__ float warp_rate_max(float r)
-{
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(r)));
-}
-__device__ __forceinline__ double warp_rate_max(double r)
-{
-    const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
-    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    return __hiloint2double((int)mh, (int)ml);
-}
-
 template <typename T, bool MUSCL, bool CURV, bool WALLS, int STAGES>
 __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<T> a)
 {
