@@ -535,22 +535,41 @@ template <typename T> __device__ __forceinline__ T ratio_P(T r0, T p0, T r1, T p
 // (a|b| + |a|b) / (|a|+|b|) = 2 a b / (a + b) when ab > 0, else 0. The sign test and the van
 // Leer quotient avoid the product a b, which in FP32 underflows for differences below ~1e-19
 // (a state scaled by 1e-24 is as valid as the unscaled one).
-template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V b)
-{
-    const V zero = splat<V>(0);
-    const auto keep = gt(a * vcopysign(splat<V>(1), b), zero);   // same signs, a != 0
-    if (vanleer) {
-        return sel(keep, (a + a) * (b * rcp(a + b)), zero);
-    }
-    return sel(keep, sel(gt(a, zero), vmin(a, b), vmax(a, b)), zero);
-}
-
-// The same in FP64 with its sign tests on the bit patterns.
+template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V b);
 template <> __device__ __forceinline__ double limiter<double>(bool vanleer, double a, double b)
 {
+    // (sign tests on the bit patterns)
     const bool keep = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && ((dbits(a) << 1) != 0);
     const double m = vanleer ? (a + a) * (b * rcp(a + b)) : copysign(imin(fabs(a), fabs(b)), a);
     return keep ? m : 0.0;
+}
+
+// Half the limited slope in FP32, without sign tests. Van Leer: with s = a + b, the fractions a / s and
+// b / s lie in (0, 1) when the signs agree and multiply to a b / s^2; when they differ, one is negative
+// and the other above 1, and clamped to [0, 1] their product is 0 (as is 0 / 0, which clamps to 0).
+// Minmod: max(0, min(a, b)) + min(0, max(a, b)). Nine and ten instructions for a pair, against thirteen
+// with sign tests and selects; with one branch on the limiter for the four variables instead of one each
+// (and the pairs built normal velocity first) a van Leer step of 96 grids took 2649 -> 2367 us, the
+// 4096^2 warped step 7190 -> 6822.
+__device__ __forceinline__ float mul_sat(float a, float b) { float r; asm("mul.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ V2 mul_sat(V2 a, V2 b) { return mk2(mul_sat(a.v.x, b.v.x), mul_sat(a.v.y, b.v.y)); }
+template <typename V> __device__ __forceinline__ V half_vanleer(V a, V b)
+{
+    const V s = a + b, r = rcp(s);
+    return s * (mul_sat(a, r) * mul_sat(b, r));
+}
+template <typename V> __device__ __forceinline__ V half_minmod(V a, V b)
+{
+    const V zero = splat<V>(0);
+    return splat<V>(0.5f) * (vmx(zero, vmn(a, b)) + vmn(zero, vmx(a, b)));
+}
+template <typename V> __device__ __forceinline__ V half_slope(bool vanleer, V a, V b)
+{
+    return vanleer ? half_vanleer(a, b) : half_minmod(a, b);
+}
+template <> __device__ __forceinline__ double half_slope<double>(bool vanleer, double a, double b)
+{
+    return 0.5 * limiter(vanleer, a, b);
 }
 
 // Cell-window entry: primitives (rho, u, v, p) in the global frame, the derived face
@@ -623,10 +642,10 @@ __device__ __forceinline__ void face_scalar(const Face<T> &f, const GridCoef<T> 
         if (f.Bp.fl & 1) { for (int k = 0; k < 4; ++k) M3[k] = WR[k]; mirror_vel(M3[1], M3[2], f.nBpx, f.nBpy); }
         T lL[4], lR[4], rL[4], rR[4];
         for (int k = 0; k < 4; ++k) {
-            lL[k] = limiter(vanleer, WL[k] - M0[k], WR[k] - WL[k]);
-            lR[k] = limiter(vanleer, WR[k] - WL[k], M3[k] - WR[k]);
-            rL[k] = vfma(T(0.5), lL[k], WL[k]);
-            rR[k] = vfnma(T(0.5), lR[k], WR[k]);
+            lL[k] = half_slope(vanleer, WL[k] - M0[k], WR[k] - WL[k]);
+            lR[k] = half_slope(vanleer, WR[k] - WL[k], M3[k] - WR[k]);
+            rL[k] = WL[k] + lL[k];
+            rR[k] = WR[k] - lR[k];
         }
         // Positivity of the reconstructed density and pressure, else first order. In FP32 a
         // density or pressure that comes out within rounding of zero (or below it) is
@@ -670,7 +689,8 @@ __device__ __forceinline__ void face_scalar(const Face<T> &f, const GridCoef<T> 
 // Packed FP32 evaluation of a lane's x-face (component x) and y-face (component y), both free
 // of walls. Cartesian faces enter with their normal velocity first (the y-face's (v, u) is a
 // relabelling, undone on output); curvilinear faces are rotated by their normals. WL / WR are
-// the reconstructed states (global frame) of the reconstructing kernels.
+// the reconstructed states of the reconstructing kernels, in the global frame on curvilinear grids, with
+// the normal velocity first on Cartesian ones.
 template <bool MUSCL, bool CURV>
 __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<float> &fy, const GridCoef<float> &K,
                                              int eps1, int xi_form, const V2 WL[4], const V2 WR[4], float Fx[4],
@@ -698,8 +718,8 @@ __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<f
             L = side_rot(WL[0], WL[1], WL[2], WL[3], nx, ny, K);
             R = side_rot(WR[0], WR[1], WR[2], WR[3], nx, ny, K);
         } else {
-            L = side_from_prims(WL[0], mk2(WL[1].v.x, WL[2].v.y), mk2(WL[2].v.x, WL[1].v.y), WL[3], K);
-            R = side_from_prims(WR[0], mk2(WR[1].v.x, WR[2].v.y), mk2(WR[2].v.x, WR[1].v.y), WR[3], K);
+            L = side_from_prims(WL[0], WL[1], WL[2], WL[3], K);
+            R = side_from_prims(WR[0], WR[1], WR[2], WR[3], K);
         }
     }
     V2 G2[4];
@@ -1099,9 +1119,9 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         float sy_prev[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (PACKED && MUSCL) {
             const WC<T> &a0 = Wn[H - 2], &b0 = Wn[H - 1], &c0 = Wn[H];
-            const V2 lo = limiter(vanleer, mk2(b0.r, b0.u) - mk2(a0.r, a0.u), mk2(c0.r, c0.u) - mk2(b0.r, b0.u));
-            const V2 hi = limiter(vanleer, mk2(b0.v, b0.p) - mk2(a0.v, a0.p), mk2(c0.v, c0.p) - mk2(b0.v, b0.p));
-            sy_prev[0] = lo.v.x; sy_prev[1] = lo.v.y; sy_prev[2] = hi.v.x; sy_prev[3] = hi.v.y;
+            const V2 lo = half_slope(vanleer, mk2(b0.r, b0.u) - mk2(a0.r, a0.u), mk2(c0.r, c0.u) - mk2(b0.r, b0.u));
+            const V2 hi = half_slope(vanleer, mk2(b0.v, b0.p) - mk2(a0.v, a0.p), mk2(c0.v, c0.p) - mk2(b0.v, b0.p));
+            sy_prev[0] = lo.v.x; sy_prev[CURV ? 1 : 2] = lo.v.y; sy_prev[CURV ? 2 : 1] = hi.v.x; sy_prev[3] = hi.v.y;
         }
         T acc[4] = {T(0), T(0), T(0), T(0)};
         T my_rate = T(0);
@@ -1170,16 +1190,23 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             // west cell's x-slope and the south cell's y-slope (carried from the row before)
             V2 WLp[4], WRp[4];
             if constexpr (PACKED && MUSCL) {
-                const float Ax[4] = {fx.A.r, fx.A.u, fx.A.v, fx.A.p}, Ay[4] = {fy.A.r, fy.A.u, fy.A.v, fy.A.p};
-                const float Bc[4] = {fx.B.r, fx.B.u, fx.B.v, fx.B.p};
-                const float Px_[4] = {fx.Bp.r, fx.Bp.u, fx.Bp.v, fx.Bp.p}, Py_[4] = {fy.Bp.r, fy.Bp.u, fy.Bp.v, fy.Bp.p};
-                const V2 half = mk2(0.5f, 0.5f);
+                // (Cartesian: in the order of the faces, normal velocity first)
+                const float Ax[4] = {fx.A.r, fx.A.u, fx.A.v, fx.A.p}, Bx[4] = {fx.B.r, fx.B.u, fx.B.v, fx.B.p};
+                const float Cx[4] = {fx.Bp.r, fx.Bp.u, fx.Bp.v, fx.Bp.p};
+                const float Ay[4] = {fy.A.r, CURV ? fy.A.u : fy.A.v, CURV ? fy.A.v : fy.A.u, fy.A.p};
+                const float By[4] = {fy.B.r, CURV ? fy.B.u : fy.B.v, CURV ? fy.B.v : fy.B.u, fy.B.p};
+                const float Cy[4] = {fy.Bp.r, CURV ? fy.Bp.u : fy.Bp.v, CURV ? fy.Bp.v : fy.Bp.u, fy.Bp.p};
+                V2 sg[4];
+                if (vanleer)
+                    for (int k = 0; k < 4; ++k)
+                        sg[k] = half_vanleer(mk2(Bx[k], By[k]) - mk2(Ax[k], Ay[k]), mk2(Cx[k], Cy[k]) - mk2(Bx[k], By[k]));
+                else
+                    for (int k = 0; k < 4; ++k)
+                        sg[k] = half_minmod(mk2(Bx[k], By[k]) - mk2(Ax[k], Ay[k]), mk2(Cx[k], Cy[k]) - mk2(Bx[k], By[k]));
                 for (int k = 0; k < 4; ++k) {
-                    const V2 A2 = mk2(Ax[k], Ay[k]), B2 = mk2(Bc[k], Bc[k]);
-                    const V2 sg = limiter(vanleer, B2 - A2, mk2(Px_[k], Py_[k]) - B2);
-                    WRp[k] = vfma(mk2(-0.5f, -0.5f), sg, B2);
-                    WLp[k] = vfma(half, mk2(shup(sg.v.x, 1), sy_prev[k]), A2);
-                    sy_prev[k] = sg.v.y;
+                    WRp[k] = mk2(Bx[k], By[k]) - sg[k];
+                    WLp[k] = mk2(Ax[k], Ay[k]) + mk2(shup(sg[k].v.x, 1), sy_prev[k]);
+                    sy_prev[k] = sg[k].v.y;
                 }
             }
             T Fw[4], Fs[4];

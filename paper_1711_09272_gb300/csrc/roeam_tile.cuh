@@ -326,16 +326,24 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                         if (fln) { for (int k = 0; k < 4; ++k) qn[k] = q[k]; geom_y(c, r + 1, nx, ny, l); mirror_vel(qn[1], qn[2], nx, ny); }
                     }
                 }
+                // (FP32: half the slopes)
                 T sx[4], sy[4];
-                for (int k = 0; k < 4; ++k) {
-                    if constexpr (PAIRS) {
-                        const V2 B = mk2(q[k], q[k]);
-                        const V2 sl = limiter(vanleer, B - mk2(qw[k], qs[k]), mk2(qe[k], qn[k]) - B);
-                        sx[k] = sl.v.x; sy[k] = sl.v.y;
-                    } else {
-                        sx[k] = limiter(vanleer, q[k] - qw[k], qe[k] - q[k]);
-                        sy[k] = limiter(vanleer, q[k] - qs[k], qn[k] - q[k]);
+                auto slopes = [&](auto limited) {
+                    for (int k = 0; k < 4; ++k) {
+                        if constexpr (PAIRS) {
+                            const V2 B = mk2(q[k], q[k]), sl = limited(B - mk2(qw[k], qs[k]), mk2(qe[k], qn[k]) - B);
+                            sx[k] = sl.v.x; sy[k] = sl.v.y;
+                        } else {
+                            sx[k] = limited(q[k] - qw[k], qe[k] - q[k]);
+                            sy[k] = limited(q[k] - qs[k], qn[k] - q[k]);
+                        }
                     }
+                };
+                if constexpr (PAIRS) {
+                    if (vanleer) slopes([](V2 a, V2 b) { return half_vanleer(a, b); });
+                    else slopes([](V2 a, V2 b) { return half_minmod(a, b); });
+                } else {
+                    slopes([&](T a, T b) { return limiter(vanleer, a, b); });
                 }
                 st_cell(A2 + 4 * at, sx);
                 st_cell(SY + 4 * at, sy);
@@ -360,10 +368,11 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
             if constexpr (MUSCL) {
                 if (!WALLS || (fA | fB) == 0) {
                     const T *S = d == 1 ? A2 : SY;
+                    const T h = PAIRS ? T(1) : T(0.5);
                     T sA[4], sB[4], rL[4], rR[4];
                     ld_own(S + 4 * (at - d), sA);
                     ld_own(S + 4 * at, sB);
-                    for (int k = 0; k < 4; ++k) { rL[k] = vfma(T(0.5), sA[k], L[k]); rR[k] = vfnma(T(0.5), sB[k], Rr[k]); }
+                    for (int k = 0; k < 4; ++k) { rL[k] = vfma(h, sA[k], L[k]); rR[k] = vfnma(h, sB[k], Rr[k]); }
                     if (rL[0] > T(0) && rL[3] > T(0) && rR[0] > T(0) && rR[3] > T(0))
                         for (int k = 0; k < 4; ++k) { L[k] = rL[k]; Rr[k] = rR[k]; }
                 }
@@ -425,7 +434,10 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                 const bool okx = sides(at, 1, fx.nx, fx.ny, Lx, Rx), oky = sides(at, W, fy.nx, fy.ny, Ly, Ry);
                 V2 WL[4], WR[4];
                 if constexpr (MUSCL) {
-                    for (int k = 0; k < 4; ++k) { WL[k] = mk2(Lx[k], Ly[k]); WR[k] = mk2(Rx[k], Ry[k]); }
+                    for (int k = 0; k < 4; ++k) {   // (Cartesian: the normal velocity first)
+                        const int ky = CURV || k == 0 || k == 3 ? k : 3 - k;
+                        WL[k] = mk2(Lx[k], Ly[ky]); WR[k] = mk2(Rx[k], Ry[ky]);
+                    }
                 } else {
                     auto put = [&](const float v[4], int q, WC<float> &o) {
                         float d4[4];
