@@ -1158,7 +1158,7 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
         CREATE_TRY(cudaMalloc(&g->vdy, g->esize * (size_t)g->total_vert));
     }
     if (any_solid) {
-        CREATE_TRY(cudaMalloc(&g->solid, (size_t)g->total_solid));
+        CREATE_TRY(cudaMalloc(&g->solid, (size_t)g->total_solid + 3));   // (read by aligned words)
         std::vector<uint8_t> hs(g->total_solid, 0);
         for (int k = 0; k < count; ++k)
             if (descs[k].solid)

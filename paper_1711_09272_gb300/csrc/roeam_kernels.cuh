@@ -598,11 +598,6 @@ template <typename T> struct Face {
     T nx, ny, len, nAmx, nAmy, nBpx, nBpy, s1;
 };
 
-template <typename T> __device__ __forceinline__ bool face_is_wall(const Face<T> &f, bool muscl)
-{
-    return (f.A.fl | f.B.fl) != 0 || (muscl && ((f.Am.fl | f.Bp.fl) & 1));
-}
-
 // Face-frame side from global primitives (rotation by the face normal).
 template <typename V, typename S>
 __device__ __forceinline__ FS<V> side_rot(V r, V u, V v, V p, V nx, V ny, const GridCoef<S> &K)
@@ -622,6 +617,26 @@ __device__ __forceinline__ FS<V> side_rot(V r, V u, V v, V p, V nx, V ny, const 
 // FP32 with a wide margin (rounding moves a value by a few ulps of the larger cell value, far
 // less than the smaller one); the positivity fallback to first order therefore never fires
 // there, and the scalar path keeps it for every other face.
+
+// Unit normal and length of a face from its normal vector (sx, sy); of a lane's x- and y-face (a pair in FP32).
+template <typename V> __device__ __forceinline__ void unit_normal(V sx, V sy, V &nx, V &ny, V &len)
+{
+    const V s2 = vfma(sx, sx, sy * sy), li = rsq(s2);
+    len = s2 * li;
+    nx = sx * li; ny = sy * li;
+}
+__device__ __forceinline__ void face_geom(double ax, double ay, double bx, double by, Face<double> &fx, Face<double> &fy)
+{
+    unit_normal(ax, ay, fx.nx, fx.ny, fx.len);
+    unit_normal(bx, by, fy.nx, fy.ny, fy.len);
+}
+__device__ __forceinline__ void face_geom(float ax, float ay, float bx, float by, Face<float> &fx, Face<float> &fy)
+{
+    V2 nx, ny, l;
+    unit_normal(mk2(ax, bx), mk2(ay, by), nx, ny, l);
+    fx.nx = nx.v.x; fx.ny = ny.v.x; fx.len = l.v.x;
+    fy.nx = nx.v.y; fy.ny = ny.v.y; fy.len = l.v.y;
+}
 
 // Scalar evaluation of one face: walls (first-order state and its mirror), MUSCL with solid
 // mirrors and the FP64 positivity decision in FP32, rotation to the face frame, flux, and the
@@ -679,10 +694,11 @@ __device__ __forceinline__ void face_scalar(const Face<T> &f, const GridCoef<T> 
     }
     T G2[4];
     roeam_flux2<ABL>(L, R, f.s1, K, eps1, xi_form, G2, var);
-    const T h = T(0.5) * f.len;
+    // (the same operations as in faces_packed)
+    const T h = T(0.5) * f.len, hx = h * f.nx, hy = h * f.ny;
     F[0] = h * G2[0];
-    F[1] = h * vfnma(f.ny, G2[2], f.nx * G2[1]);
-    F[2] = h * vfma(f.ny, G2[1], f.nx * G2[2]);
+    F[1] = vfma(hx, G2[1], -(hy * G2[2]));
+    F[2] = vfma(hy, G2[1], hx * G2[2]);
     F[3] = h * G2[3];
 }
 
@@ -697,14 +713,14 @@ __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<f
                                              float Fy[4])
 {
     FS<V2> L, R;
+    const V2 nx = mk2(fx.nx, fy.nx), ny = mk2(fx.ny, fy.ny), nyn = mk2(-fx.ny, -fy.ny);
     if constexpr (!MUSCL) {
         const WC<float> &a = fx.A, &b = fx.B, &c = fy.A, &d = fy.B;
         if constexpr (CURV) {
-            const V2 nx = mk2(fx.nx, fy.nx), ny = mk2(fx.ny, fy.ny);
             const V2 uL = mk2(a.u, c.u), vL = mk2(a.v, c.v), uR = mk2(b.u, d.u), vR = mk2(b.v, d.v);
-            L = {mk2(a.r, c.r), vfma(nx, uL, ny * vL), vfma(nx, vL, -(ny * uL)), mk2(a.p, c.p), mk2(a.c2, c.c2),
+            L = {mk2(a.r, c.r), vfma(nx, uL, ny * vL), vfma(nx, vL, nyn * uL), mk2(a.p, c.p), mk2(a.c2, c.c2),
                  mk2(a.H, c.H), mk2(a.sr, c.sr), mk2(a.Mq, c.Mq)};
-            R = {mk2(b.r, d.r), vfma(nx, uR, ny * vR), vfma(nx, vR, -(ny * uR)), mk2(b.p, d.p), mk2(b.c2, d.c2),
+            R = {mk2(b.r, d.r), vfma(nx, uR, ny * vR), vfma(nx, vR, nyn * uR), mk2(b.p, d.p), mk2(b.c2, d.c2),
                  mk2(b.H, d.H), mk2(b.sr, d.sr), mk2(b.Mq, d.Mq)};
         } else {
             L = {mk2(a.r, c.r), mk2(a.u, c.v), mk2(a.v, c.u), mk2(a.p, c.p), mk2(a.c2, c.c2), mk2(a.H, c.H),
@@ -714,9 +730,8 @@ __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<f
         }
     } else {
         if constexpr (CURV) {
-            const V2 nx = mk2(fx.nx, fy.nx), ny = mk2(fx.ny, fy.ny);
-            L = side_rot(WL[0], WL[1], WL[2], WL[3], nx, ny, K);
-            R = side_rot(WR[0], WR[1], WR[2], WR[3], nx, ny, K);
+            L = side_from_prims(WL[0], vfma(nx, WL[1], ny * WL[2]), vfma(nx, WL[2], nyn * WL[1]), WL[3], K);
+            R = side_from_prims(WR[0], vfma(nx, WR[1], ny * WR[2]), vfma(nx, WR[2], nyn * WR[1]), WR[3], K);
         } else {
             L = side_from_prims(WL[0], WL[1], WL[2], WL[3], K);
             R = side_from_prims(WR[0], WR[1], WR[2], WR[3], K);
@@ -725,15 +740,10 @@ __device__ __forceinline__ void faces_packed(const Face<float> &fx, const Face<f
     V2 G2[4];
     roeam_flux2(L, R, mk2(fx.s1, fy.s1), K, eps1, xi_form, G2);
     if constexpr (CURV) {
-        const float hx = 0.5f * fx.len, hy = 0.5f * fy.len;
-        Fx[0] = hx * G2[0].v.x;
-        Fx[3] = hx * G2[3].v.x;
-        Fy[0] = hy * G2[0].v.y;
-        Fy[3] = hy * G2[3].v.y;
-        Fx[1] = hx * vfnma(fx.ny, G2[2].v.x, fx.nx * G2[1].v.x);
-        Fx[2] = hx * vfma(fx.ny, G2[1].v.x, fx.nx * G2[2].v.x);
-        Fy[1] = hy * vfnma(fy.ny, G2[2].v.y, fy.nx * G2[1].v.y);
-        Fy[2] = hy * vfma(fy.ny, G2[1].v.y, fy.nx * G2[2].v.y);
+        const V2 h = mk2(0.5f, 0.5f) * mk2(fx.len, fy.len), hx = h * nx;
+        const V2 F0 = h * G2[0], F1 = vfma(hx, G2[1], (h * nyn) * G2[2]), F2 = vfma(h * ny, G2[1], hx * G2[2]), F3 = h * G2[3];
+        Fx[0] = F0.v.x; Fx[1] = F1.v.x; Fx[2] = F2.v.x; Fx[3] = F3.v.x;
+        Fy[0] = F0.v.y; Fy[1] = F1.v.y; Fy[2] = F2.v.y; Fy[3] = F3.v.y;
     } else {
         // (twice the flux: the residual applies the half lengths)
         Fx[0] = G2[0].v.x;
@@ -823,7 +833,7 @@ __device__ __forceinline__ void st_cell(double *p, const double q[4])
 // Address of the four values of cell c (row * pitch + column) of a grid's block.
 template <typename T> __device__ __forceinline__ T *cell_at(T *base, int c) { return base + 4 * (long long)c; }
 
-// Loading a cell is split in two: issue_cell resolves row j (the column is resolved once per unit
+// Loading a cell is split in two: issue_group resolves row j (the column is resolved once per unit
 // into isrc / kx) and starts an asynchronous copy of the cell into this lane's slot of the warp's
 // shared-memory ring, RING_AHEAD rows before finish_cell turns the slot into primitives, derived
 // face quantities and flags. Each lane reads only what it copied itself, so waiting for its own
@@ -843,12 +853,23 @@ template <typename T> __device__ __forceinline__ T *cell_at(T *base, int c) { re
 // at 91 registers (20 warps). 512-grid batch (8 steps, state in and out) 8840 -> 7713 us, 96-grid
 // van Leer batch 2860 -> 2630, 4096^2 warped step 7968 -> 7201.
 constexpr int RING_ROWS = 8, RING_UN = 4, RING_AHEAD = 2;
-template <typename T> __host__ __device__ constexpr int ring_bytes() { return (RING_ROWS + RING_UN) * 32 * 4 * (int)sizeof(T); }
+// The rings of the vertex rows (displacements x, y of each lane's column; curvilinear) and of the solid
+// mask (the aligned word that holds the cell's byte; walls) follow, RING_ROWS rows each: loaded into
+// registers a row ahead, they were waited for where the rows shift (long-scoreboard stalls 1.4 per
+// instruction; now 0.1). With the flags left alone where a warp's rows have none, the faces' geometry and
+// rotation as pairs, and row j - 2 read again only on the scalar path: 4096^2 warped step 6820 -> 6515.
+constexpr int RING_MASK = 32 * 4;
+template <typename T> __host__ __device__ constexpr int ring_vertex() { return 32 * 2 * (int)sizeof(T); }
+template <typename T> __host__ __device__ constexpr int ring_cells() { return (RING_ROWS + RING_UN) * 32 * 4 * (int)sizeof(T); }
+template <typename T, bool CURV, bool WALLS> __host__ __device__ constexpr int ring_bytes()
+{
+    return ring_cells<T>() + (CURV ? RING_ROWS * ring_vertex<T>() : 0) + (WALLS ? RING_ROWS * RING_MASK : 0);
+}
 
 template <typename T> struct Pending {
     T raw[4];
-    int jsrc, ky;
-    int solid;   // the cell's solid-mask byte (kernels with walls)
+    int ky;
+    int solid;   // the cell's solid-mask byte (kernels with walls; 0 without a mask)
 };
 
 __device__ __forceinline__ void cp16(unsigned dst, const void *src)
@@ -860,22 +881,15 @@ template <typename T> __device__ __forceinline__ void copy_cell(unsigned dst, co
     cp16(dst, src);
     if constexpr (sizeof(T) == 8) cp16(dst + 16, src + 2);
 }
+template <typename T> __device__ __forceinline__ void copy_word(unsigned dst, const T *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"((int)sizeof(T)) : "memory");
+}
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename T>
-__device__ __forceinline__ void issue_cell(const GridRegs<T> &R, int isrc, int j, unsigned slot)
-{
-    int ky;
-    const int x = resolve_index(j, R.nj, R.bcS, R.bcN, ky) * R.pitch + isrc;
-    copy_cell(slot, DBG_LD4(R, DB_SRC, cell_at(R.src, x)));
-}
-
-// LATE_SOLID reads the solid-mask byte here instead of taking the one prefetched a row earlier
-// (the ablation kernels, whose scalar path measured faster that way; the main kernels hide
-// that load's latency behind a row of work).
-template <typename T, bool MUSCL, bool CURV, bool WALLS, bool LATE_SOLID = false>
-__device__ __forceinline__ void finish_cell(const GridRegs<T> &R, const GridCoef<T> &K, int i, int isrc, int kx, int j,
+template <typename T, bool MUSCL, bool CURV, bool WALLS>
+__device__ __forceinline__ void finish_cell(const GridRegs<T> &R, const GridCoef<T> &K, int i, int isrc, int kx, bool edge, int j,
                                             const Pending<T> &q, WC<T> &c)
 {
     const int ky = q.ky;
@@ -884,58 +898,61 @@ __device__ __forceinline__ void finish_cell(const GridRegs<T> &R, const GridCoef
     c.r = q.raw[0]; c.u = q.raw[1] * ri; c.v = q.raw[2] * ri;
     c.p = K.gm1 * vfnma(T(0.5) * q.raw[0], vfma(c.u, c.u, c.v * c.v), q.raw[3]);
     if constexpr (WALLS) {
-        if constexpr (LATE_SOLID) { if (R.solid && *DBG_LD(R, DB_SOLID, R.solid + q.jsrc * R.ni + isrc)) c.fl = 1; }
-        else if (q.solid) c.fl = 1;
+        if (q.solid) c.fl = 1;
     }
-    if (kx == 2 || ky == 2) {
-        c.fl = 0;
-        c.r = K.inflow[0]; c.u = K.inflow[1]; c.v = K.inflow[2]; c.p = K.inflow[3];
-    }
-    if constexpr (WALLS) if (kx == 1 || ky == 1) {
-        if (ky == 1 && kx != 2) {
-            T nx = T(0), ny = T(1);
-            if constexpr (CURV) {
-                const int b = (j < 0 ? 0 : R.nj) * R.vpitch + isrc;
-                const T sx = -(*DBG_LD(R, DB_VDY, R.vdy + (b + 1)) - *DBG_LD(R, DB_VDY, R.vdy + b)),
-                        sy = K.dx + (*DBG_LD(R, DB_VDX, R.vdx + (b + 1)) - *DBG_LD(R, DB_VDX, R.vdx + b));
-                const T l = rsq(vfma(sx, sx, sy * sy));
-                nx = sx * l; ny = sy * l;
-            }
-            mirror_vel(c.u, c.v, nx, ny);
+    // (kernels with walls: one uniform test for anything but an interior cell, `edge` saying whether any of
+    //  the warp's columns is a ghost column; without walls the selects below are faster than a branch)
+    if (!WALLS || edge || ky != 0) {
+        if (kx == 2 || ky == 2) {
+            c.fl = 0;
+            c.r = K.inflow[0]; c.u = K.inflow[1]; c.v = K.inflow[2]; c.p = K.inflow[3];
         }
-        if (kx == 1) {
-            T nx = T(1), ny = T(0);
-            if constexpr (CURV) {
-                // (the W/E boundary face of row j, ghost rows of EXCHANGE sides included)
-                const int b = clampi(j, R.bcS == BC_EXCHANGE ? -2 : 0, R.bcN == BC_EXCHANGE ? R.nj + 1 : R.nj - 1) *
-                                  R.vpitch + (i < 0 ? 0 : R.ni);
-                const T sx = K.dy + (*DBG_LD(R, DB_VDY, R.vdy + (b + R.vpitch)) - *DBG_LD(R, DB_VDY, R.vdy + b)),
-                        sy = -(*DBG_LD(R, DB_VDX, R.vdx + (b + R.vpitch)) - *DBG_LD(R, DB_VDX, R.vdx + b));
-                const T l = rsq(vfma(sx, sx, sy * sy));
-                nx = sx * l; ny = sy * l;
+        if constexpr (WALLS) if (kx == 1 || ky == 1) {
+            if (ky == 1 && kx != 2) {
+                T nx = T(0), ny = T(1);
+                if constexpr (CURV) {
+                    const int b = (j < 0 ? 0 : R.nj) * R.vpitch + isrc;
+                    const T sx = -(*DBG_LD(R, DB_VDY, R.vdy + (b + 1)) - *DBG_LD(R, DB_VDY, R.vdy + b)),
+                            sy = K.dx + (*DBG_LD(R, DB_VDX, R.vdx + (b + 1)) - *DBG_LD(R, DB_VDX, R.vdx + b));
+                    const T l = rsq(vfma(sx, sx, sy * sy));
+                    nx = sx * l; ny = sy * l;
+                }
+                mirror_vel(c.u, c.v, nx, ny);
             }
-            mirror_vel(c.u, c.v, nx, ny);
+            if (kx == 1) {
+                T nx = T(1), ny = T(0);
+                if constexpr (CURV) {
+                    // (the W/E boundary face of row j, ghost rows of EXCHANGE sides included)
+                    const int b = clampi(j, R.bcS == BC_EXCHANGE ? -2 : 0, R.bcN == BC_EXCHANGE ? R.nj + 1 : R.nj - 1) *
+                                      R.vpitch + (i < 0 ? 0 : R.ni);
+                    const T sx = K.dy + (*DBG_LD(R, DB_VDY, R.vdy + (b + R.vpitch)) - *DBG_LD(R, DB_VDY, R.vdy + b)),
+                            sy = -(*DBG_LD(R, DB_VDX, R.vdx + (b + R.vpitch)) - *DBG_LD(R, DB_VDX, R.vdx + b));
+                    const T l = rsq(vfma(sx, sx, sy * sy));
+                    nx = sx * l; ny = sy * l;
+                }
+                mirror_vel(c.u, c.v, nx, ny);
+            }
+            if ((kx == 1 || ky == 1) && kx != 2) c.fl |= 2;
         }
-        if ((kx == 1 || ky == 1) && kx != 2) c.fl |= 2;
     }
     derive<T, MUSCL>(c, K);
 }
 
-template <bool WALLS, typename T> __device__ __forceinline__ WC<T> shup_c(const WC<T> &c, int d, bool derived)
+template <typename T> __device__ __forceinline__ WC<T> shup_c(const WC<T> &c, int d, bool derived)
 {
     WC<T> o;
     o.r = shup(c.r, d); o.u = shup(c.u, d); o.v = shup(c.v, d); o.p = shup(c.p, d);
     if (derived) { o.c2 = shup(c.c2, d); o.H = shup(c.H, d); o.sr = shup(c.sr, d); o.Mq = shup(c.Mq, d); }
     else { o.c2 = o.H = o.sr = o.Mq = T(0); }
-    o.fl = WALLS ? __shfl_up_sync(0xffffffffu, c.fl, d) : 0;
+    o.fl = 0;   // (flags: set on the scalar path, the only one that reads them)
     return o;
 }
-template <bool WALLS, typename T> __device__ __forceinline__ WC<T> shdn_c(const WC<T> &c, int d)
+template <typename T> __device__ __forceinline__ WC<T> shdn_c(const WC<T> &c, int d)
 {
     WC<T> o;
     o.r = shdn(c.r, d); o.u = shdn(c.u, d); o.v = shdn(c.v, d); o.p = shdn(c.p, d);
     o.c2 = o.H = o.sr = o.Mq = T(0);
-    o.fl = WALLS ? __shfl_down_sync(0xffffffffu, c.fl, d) : 0;
+    o.fl = 0;
     return o;
 }
 
@@ -968,8 +985,11 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS, int NT, bool ABL>
 __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>())) stage_kernel(const StageArgs<T> a)
 {
     constexpr int H = MUSCL ? 2 : 1;
-    constexpr int NW = H + 2;          // window rows j-H .. j+1
-    constexpr int NV = 4;              // vertex rows j-1 .. j+2 (curvilinear)
+    // window rows j-B0 .. j+1 (row j - 2 is read only by the scalar path; where that is the exception, it
+    // takes the row from the ring again)
+    constexpr bool REREAD = sizeof(T) == 4 && MUSCL && !ABL;
+    constexpr int B0 = REREAD ? 1 : H;
+    constexpr int NW = B0 + 2;
     constexpr int WIDTH = 32 - 2 * H;  // interior columns per strip
     constexpr bool PACKED = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
@@ -985,15 +1005,18 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
     // memory (slot k * NT + thread; only norm launches ask for it), rather than in sixteen
     // registers that every launch would hold
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *const nacc = reinterpret_cast<double *>(smem_raw + NT / 32 * ring_bytes<T>()) + threadIdx.x;
+    constexpr int RING = ring_bytes<T, CURV, WALLS>();
+    double *const nacc = reinterpret_cast<double *>(smem_raw + NT / 32 * RING) + threadIdx.x;
     if (a.mode == MODE_NORM)
         for (int k = 0; k < 8; ++k) nacc[k * NT] = 0.0;
 
-    // this lane's slots of its warp's ring (see issue_cell): state row r, and U^n of row r
+    // this lane's slots of its warp's ring (see issue_group): state row r, and U^n of row r
     constexpr int ROWB = 32 * 4 * (int)sizeof(T);
-    unsigned char *const ring_p = smem_raw + (threadIdx.x >> 5) * ring_bytes<T>() + lane * (4 * (int)sizeof(T));
+    unsigned char *const ring_p = smem_raw + (threadIdx.x >> 5) * RING + lane * (4 * (int)sizeof(T));
     const unsigned ring = (unsigned)__cvta_generic_to_shared(ring_p);
     auto slot_row = [&](int r) { return (r & (RING_ROWS - 1)) * ROWB; };
+    unsigned char *const verts = smem_raw + (threadIdx.x >> 5) * RING + ring_cells<T>();
+    unsigned char *const masks = verts + (CURV ? RING_ROWS * ring_vertex<T>() : 0) + lane * 4;
     auto slot_un = [&](int r) { return (RING_ROWS + (r & (RING_UN - 1))) * ROWB; };
 
     // Each warp takes unit tile_lo + warp first, then (dynamic scheduling) the next unclaimed
@@ -1021,7 +1044,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         R.dbg.lo[DB_DST] = (const unsigned char *)a.dst; R.dbg.bytes[DB_DST] = sizeof(T) * a.n_dst;
         R.dbg.lo[DB_VDX] = (const unsigned char *)a.vdx; R.dbg.bytes[DB_VDX] = sizeof(T) * a.n_vert;
         R.dbg.lo[DB_VDY] = (const unsigned char *)a.vdy; R.dbg.bytes[DB_VDY] = sizeof(T) * a.n_vert;
-        R.dbg.lo[DB_SOLID] = a.solid; R.dbg.bytes[DB_SOLID] = a.n_solid;
+        R.dbg.lo[DB_SOLID] = a.solid; R.dbg.bytes[DB_SOLID] = a.n_solid + 3;   // (aligned words)
         R.dbg.status = a.status;
 #endif
         R.solid = (WALLS && G.soff >= 0) ? a.solid + G.soff : nullptr;
@@ -1035,6 +1058,8 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         }
         int kx;
         const int isrc = resolve_index(i, ni, R.bcW, R.bcE, kx);
+        bool edge = true;
+        if constexpr (WALLS) edge = __any_sync(0xffffffffu, kx != 0);
         const bool icol = i >= 0 && i < ni;
         const bool out_lane = lane >= H && lane < H + WIDTH && icol;
         const T rxy = K.dy / K.dx, cy = T(0.5) * K.dx * K.Vi;   // Cartesian residual weights
@@ -1046,79 +1071,105 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
 
         WC<T> Wn[NW];
         T Px[NW], Py[NW - 1];
-        T vX[NV], vY[NV];
         const bool stage_mode = a.mode == MODE_STAGE;
         const bool combine = stage_mode && a.alpha != T(0);
         const bool un_lane = combine && out_lane;
-        // One copy group per state row r: the row itself and U^n of row r - 2, which is combined
-        // in the iteration after the one that waits for row r. Rows beyond j1 + 1 are not needed.
-        auto issue_group = [&](int r) {
+        // vertex rows 0..nj, and the two ghost vertex rows beyond an EXCHANGE side
+        const int vjlo = R.bcS == BC_EXCHANGE ? -2 : 0, vjhi = R.bcN == BC_EXCHANGE ? nj + 2 : nj;
+        const int vcol = clampi(i, 0, ni);
+        // the word that holds the solid-mask byte of this lane's cell in row j (source row js), and the byte in it
+        auto solid_at = [&](int js) { return reinterpret_cast<unsigned long long>(R.solid + ((long long)js * ni + isrc)); };
+        // One copy group per state row r: the row itself, its vertex row and solid-mask bytes, and U^n of
+        // row r - 2, which is combined in the iteration after the one that waits for row r. Rows beyond
+        // j1 + 1 are not needed.
+        struct Row { int js, ky; };
+        auto row_of = [&](int r) {
+            Row q;
+            q.js = resolve_index(r, nj, R.bcS, R.bcN, q.ky);
+            return q;
+        };
+        auto issue_group = [&](int r, const Row &known) {
             if (r <= j1 + 1) {
-                issue_cell(R, isrc, r, ring + slot_row(r));
+                const Row at = CURV ? known : row_of(r);
+                copy_cell(ring + slot_row(r), DBG_LD4(R, DB_SRC, cell_at(R.src, at.js * R.pitch + isrc)));
                 if (un_lane && r >= j0 + 2)
                     copy_cell(ring + slot_un(r - 2), DBG_LD4(R, DB_UN, cell_at(R.un, (r - 2) * R.pitch + i)));
+                if constexpr (CURV) {
+                    const int b = clampi(r, vjlo, vjhi) * R.vpitch + vcol;
+                    const unsigned d = (unsigned)__cvta_generic_to_shared(verts) + (r & (RING_ROWS - 1)) * ring_vertex<T>() + lane * (2 * (int)sizeof(T));
+                    copy_word(d, DBG_LD(R, DB_VDX, R.vdx + b));
+                    copy_word(d + (int)sizeof(T), DBG_LD(R, DB_VDY, R.vdy + b));
+                }
+                if constexpr (WALLS) {
+                    if (R.solid) {
+                        const unsigned *q = reinterpret_cast<const unsigned *>(solid_at(at.js) & ~3ull);
+                        copy_word((unsigned)__cvta_generic_to_shared(masks) + (r & (RING_ROWS - 1)) * RING_MASK, DBG_LD(R, DB_SOLID, q));
+                    }
+                }
             }
             copies_commit();
         };
-        // the solid-mask byte of row j's cell; without a mask an unused byte (any readable address),
-        // so that the load is unconditional (a load that merges with another value at the end of a
-        // branch is waited for there)
-        const uint8_t *solid_p = R.solid ? R.solid : reinterpret_cast<const uint8_t *>(a.grids);
-        const int solid_pitch = R.solid ? R.ni : 0;
-        auto solid_of = [&](int j) {
-            int ky;
-            const int js = resolve_index(j, R.nj, R.bcS, R.bcN, ky);
-            return (int)__ldg(solid_p + (long long)js * solid_pitch + (solid_pitch ? isrc : 0));
+        // waits for all but the last RING_AHEAD groups; vertices are read by the neighbour lane, too
+        auto wait_rows = [&]() {
+            copies_wait<RING_AHEAD>();
+            if constexpr (CURV) __syncwarp();
         };
-        auto finish_row = [&](int j, int sol, WC<T> &c) {
+        // displacements of vertex (i + d, r), d = 0 or 1 (the last lane: its own)
+        auto vertex = [&](int r, int d, T &x, T &y) {
+            const T *v = reinterpret_cast<const T *>(verts + (r & (RING_ROWS - 1)) * ring_vertex<T>()) + 2 * (d ? (lane < 31 ? lane + 1 : 31) : lane);
+            x = v[0]; y = v[1];
+        };
+        auto finish_row = [&](int j, const Row &at, WC<T> &c) {
             Pending<T> q;
-            q.jsrc = resolve_index(j, R.nj, R.bcS, R.bcN, q.ky);
-            q.solid = R.solid ? sol : 0;
+            q.ky = at.ky;
+            q.solid = 0;
+            if constexpr (WALLS)
+                if (R.solid) q.solid = masks[(j & (RING_ROWS - 1)) * RING_MASK + (int)(solid_at(at.js) & 3)];
             ld_own(reinterpret_cast<const T *>(ring_p + slot_row(j)), q.raw);
-            finish_cell<T, MUSCL, CURV, WALLS, ABL>(R, K, i, isrc, kx, j, q, c);
+            finish_cell<T, MUSCL, CURV, WALLS>(R, K, i, isrc, kx, edge, j, q, c);
         };
-        // vertex rows 0..nj, and the two ghost vertex rows beyond an EXCHANGE side
-        const int vjlo = R.bcS == BC_EXCHANGE ? -2 : 0, vjhi = R.bcN == BC_EXCHANGE ? nj + 2 : nj;
-        auto vload = [&](int J, T &x, T &y) {
-            if constexpr (CURV) {
-                const int b = clampi(J, vjlo, vjhi) * R.vpitch + clampi(i, 0, ni);
-                x = __ldg(DBG_LD(R, DB_VDX, R.vdx + b)); y = __ldg(DBG_LD(R, DB_VDY, R.vdy + b));
-            } else { x = y = T(0); }
+        // Rows with a solid or wall-ghost cell in any of the warp's columns: bit 0 the row last finished,
+        // bit 1 the one below it, and so on. Where there are none, nothing looks at flags: a lane's
+        // flags, its neighbours' and the selects that depend on them cost a sixth of a row's instructions.
+        unsigned walled = 0;
+        auto wall_row = [&](const WC<T> &c) {
+            if constexpr (WALLS) walled = walled << 1 | (__any_sync(0xffffffffu, c.fl != 0) ? 1u : 0u);
         };
         auto px_of = [&](const WC<T> &c) {   // Eq. 97 on this lane's west face; 1 at solid sides
             const T rl = shup(c.r, 1), pl = shup(c.p, 1);
-            const T P = ratio_P(rl, pl, c.r, c.p);
-            if constexpr (WALLS) {   // (a select: a branch around the ratio would diverge at every wall)
+            T P = ratio_P(rl, pl, c.r, c.p);
+            if (WALLS && (walled & 1)) {
                 const int fl = __shfl_up_sync(0xffffffffu, c.fl, 1);
-                return ((c.fl | fl) & 1) ? T(1) : P;
+                if ((c.fl | fl) & 1) P = T(1);
             }
             return P;
         };
         auto py_of = [&](const WC<T> &lo, const WC<T> &hi) {
-            const T P = ratio_P(lo.r, lo.p, hi.r, hi.p);
-            if constexpr (WALLS) return ((lo.fl | hi.fl) & 1) ? T(1) : P;
+            T P = ratio_P(lo.r, lo.p, hi.r, hi.p);
+            if (WALLS && (walled & 3) && ((lo.fl | hi.fl) & 1)) P = T(1);
             return P;
         };
         // window rows j0-H .. j0+1, and RING_AHEAD rows more on their way
-        for (int r = j0 - H; r <= j0 + 1 + RING_AHEAD; ++r) issue_group(r);
-        for (int v = 0; v < NV; ++v) vload(j0 - 1 + v, vX[v], vY[v]);
-        int sol = 0;
-        int sols[NW];
-        if constexpr (WALLS && !ABL) {
-            for (int w = 0; w < NW; ++w) sols[w] = solid_of(j0 - H + w);
-            sol = solid_of(j0 + 2);
-        }
-        copies_wait<RING_AHEAD>();
+        if constexpr (CURV) __syncwarp();   // (the last unit's vertex rows have been read by all lanes)
+        // row_of rows j + 2 .. j + 2 + RING_AHEAD (curvilinear; on Cartesian grids resolving again is faster)
+        Row rows[RING_AHEAD + 1];
+        for (int r = j0 - H; r <= j0 + 1 + RING_AHEAD; ++r) issue_group(r, row_of(r));
+        if constexpr (CURV)
+            for (int d = 0; d < RING_AHEAD; ++d) rows[d] = row_of(j0 + 2 + d);
+        wait_rows();
+        WC<T> Wm2;   // row j0 - 2
+        if constexpr (REREAD) { finish_row(j0 - 2, row_of(j0 - 2), Wm2); wall_row(Wm2); }
         for (int w = 0; w < NW; ++w) {
-            const int jr = j0 - H + w;
-            finish_row(jr, WALLS && !ABL ? sols[w] : 0, Wn[w]);
+            finish_row(j0 - B0 + w, row_of(j0 - B0 + w), Wn[w]);
+            wall_row(Wn[w]);
             Px[w] = px_of(Wn[w]);
             if (w > 0) Py[w - 1] = py_of(Wn[w - 1], Wn[w]);
         }
         // the y-slope of row j0 - 1 (packed reconstruction), as the loop would have left it
         float sy_prev[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (PACKED && MUSCL) {
-            const WC<T> &a0 = Wn[H - 2], &b0 = Wn[H - 1], &c0 = Wn[H];
+            const WC<T> &a0 = REREAD ? Wm2 : Wn[B0 >= 2 ? B0 - 2 : 0];
+            const WC<T> &b0 = Wn[B0 - 1], &c0 = Wn[B0];
             const V2 lo = half_slope(vanleer, mk2(b0.r, b0.u) - mk2(a0.r, a0.u), mk2(c0.r, c0.u) - mk2(b0.r, b0.u));
             const V2 hi = half_slope(vanleer, mk2(b0.v, b0.p) - mk2(a0.v, a0.p), mk2(c0.v, c0.p) - mk2(b0.v, b0.p));
             sy_prev[0] = lo.v.x; sy_prev[CURV ? 1 : 2] = lo.v.y; sy_prev[CURV ? 2 : 1] = hi.v.x; sy_prev[3] = hi.v.y;
@@ -1133,26 +1184,25 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             // ---- the two faces of this lane: west x-face of row j (cells lane-1 | lane) and
             //      the y-face between rows j-1 and j (window H-1 | H)
             Face<T> fx, fy;
-            fx.A = shup_c<WALLS>(Wn[H], 1, !MUSCL);
-            fx.B = Wn[H];
-            fy.A = Wn[H - 1];
-            fy.B = Wn[H];
+            fx.A = shup_c(Wn[B0], 1, !MUSCL);
+            fx.B = Wn[B0];
+            fy.A = Wn[B0 - 1];
+            fy.B = Wn[B0];
             if constexpr (MUSCL) {
-                // (fx.Am's values are shuffled in on the scalar path, the only one that reads them)
-                fx.Am.fl = WALLS ? __shfl_up_sync(0xffffffffu, Wn[H].fl, 2) : 0;
-                fx.Bp = shdn_c<WALLS>(Wn[H], 1);
-                fy.Am = Wn[H - 2];
-                fy.Bp = Wn[H + 1];
+                // (fx.Am, in FP32 fy.Am, and the flags are fetched on the scalar path, the only one that reads them)
+                fx.Bp = shdn_c(Wn[B0], 1);
+                if constexpr (!REREAD) fy.Am = Wn[B0 - 2];
+                fy.Bp = Wn[B0 + 1];
             } else {
                 fx.Am = fx.Bp = fx.A;
                 fy.Am = fy.Bp = fy.A;
             }
             if (use_s1) {
                 // Eq. 96 in 2D: the face and the transverse faces of both cells.
-                const T pym_l = shup(Py[H - 1], 1), pyp_l = shup(Py[H], 1);
-                const T pxm_r = shdn(Px[H - 1], 1), px0_r = shdn(Px[H], 1);
-                T ax = fmn3(fmn3(Px[H], pym_l, pyp_l), Py[H - 1], Py[H]);
-                T ay = fmn3(fmn3(Py[H - 1], Px[H - 1], pxm_r), Px[H], px0_r);
+                const T pym_l = shup(Py[B0 - 1], 1), pyp_l = shup(Py[B0], 1);
+                const T pxm_r = shdn(Px[B0 - 1], 1), px0_r = shdn(Px[B0], 1);
+                T ax = fmn3(fmn3(Px[B0], pym_l, pyp_l), Py[B0 - 1], Py[B0]);
+                T ay = fmn3(fmn3(Py[B0 - 1], Px[B0 - 1], pxm_r), Px[B0], px0_r);
                 if constexpr (PACKED) {
                     const V2 s1 = detector_of(mk2(ax, ay));
                     fx.s1 = s1.v.x; fy.s1 = s1.v.y;
@@ -1162,17 +1212,14 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             } else {
                 fx.s1 = fy.s1 = T(1);
             }
+            T x00, y00;   // vertex (i, j)
             if constexpr (CURV) {
                 // x-face: vertices (i, j), (i, j+1); y-face: vertices (i, j), (i+1, j)
-                T sx = K.dy + (vY[2] - vY[1]), sy = -(vX[2] - vX[1]);
-                fx.len = sqrt0(vfma(sx, sx, sy * sy));
-                T li = rcp(fx.len);
-                fx.nx = sx * li; fx.ny = sy * li;
-                const T xr = shdn(vX[1], 1), yr = shdn(vY[1], 1);
-                sx = -(yr - vY[1]); sy = K.dx + (xr - vX[1]);
-                fy.len = sqrt0(vfma(sx, sx, sy * sy));
-                li = rcp(fy.len);
-                fy.nx = sx * li; fy.ny = sy * li;
+                T x01, y01, x10, y10;   // (vertices of row j + 1 and of the column to the east)
+                vertex(j, 0, x00, y00);
+                vertex(j + 1, 0, x01, y01);
+                vertex(j, 1, x10, y10);
+                face_geom(K.dy + (y01 - y00), -(x01 - x00), -(y10 - y00), K.dx + (x10 - x00), fx, fy);
                 if constexpr (!MUSCL) {
                     fx.nAmx = fx.nBpx = fx.nx; fx.nAmy = fx.nBpy = fx.ny;
                     fy.nAmx = fy.nBpx = fy.nx; fy.nAmy = fy.nBpy = fy.ny;
@@ -1214,7 +1261,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             // batches without walls or solid cells never do in FP32
             bool scalar = !PACKED || ABL;
             if constexpr (PACKED && WALLS && !ABL)
-                scalar = __any_sync(0xffffffffu, face_is_wall(fx, MUSCL) || face_is_wall(fy, MUSCL));
+                scalar = (walled & (MUSCL ? 15u : 6u)) != 0;   // rows j - 2 .. j + 1, or j - 1 and j
             if constexpr (PACKED && MUSCL) {
                 // faces across a density or pressure jump of 1e5 or more take the scalar path,
                 // where a reconstruction within rounding of zero is decided in FP64 (the
@@ -1223,15 +1270,19 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                     // (the faces' Eq. 97 ratios min/max of rho and p, already at hand for the
                     //  detector, say whether the jump is 1e5 or more)
                     const T eps = T(1e-5);
-                    const bool marginal = Px[H] < eps || Py[H - 1] < eps;
+                    const bool marginal = Px[B0] < eps || Py[B0 - 1] < eps;
                     scalar = __any_sync(0xffffffffu, marginal);
                 }
             }
-            if (scalar) {
-                if constexpr (MUSCL) {
-                    const int fl = fx.Am.fl;
-                    fx.Am = shup_c<WALLS>(Wn[H], 2, false);
-                    fx.Am.fl = fl;
+            if (PACKED && !ABL ? __builtin_expect(scalar, 0) : scalar) {
+                if constexpr (REREAD) finish_row(j - 2, row_of(j - 2), fy.Am);
+                if constexpr (MUSCL) fx.Am = shup_c(Wn[B0], 2, false);
+                if constexpr (WALLS) {
+                    fx.A.fl = __shfl_up_sync(0xffffffffu, Wn[B0].fl, 1);
+                    if constexpr (MUSCL) {
+                        fx.Am.fl = __shfl_up_sync(0xffffffffu, Wn[B0].fl, 2);
+                        fx.Bp.fl = __shfl_down_sync(0xffffffffu, Wn[B0].fl, 1);
+                    }
                 }
                 if constexpr (CURV && MUSCL) {
                     // normals of the faces Am|A and B|Bp of both faces (mirrors at solid cells;
@@ -1239,10 +1290,12 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
                     fx.nAmx = shup(fx.nx, 1); fx.nAmy = shup(fx.ny, 1);
                     fx.nBpx = shdn(fx.nx, 1); fx.nBpy = shdn(fx.ny, 1);
                     // (vertex rows j - 1 and j + 1)
-                    const T x0 = shdn(vX[0], 1), y0 = shdn(vY[0], 1), x2 = shdn(vX[2], 1), y2 = shdn(vY[2], 1);
-                    T tx = -(y0 - vY[0]), ty = K.dx + (x0 - vX[0]), l = rsq(vfma(tx, tx, ty * ty));
+                    T xa, ya, xb, yb, xc, yc, xd, yd;
+                    vertex(j - 1, 0, xa, ya); vertex(j - 1, 1, xb, yb);
+                    vertex(j + 1, 0, xc, yc); vertex(j + 1, 1, xd, yd);
+                    T tx = -(yb - ya), ty = K.dx + (xb - xa), l = rsq(vfma(tx, tx, ty * ty));
                     fy.nAmx = tx * l; fy.nAmy = ty * l;
-                    tx = -(y2 - vY[2]); ty = K.dx + (x2 - vX[2]); l = rsq(vfma(tx, tx, ty * ty));
+                    tx = -(yd - yc); ty = K.dx + (xd - xc); l = rsq(vfma(tx, tx, ty * ty));
                     fy.nBpx = tx * l; fy.nBpy = ty * l;
                 }
                 if constexpr (!PACKED || WALLS || MUSCL) {
@@ -1259,18 +1312,21 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             if (j > j0) {
                 CellGeom<T> cg;
                 if constexpr (CURV) {
-                    const T x00 = vX[0], y00 = vY[0], x01 = vX[1], y01 = vY[1];
-                    const T x10 = shdn(x00, 1), y10 = shdn(y00, 1), x11 = shdn(x01, 1), y11 = shdn(y01, 1);
-                    cg = cell_geom(x00, x10, x01, x11, y00, y10, y01, y11, K.dx, K.dy);
+                    // (the cell's upper vertices are this iteration's row j)
+                    T xa, ya, xb, yb, xd, yd;
+                    vertex(j - 1, 0, xa, ya); vertex(j - 1, 1, xb, yb); vertex(j, 1, xd, yd);
+                    cg = cell_geom(xa, xb, x00, xd, ya, yb, y00, yd, K.dx, K.dy);
                 } else {
                     cg.Xx = K.dy; cg.Xy = T(0); cg.Yx = T(0); cg.Yy = K.dx; cg.V = K.V;
                 }
                 if (out_lane) {
-                    const bool solid = WALLS && (Wn[H - 1].fl & 1);
+                    const bool solid = WALLS && (walled & 4) && (Wn[B0 - 1].fl & 1);
                     // R = D sc: the face sum D and its scale (1 / V, or 1 / (2 dy) for Cartesian
                     // faces); a stage applies dt sc to D in one product
                     T D[4];
-                    for (int k = 0; k < 4; ++k) D[k] = solid ? T(0) : acc[k] - Fs[k];
+                    for (int k = 0; k < 4; ++k) D[k] = acc[k] - Fs[k];
+                    if (solid)
+                        for (int k = 0; k < 4; ++k) D[k] = T(0);
                     const T sc = CURV ? rcp(cg.V) : cy;
                     const int x = (j - 1) * R.pitch + i;
                     if (stage_mode) {
@@ -1330,16 +1386,14 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             // ---- advance the window: row j+2 enters from the ring
             for (int w = 0; w < NW - 1; ++w) { Wn[w] = Wn[w + 1]; Px[w] = Px[w + 1]; }
             for (int w = 0; w < NW - 2; ++w) Py[w] = Py[w + 1];
-            issue_group(j + 2 + RING_AHEAD);
-            copies_wait<RING_AHEAD>();
-            finish_row(j + 2, sol, Wn[NW - 1]);
-            if constexpr (WALLS && !ABL) sol = solid_of(j + 3);
+            if constexpr (CURV) rows[RING_AHEAD] = row_of(j + 2 + RING_AHEAD);
+            issue_group(j + 2 + RING_AHEAD, rows[RING_AHEAD]);
+            wait_rows();
+            finish_row(j + 2, CURV ? rows[0] : row_of(j + 2), Wn[NW - 1]);
+            wall_row(Wn[NW - 1]);
+            for (int d = 0; d < RING_AHEAD; ++d) rows[d] = rows[d + 1];
             Px[NW - 1] = px_of(Wn[NW - 1]);
             Py[NW - 2] = py_of(Wn[NW - 2], Wn[NW - 1]);
-            if constexpr (CURV) {
-                for (int v = 0; v < NV - 1; ++v) { vX[v] = vX[v + 1]; vY[v] = vY[v + 1]; }
-                vload(j + NV - 1, vX[NV - 1], vY[NV - 1]);
-            }
         }
         if (a.want_rate) {
             for (int o = 16; o > 0; o >>= 1) my_rate = vmax(my_rate, __shfl_xor_sync(0xffffffffu, my_rate, o));
@@ -1542,14 +1596,14 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS, bool ABL = false> struc
     static cudaError_t launch(const StageArgs<T> &a, int nblocks, cudaStream_t s)
     {
         // (the rings, and the norm accumulators)
-        const size_t smem = NT / 32 * ring_bytes<T>() + (a.mode == MODE_NORM ? 8 * NT * sizeof(double) : 0);
+        const size_t smem = NT / 32 * ring_bytes<T, CURV, WALLS>() + (a.mode == MODE_NORM ? 8 * NT * sizeof(double) : 0);
         return launch_pdl(stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL>, dim3(nblocks), dim3(NT), smem, s, a);
     }
     static int occupancy()
     {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL>, NT,
-                                                          NT / 32 * ring_bytes<T>()) != cudaSuccess)
+                                                          NT / 32 * ring_bytes<T, CURV, WALLS>()) != cudaSuccess)
             return 1;
         return n > 0 ? n : 1;
     }

@@ -154,9 +154,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
             T xa, ya, xb, yb;
             vtx(c, r, xa, ya); vtx(c, r + 1, xb, yb);
             const T sx = K.dy + (yb - ya), sy = -(xb - xa);
-            len = sqrt0(vfma(sx, sx, sy * sy));
-            const T li = rcp(len);
-            nx = sx * li; ny = sy * li;
+            unit_normal(sx, sy, nx, ny, len);
         } else { nx = T(1); ny = T(0); len = T(2); }   // (the residual applies the Cartesian lengths)
     };
     auto geom_y = [&](int c, int r, T &nx, T &ny, T &len) {
@@ -164,9 +162,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
             T xa, ya, xb, yb;
             vtx(c, r, xa, ya); vtx(c + 1, r, xb, yb);
             const T sx = -(yb - ya), sy = K.dx + (xb - xa);
-            len = sqrt0(vfma(sx, sx, sy * sy));
-            const T li = rcp(len);
-            nx = sx * li; ny = sy * li;
+            unit_normal(sx, sy, nx, ny, len);
         } else { nx = T(0); ny = T(1); len = T(2); }
     };
 
@@ -501,10 +497,10 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                     T G2[4];
                     roeam_flux2(sl, sr, s1, K, eps1, xi_form, G2);
                     if constexpr (CURV) {
-                        const T hl = T(0.5) * len;
+                        const T hl = T(0.5) * len, hx = hl * nx, hy = hl * ny;   // (as face_scalar)
                         F[0] = hl * G2[0];
-                        F[1] = hl * vfnma(ny, G2[2], nx * G2[1]);
-                        F[2] = hl * vfma(ny, G2[1], nx * G2[2]);
+                        F[1] = vfma(hx, G2[1], -(hy * G2[2]));
+                        F[2] = vfma(hy, G2[1], hx * G2[2]);
                         F[3] = hl * G2[3];
                     } else {   // (twice the flux: the residual applies the half lengths)
                         F[0] = G2[0]; F[1] = isx ? G2[1] : G2[2]; F[2] = isx ? G2[2] : G2[1]; F[3] = G2[3];
