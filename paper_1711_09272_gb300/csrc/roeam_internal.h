@@ -91,21 +91,22 @@ struct StageArgs {
 #define STAGE_THREADS_DEF 32
 #endif
 constexpr int STAGE_THREADS = STAGE_THREADS_DEF;
-// Resident CTAs per SM the compiler is asked to fit (register budget): 20 holds the FP32
-// first-order Cartesian kernels to 96 registers, which they fit without spills since the rows in
-// flight left the registers (512-grid batch, 8 steps: 16 warps per SM 8350 us, 20 warps 7927 us);
-// the reconstructing and curvilinear FP32 variants are held to 128 registers (16 warps per SM;
-// at 96 they spill 40 to 250 bytes); FP64 and the ablation variants are left to the compiler.
-#ifndef STAGE_MIN_BLOCKS_FAST
-#define STAGE_MIN_BLOCKS_FAST 20
+// Resident CTAs per SM the compiler is asked to fit (register budget): 20 holds the FP32 Cartesian
+// kernels to 96 registers, which they fit with no spill to speak of since the rows in flight and row
+// j - 2 left the registers (512-grid batch, 8 steps: 16 warps per SM 8350 us, 20 warps 7927 us; 96-grid
+// van Leer batch 2351 and 2226 us). The curvilinear FP32 variants are held to 128 registers (16 warps
+// per SM; at 96 they spill 16 to 80 bytes, and the 4096^2 warped step takes 6957 us against 6514);
+// FP64 and the ablation variants are left to the compiler.
+#ifndef STAGE_MIN_BLOCKS_CART
+#define STAGE_MIN_BLOCKS_CART 20
 #endif
-#ifndef STAGE_MIN_BLOCKS_OTHER
-#define STAGE_MIN_BLOCKS_OTHER 16
+#ifndef STAGE_MIN_BLOCKS_CURV
+#define STAGE_MIN_BLOCKS_CURV 16
 #endif
 template <typename T, bool MUSCL, bool CURV, bool ABL = false>
 constexpr int stage_min_blocks()
 {
-    return (sizeof(T) != 4 || ABL) ? 1 : ((!MUSCL && !CURV) ? STAGE_MIN_BLOCKS_FAST : STAGE_MIN_BLOCKS_OTHER);
+    return (sizeof(T) != 4 || ABL) ? 1 : (!CURV ? STAGE_MIN_BLOCKS_CART : STAGE_MIN_BLOCKS_CURV);
 }
 // dyn: dynamic unit scheduling (the kernels that support it claim units from a counter after
 // their first; 0 = static round robin over the unit table).

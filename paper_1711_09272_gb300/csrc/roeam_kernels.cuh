@@ -1119,9 +1119,11 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
             const T *v = reinterpret_cast<const T *>(verts + (r & (RING_ROWS - 1)) * ring_vertex<T>()) + 2 * (d ? (lane < 31 ? lane + 1 : 31) : lane);
             x = v[0]; y = v[1];
         };
+        // (without walls a row's kind matters only as INFLOW: outside [in_lo, in_hi))
+        const int in_lo = R.bcS == BC_INFLOW ? 0 : -4, in_hi = R.bcN == BC_INFLOW ? nj : nj + 4;
         auto finish_row = [&](int j, const Row &at, WC<T> &c) {
             Pending<T> q;
-            q.ky = at.ky;
+            q.ky = WALLS ? at.ky : (j < in_lo || j >= in_hi ? 2 : 0);
             q.solid = 0;
             if constexpr (WALLS)
                 if (R.solid) q.solid = masks[(j & (RING_ROWS - 1)) * RING_MASK + (int)(solid_at(at.js) & 3)];
