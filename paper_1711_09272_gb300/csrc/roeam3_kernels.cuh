@@ -24,7 +24,7 @@ __device__ __forceinline__ void derive3(C3<T, NS> &c, T ri, const GridCoef3<T> &
     c.c2 = K.g * c.p * ri;
     const T q2 = c.u * c.u + c.v * c.v + c.w * c.w;
     c.H = vfma(c.c2, K.gm1i, T(0.5) * q2);
-    c.sr = c.r * rsq(c.r);
+    c.sr = sqrt1(c.r);
     c.Mq = sqrt0(q2 * rcp(c.c2));
 }
 
@@ -74,11 +74,9 @@ __device__ __forceinline__ void roeam_flux3(const FS3<V, NS> &L, const FS3<V, NS
     const V w = rcp(L.sr + R.sr);
     const V wl = L.sr * w, wr = R.sr * w;
     const V rh = L.sr * R.sr;
-    const V uh = vfma(wl, L.un, wr * R.un);
-    const V vh = vfma(wl, L.ut, wr * R.ut);
-    const V wh = vfma(wl, L.uw, wr * R.uw);
     const V Hh = vfma(wl, L.H, wr * R.H);
     const V du = R.un - L.un, dv = R.ut - L.ut, dw = R.uw - L.uw;
+    const V uh = vfma(wr, du, L.un), vh = vfma(wr, dv, L.ut), wh = vfma(wr, dw, L.uw);   // (wl + wr = 1)
     const V dq2 = vfma(du, du, vfma(dv, dv, dw * dw));
     const V c2h = vfma(splat<V>(K.hgm1) * wl * wr, dq2, vfma(wl, L.c2, wr * R.c2));
     const V chi = rsq(c2h);
@@ -91,8 +89,8 @@ __device__ __forceinline__ void roeam_flux3(const FS3<V, NS> &L, const FS3<V, NS
     const V fM8 = pow8(fM), fMb8 = pow8(fMb);
     const V dp = R.p - L.p;
 
-    const V br = bracket(aU, ch);
-    const V Up = vmx(vfma(splat<V>(S(-0.25)) * fMb * br, vmx(du, zero), aU), zero);   // du <= 0 leaves |U|
+    const V br = bracket4(aU, ch);
+    const V Up = vmx(vfma(fMb * br, vmx(du, zero), aU), zero);   // du <= 0 leaves |U|
 
     const V xfh = xi_form ? half : vfma(splat<V>(S(-0.5)), fMb8, half);   // [1 - f^8(Mbar)] / 2
     V xi = vmx(vfma(xfh, du, vabs(vfma(half, du, L.un))), zero);
@@ -118,11 +116,11 @@ __device__ __forceinline__ void roeam_flux3(const FS3<V, NS> &L, const FS3<V, NS
     const V ct = X * rX;
     const V term = vfma(nh, rX * vmn(aU + nh, ct), vfma(om, Up, vmx(ct - Up, zero)));
     const V nA = s1 * (fM8 - one) * term * dp * rcp(Z);   // -rho delta U_p
-    const V dUu = half * smc * du;
+    const V ns = splat<V>(S(-0.5)) * smc;   // (-delta U_u = ns du)
 
     // Eq. 85 per side (as in roeam_flux2): rho_side (U_side +- xi - dUu) times the side's
     // (1, U, V, W, H, k), plus the pressure and delta U_p terms.
-    const V gL = L.r * (L.un + (xi - dUu)), gR = R.r * (R.un - (xi + dUu));
+    const V gL = L.r * (L.un + vfma(ns, du, xi)), gR = R.r * vfma(ns, du, R.un - xi);
     F[0] = (gL + gR) + nA;
     F[1] = vfma(gL, L.un, vfma(gR, R.un, vfma(nA, uh, L.p + R.p) - pp));
     F[2] = vfma(gL, L.ut, vfma(gR, R.ut, nA * vh));

@@ -181,9 +181,20 @@ __device__ __forceinline__ double rsq(double x)
     const double e = fma(-x * y, y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ double sqrt0(double x) { return dbits(x) > 0 ? x * rsq(x) : 0.0; }
+// Square root of a positive value; in FP64 the same step on x y, one operation and one rounding less
+// than x times the reciprocal square root.
+__device__ __forceinline__ float sqrt1(float x) { return x * rsq(x); }
+__device__ __forceinline__ double sqrt1(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double s = x * y, e = fma(-s, y, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
+}
+__device__ __forceinline__ double sqrt0(double x) { return dbits(x) > 0 ? sqrt1(x) : 0.0; }
 __device__ __forceinline__ V2 rcp(V2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
 __device__ __forceinline__ V2 rsq(V2 x) { return mk2(rsq(x.v.x), rsq(x.v.y)); }
+__device__ __forceinline__ V2 sqrt1(V2 x) { return x * rsq(x); }
 __device__ __forceinline__ V2 sqrt0(V2 x) { return mk2(sqrt0(x.v.x), sqrt0(x.v.y)); }
 
 // copysign(a, b): magnitude of a, sign of b.
@@ -249,21 +260,21 @@ __device__ __forceinline__ FS<V> side_from_prims(V r, V un, V ut, V p, const Gri
     s.c2 = splat<V>(K.g) * p * ri;
     const V q2 = vfma(un, un, ut * ut);
     s.H = vfma(s.c2, splat<V>(K.gm1i), splat<V>(S(0.5)) * q2);
-    s.sr = r * rsq(r);
+    s.sr = sqrt1(r);
     s.Mq = sqrt0(q2 * rcp(s.c2));
     return s;
 }
 
-// The bracket sgn(U + c) - sgn(U - c) of Eq. 92 for |U| and c >= 0: 2 for |U| < c, 1 for
-// |U| = c, 0 above (in FP32 as the sum of two set instructions).
-__device__ __forceinline__ float bracket(float aU, float c) { return setlt(aU, c) + setle(aU, c); }
-__device__ __forceinline__ double bracket(double aU, double c)
+// -1/4 of the bracket sgn(U + c) - sgn(U - c) of Eq. 92 for |U| and c >= 0, which is 2 for |U| < c,
+// 1 for |U| = c and 0 above (in FP32 from the sum of two set instructions).
+__device__ __forceinline__ double bracket4(double aU, double c)
 {
-    return dbits(aU) < dbits(c) ? 2.0 : (dbits(aU) == dbits(c) ? 1.0 : 0.0);
+    return dbits(aU) < dbits(c) ? -0.5 : (dbits(aU) == dbits(c) ? -0.25 : 0.0);
 }
-__device__ __forceinline__ V2 bracket(V2 aU, V2 c)
+__device__ __forceinline__ float bracket4(float aU, float c) { return -0.25f * (setlt(aU, c) + setle(aU, c)); }
+__device__ __forceinline__ V2 bracket4(V2 aU, V2 c)
 {
-    return mk2(setlt(aU.v.x, c.v.x), setlt(aU.v.y, c.v.y)) + mk2(setle(aU.v.x, c.v.x), setle(aU.v.y, c.v.y));
+    return splat<V2>(-0.25f) * (mk2(setlt(aU.v.x, c.v.x), setlt(aU.v.y, c.v.y)) + mk2(setle(aU.v.x, c.v.x), setle(aU.v.y, c.v.y)));
 }
 
 // Ablation variants of the flux (the schemes Section 7 compares with), read per grid by the
@@ -284,7 +295,9 @@ struct Variant { int scheme = 0, dup_mode = 0, ufix = 1, xi_roe = 0; };
 // h = (1 - theta) |U| / 2, one reciprocal for 1 / (theta c^2), Eq. 98 clamped once, Eq. 95
 // without the square root; about 30 of 400 instructions per lane and row. 512-grid batch, 8 steps
 // with the state loaded and read back: 9159 -> 8840 us; 4096^2 warped step, 4 steps: 8109 -> 7968
-// us; FP64 64^2 vortex, 20 steps: 3931 -> 3701 us.
+// us; FP64 64^2 vortex, 20 steps: 3931 -> 3701 us. Velocities averaged from their difference (wl + wr = 1),
+// the factor -1/4 in the bracket and -delta U_u = ns du in the sides' sums save four more: the same batch
+// 7721 -> 7667 us, FP64 256^2 Gresho vortex (10 steps) 2587 -> 2549, FP64 64^3 4 steps 5560 -> 5460.
 template <bool ABL = false, typename V, typename S>
 __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1, const GridCoef<S> &K, int eps1,
                                             int xi_form, V F[4], const Variant &var = Variant())
@@ -296,10 +309,9 @@ __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1
     const V w = rcp(L.sr + R.sr);
     const V wl = L.sr * w, wr = R.sr * w;
     const V rh = L.sr * R.sr;
-    const V uh = vfma(wl, L.un, wr * R.un);
-    const V vh = vfma(wl, L.ut, wr * R.ut);
     const V Hh = vfma(wl, L.H, wr * R.H);
     const V du = R.un - L.un, dv = R.ut - L.ut;
+    const V uh = vfma(wr, du, L.un), vh = vfma(wr, dv, L.ut);   // (wl + wr = 1)
     const V dq2 = vfma(du, du, dv * dv);
     const V c2h = vfma(splat<V>(K.hgm1) * wl * wr, dq2, vfma(wl, L.c2, wr * R.c2));
     const V chi = rsq(c2h);
@@ -346,9 +358,9 @@ __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1
     const V dp = R.p - L.p;
 
     // |U|': the bracket sgn(U + c) - sgn(U - c) is 2 for |U| < c, 1 for |U| = c, 0 above.
-    const V br = bracket(aU, ch);
+    const V br = bracket4(aU, ch);
     // (du <= 0 leaves |U|: the correction is applied to max(du, 0))
-    V Up = vmx(vfma(splat<V>(S(-0.25)) * fMb * br, vmx(du, zero), aU), zero);
+    V Up = vmx(vfma(fMb * br, vmx(du, zero), aU), zero);
     if constexpr (ABL) {
         if (!var.ufix) Up = aU;
     }
@@ -392,13 +404,13 @@ __device__ __forceinline__ void roeam_flux2(const FS<V> &L, const FS<V> &R, V s1
         if (var.dup_mode == 1) nA = zero;
         else if (var.dup_mode == 2) nA = -(vmx(ch - aU, zero) * dp * chi * chi);   // rho x Eq. 17
     }
-    const V dUu = half * smc * du;
+    const V ns = splat<V>(S(-0.5)) * smc;   // (-delta U_u = ns du)
 
     // Eq. 85 assembled per side: the central flux, the xi and delta U_u terms of a side carry
     // the same factor rho_side (U_side + xi - dUu) or rho_side (U_side - xi - dUu) times the
     // side's (1, U, V, H), so each component is two products of that factor plus the
     // pressure and delta U_p terms.
-    const V gL = L.r * (L.un + (xi - dUu)), gR = R.r * (R.un - (xi + dUu));
+    const V gL = L.r * (L.un + vfma(ns, du, xi)), gR = R.r * vfma(ns, du, R.un - xi);
     F[0] = (gL + gR) + nA;
     F[1] = vfma(gL, L.un, vfma(gR, R.un, vfma(nA, uh, L.p + R.p) - pp));
     F[2] = vfma(gL, L.ut, vfma(gR, R.ut, nA * vh));
