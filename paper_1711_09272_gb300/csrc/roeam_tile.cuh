@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                     ld_own(S + 4 * (at - d), sA);
                     ld_own(S + 4 * at, sB);
                     for (int k = 0; k < 4; ++k) { rL[k] = vfma(h, sA[k], L[k]); rR[k] = vfnma(h, sB[k], Rr[k]); }
-                    if (rL[0] > T(0) && rL[3] > T(0) && rR[0] > T(0) && rR[3] > T(0))
+                    // (FP32: positive by the limiters' bounds, the faces where it could fail being marginal_face's)
+                    if (PAIRS || (rL[0] > T(0) && rL[3] > T(0) && rR[0] > T(0) && rR[3] > T(0)))
                         for (int k = 0; k < 4; ++k) { L[k] = rL[k]; Rr[k] = rR[k]; }
                 }
             }
