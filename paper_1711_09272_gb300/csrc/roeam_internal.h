@@ -188,13 +188,13 @@ struct TileArgs {
 };
 
 // Shared memory of a tile of W x R positions (the rectangle and its halo): quads of T per position
-// (U, primitives, two fluxes, derived quantities or two slopes, U^n), the Eq. 97 ratios (one row
+// (U, primitives, two fluxes, derived quantities or two slopes, U^n or U^(1) and U^(2)), the Eq. 97 ratios (one row
 // more: the pair list's unused faces past the last row read it), vertices, column and row maps,
 // flags.
 template <typename T> inline size_t tile_bytes(int W, int R, bool muscl, bool curv, bool walls, int stages)
 {
     const size_t P = (size_t)W * R;
-    return sizeof(T) * (4 * P * (4 + (muscl ? 2 : 1) + (stages == 3 ? 1 : 0)) + 2 * (P + W + 2) +
+    return sizeof(T) * (4 * P * (4 + (muscl ? 2 : 1) + (stages == 3 ? (walls ? 2 : 1) : 0)) + 2 * (P + W + 2) +
                         (curv ? 2 * (size_t)(W + 1) * (R + 1) : 0)) +
            sizeof(int) * 2 * (W + 1 + R + 1) + (walls ? (P + 15) / 16 * 16 : 0);
 }

@@ -11,11 +11,11 @@
 // (H = 1 at first order, 2 with MUSCL) and updates a margin of 2 H, H and 0 cells around its
 // rectangle in the three stages, recomputing what its neighbours also compute, so no CTA waits
 // for another and U^(1), U^(2) never leave shared memory. What bounds a step is then latency and, on
-// the larger grids, instruction issue: of 7 us for a 12 x 10 rectangle, 0.8 are descriptors and maps,
-// 0.5 the load, and a stage takes 0.45 ghost cells, 0.2 ratios, 0.7 fluxes, 0.45 update. The strips
-// take 17 to 25 us a step on these grids whatever their size (three launches of a few serial row
-// iterations each): 256^2 van Leer 24.5 -> 12.7 us a step, 400^2 corner 32 -> 19, 800 x 20 duct
-// 25 -> 7.9.
+// the larger grids, instruction issue: of 7 us for a 16 x 6 rectangle, 0.8 are descriptors and maps,
+// 0.5 the load, and a stage takes 0.2 ratios, 0.7 fluxes, 0.5 update. The strips take 17 to 25 us a step
+// on these grids whatever their size (three launches of a few serial row iterations each): 256^2 van
+// Leer 24.5 -> 12 us a step, 400^2 corner 32 -> 19, 800 x 20 duct 25 -> 7.5 (7.9 with ghost cells in a
+// phase of their own).
 // STAGES = 1 (FP64): one stage per launch. FP64 kernels are bound by the FP64 pipe, so recomputed
 // halos cost time; the phases evaluate each face once per CTA and keep all lanes busy where the
 // strips of a small grid evaluated three rows of faces per two rows of cells. The fluxes take 75 % of
@@ -49,6 +49,8 @@ template <typename T> __device__ __forceinline__ void copy_value(T *dst, const T
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"((int)sizeof(T)) : "memory");
 }
 
+template <bool B> struct Flag { static constexpr bool value = B; };
+
 template <typename T, bool MUSCL, bool CURV, bool WALLS, int STAGES>
 __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<T> a)
 {
@@ -71,14 +73,16 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
     const int eps1 = G.eps1, xi_form = G.xi_form;
     const int W = w + 2 * E, R = h + 2 * E, P = W * R;   // positions: column c is ix0 + c, row r is jy0 + r
     const int ix0 = x0 - E, jy0 = y0 - E;
+    // ghost cells among the positions
+    const bool edge = (!perx && (ix0 < 0 || ix0 + W > ni)) || (!pery && (jy0 < 0 || jy0 + R > nj));
 
     T *const U = reinterpret_cast<T *>(smem_raw);
     T *const A1 = U + 4 * P;
     T *const FX = A1 + 4 * P, *const FY = FX + 4 * P;
     T *const A2 = FY + 4 * P;                       // derived quantities, or x-slopes
     T *const SY = A2 + 4 * P;                       // y-slopes (MUSCL)
-    T *const Un = A2 + (MUSCL ? 8 : 4) * P;         // U^n (STAGES = 3)
-    T *const PP = A2 + ((MUSCL ? 8 : 4) + (STAGES == 3 ? 4 : 0)) * P;   // Eq. 97 ratios of the west and south faces
+    T *const V = A2 + (MUSCL ? 8 : 4) * P;          // STAGES = 3: U^n; with walls U^(1) and U^(2), U staying U^n
+    T *const PP = V + (STAGES == 3 ? (WALLS ? 8 : 4) : 0) * P;   // Eq. 97 ratios of the west and south faces
     T *const VV = PP + 2 * (P + W + 2);                       // vertex displacements (CURV): (W + 1) x (R + 1) pairs
     int *const CM = reinterpret_cast<int *>(VV + (CURV ? 2 * (W + 1) * (R + 1) : 0));   // columns, then rows: see below
     int *const RM = CM + 2 * (W + 1);
@@ -92,9 +96,9 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
         lox = perx ? E - e : max(E - e, -ix0); hix = perx ? E + w + e : min(E + w + e, ni - ix0);
         loy = pery ? E - e : max(E - e, -jy0); hiy = pery ? E + h + e : min(E + h + e, nj - jy0);
     };
-    // Per column (and row): [0] the grid column its cells are loaded from (-1: none), or the vertex
-    // column; [1] for ghost cells the position their values come from and their kind (resolve_index)
-    // in bits 16 and up. Divisions happen here once, not per position and phase: `recip` holds
+    // Per column (and row): [0] the grid column its cells are loaded from (-1: none, more than H cells
+    // outside the grid), or the vertex column; [1] the position its cells' values come from (its own but
+    // for ghost cells) and their kind (resolve_index) in bits 16 and up. Divisions happen here once, not per position and phase: `recip` holds
     // 2^32 / n + 1 for the width n of every rectangle that a phase covers.
     __shared__ unsigned recip[4 * STAGES + 2];
     if (tid < 4 * STAGES + 2) {
@@ -115,9 +119,9 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
         if (per) { src = v % n; src = src < 0 ? src + n : src; }
         else if (v < 0 || v >= n) {
             int kind;
-            from = resolve_index(v, n, col ? bcW : bcS, col ? bcE : bcN, kind) - o;
-            from = (from & 0xffff) | kind << 16;
-            src = -1;
+            src = resolve_index(v, n, col ? bcW : bcS, col ? bcE : bcN, kind);
+            from = ((src - o) & 0xffff) | kind << 16;
+            if (v < -H || v >= n + H) src = -1;
         }
         (col ? CM : RM)[2 * x] = src;
         (col ? CM : RM)[2 * x + 1] = from;
@@ -181,16 +185,16 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
         copies_commit();
     }
     if constexpr (WALLS) {
-        // (solid cells are never combined with periodic sides; ghost cells are flagged below)
         const unsigned mw = recip[4 * STAGES + 1];
         const bool mask = G.soff >= 0;
 #pragma unroll 4
         for (int at = tid; at < P; at += nt) {
             const int r = (int)__umulhi((unsigned)at, mw), c = at - r * W;
-            const int i = CM[2 * c], j = RM[2 * r];
+            const int i = CM[2 * c], j = RM[2 * r], kx = CM[2 * c + 1] >> 16, ky = RM[2 * r + 1] >> 16;
             uint8_t f = 0;
             const long long x = G.soff + (long long)j * ni + i;
-            if (mask && (i | j) >= 0 && TILE_OK(x, 1, n_solid)) f = __ldg(a.solid + x);
+            if (mask && (i | j) >= 0 && kx != 2 && ky != 2 && TILE_OK(x, 1, n_solid)) f = __ldg(a.solid + x) & 1;
+            if ((kx == 1 || ky == 1) && kx != 2) f |= 2;
             FL[at] = f;
         }
     }
@@ -209,48 +213,40 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
             st_cell(A2 + 4 * at, a2);
         }
     };
-    // A ghost cell (outside the grid in a direction that is not periodic) from its source cell.
-    auto ghost_cell = [&](int c, int r) {
-        const int at = r * W + c, cm = CM[2 * c + 1], rm = RM[2 * r + 1];
-        const int cs = cm & 0xffff, kx = cm >> 16, rs = rm & 0xffff, ky = rm >> 16;
-        WC<T> q;
-        if (kx == 2 || ky == 2) {
-            q.r = K.inflow[0]; q.u = K.inflow[1]; q.v = K.inflow[2]; q.p = K.inflow[3];
-        } else {
-            T raw[4];
-            ld_own(U + 4 * (rs * W + cs), raw);
-            prims(raw, q);
+    auto inflow = [&](WC<T> &q) { q.r = K.inflow[0]; q.u = K.inflow[1]; q.v = K.inflow[2]; q.p = K.inflow[3]; };
+    // Wall mirrors of the ghost cell at (c, r), whose values q are those of the cell at (cs, rs).
+    auto mirror_ghost = [&](WC<T> &q, int c, int r, int cs, int kx, int ky) {
+        const int i = ix0 + c, j = jy0 + r;
+        // (the boundary face's row clamped to the grid: corner ghost cells, whose velocities are
+        //  never used)
+        if (ky == 1 && kx != 2) {
+            T nx, ny, l;
+            geom_y(cs, (j < 0 ? 0 : nj) - jy0, nx, ny, l);
+            mirror_vel(q.u, q.v, nx, ny);
         }
-        if constexpr (WALLS) {
-            const int i = ix0 + c, j = jy0 + r;
-            uint8_t f = (kx == 2 || ky == 2) ? (uint8_t)0 : (uint8_t)(FL[rs * W + cs] & 1);
-            // (the boundary face's row clamped to the grid: corner ghost cells, whose velocities are
-            //  never used)
-            if (ky == 1 && kx != 2) {
-                T nx, ny, l;
-                geom_y(cs, (j < 0 ? 0 : nj) - jy0, nx, ny, l);
-                mirror_vel(q.u, q.v, nx, ny);
-            }
-            if (kx == 1) {
-                T nx, ny, l;
-                geom_x((i < 0 ? 0 : ni) - ix0, pery ? r : clampi(j, 0, nj - 1) - jy0, nx, ny, l);
-                mirror_vel(q.u, q.v, nx, ny);
-            }
-            if ((kx == 1 || ky == 1) && kx != 2) f |= 2;
-            FL[at] = f;
+        if (kx == 1) {
+            T nx, ny, l;
+            geom_x((i < 0 ? 0 : ni) - ix0, pery ? r : clampi(j, 0, nj - 1) - jy0, nx, ny, l);
+            mirror_vel(q.u, q.v, nx, ny);
         }
-        put_cell(at, q);
     };
     const T dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_value<T>(__ldg(a.rate_rd + g));
     const T rxy = K.dy / K.dx, cy = T(0.5) * K.dx * K.Vi;   // Cartesian residual weights
     copies_wait<0>();
-    // (each thread turns the cells that it copied itself into primitives: no barrier in between)
+    // (each thread turns the cells that it copied itself into primitives: no barrier in between, but for
+    //  the vertices that mirrors at curved walls need)
+    if constexpr (CURV && WALLS) __syncthreads();
     over(recip[4 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
         if ((CM[2 * c] | RM[2 * r]) >= 0) {
             T raw[4];
             WC<T> q;
             ld_own(U + 4 * (r * W + c), raw);
             prims(raw, q);
+            if (WALLS && edge) {
+                const int cm = CM[2 * c + 1], kx = cm >> 16, ky = RM[2 * r + 1] >> 16;
+                if (kx == 2 || ky == 2) inflow(q);
+                if (kx | ky) mirror_ghost(q, c, r, cm & 0xffff, kx, ky);
+            }
             put_cell(r * W + c, q);
         }
     });
@@ -266,26 +262,41 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
         const T beta = STAGES == 1 ? a.beta : (s == 0 ? T(1) : (s == 1 ? T(0.25) : T(2.0 / 3.0)));
         const bool last = s == STAGES - 1;
 
-        // ---- ghost cells, where the cells that the stage reads (H beyond its margin) leave the grid on
-        //      a side that is not periodic: columns west and east (all rows), then rows south and north
-        const int gW = perx ? 0 : max(0, -ix0 - (lox - H)), gE = perx ? 0 : max(0, hix + H - (ni - ix0));
-        const int gS = pery ? 0 : max(0, -jy0 - (loy - H)), gN = pery ? 0 : max(0, hiy + H - (nj - jy0));
-        if (gW | gE | gS | gN) {   // (0 to H columns or rows each)
-            const int rows = hiy - loy + 2 * H, cl = lox - H + gW, cols = hix + H - gE - cl;
+        // The ghost cells that a stage reads: H beyond its margin, where that leaves the grid on a side that is
+        // not periodic; columns west and east (all rows), then rows south and north (0 to H of each).
+        auto ghosts = [&](int s, int from, auto &&body) {
+            int lx, hx, ly, hy;
+            margin(s, lx, hx, ly, hy);
+            const int gW = perx ? 0 : max(0, -ix0 - (lx - H)), gE = perx ? 0 : max(0, hx + H - (ni - ix0));
+            const int gS = pery ? 0 : max(0, -jy0 - (ly - H)), gN = pery ? 0 : max(0, hy + H - (nj - jy0));
+            const int rows = hy - ly + 2 * H, cl = lx - H + gW, cols = hx + H - gE - cl;
             const int nW = gW * rows, nE = nW + gE * rows, nS = nE + gS * cols, nN = nS + gN * cols;
-            for (int k = tid; k < nN; k += nt) {
+#pragma unroll 1
+            for (int k = from; k < nN; k += nt) {
                 int c, r;
                 if (k < nE) {
                     const int q = k < nW ? k : k - nW, two = (k < nW ? gW : gE) - 1;
-                    c = (k < nW ? lox - H : hix + H - gE) + (two ? q & 1 : 0);
-                    r = loy - H + (q >> two);
+                    c = (k < nW ? lx - H : hx + H - gE) + (two ? q & 1 : 0);
+                    r = ly - H + (q >> two);
                 } else {
                     const int q = k < nS ? k - nE : k - nS, d = q >= cols;
                     c = cl + q - (d ? cols : 0);
-                    r = (k < nS ? loy - H : hiy + H - gN) + d;
+                    r = (k < nS ? ly - H : hy + H - gN) + d;
                 }
-                ghost_cell(c, r);
+                body(c, r, CM[2 * c + 1], RM[2 * r + 1]);
             }
+        };
+        if (!WALLS && edge) {
+            ghosts(s, tid, [&](int c, int r, int cm, int rm) {
+                WC<T> q;
+                if (cm >> 16 == 2 || rm >> 16 == 2) inflow(q);
+                else {
+                    T raw[4];
+                    ld_own(U + 4 * ((rm & 0xffff) * W + (cm & 0xffff)), raw);
+                    prims(raw, q);
+                }
+                put_cell(r * W + c, q);
+            });
             __syncthreads();
         }
 
@@ -512,25 +523,33 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
         }
         __syncthreads();
 
-        // ---- cells: R = D sc, then the stage combination
-        over(m[3], lox, hix, loy, hiy, [&](int c, int r) {
+        // ---- cells: R = D sc, then the stage combination. With walls also the ghost cells of the next stage,
+        //      each from another update of its source cell: they need neither a phase of their own nor a
+        //      barrier (0.4 us a stage on a curved duct), for which U^(k) must not be overwritten meanwhile.
+        //      (Without walls ghost cells are cheap, and one buffer for U^(k) is 2 % faster.)
+        T *const cur = !WALLS || s == 0 ? U : V + 4 * P * (s - 1), *const nxt = WALLS ? V + 4 * P * s : U;
+        // (c, r): the cell; (gc, gr): where its values go, of kind (kx, ky)
+        auto update = [&](auto is_ghost, int c, int r, int gc, int gr, int kx, int ky) {
+            constexpr bool ghost = decltype(is_ghost)::value;
             const int at = r * W + c;
             T fw[4], fe[4], fs[4], fn[4], uk[4], un[4], out[4];
             ld_own(FX + 4 * at, fw);
             ld_own(FX + 4 * (at + 1), fe);
             ld_own(FY + 4 * at, fs);
             ld_own(FY + 4 * (at + W), fn);
-            ld_own(U + 4 * at, uk);
-            const bool own = c >= E && c < E + w && r >= E && r < E + h;   // (others also update halo cells)
+            ld_own(cur + 4 * at, uk);
+            const bool own = !ghost && c >= E && c < E + w && r >= E && r < E + h;   // (others also update halo cells)
             const long long x = G.off + 4 * ((long long)(jy0 + r) * pitch + (ix0 + c));
             if (STAGES == 1) {
                 if (alpha != T(0)) ld_own(a.un + x, un);
                 else for (int k = 0; k < 4; ++k) un[k] = uk[k];
+            } else if (WALLS) {
+                ld_own(U + 4 * at, un);
             } else if (s == 0) {
                 for (int k = 0; k < 4; ++k) un[k] = uk[k];
-                st_cell(Un + 4 * at, uk);
+                st_cell(V + 4 * at, uk);
             } else {
-                ld_own(Un + 4 * at, un);
+                ld_own(V + 4 * at, un);
             }
             bool solid = false;
             if constexpr (WALLS) solid = FL[at] & 1;
@@ -550,10 +569,11 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                 out[k] = vfma(alpha, un[k], beta * upd);
             }
             if (!last) {
-                st_cell(U + 4 * at, out);
+                if (!ghost) st_cell(nxt + 4 * at, out);
                 WC<T> q;
                 prims(out, q);
-                put_cell(at, q);
+                if constexpr (WALLS && ghost) mirror_ghost(q, gc, gr, c, kx, ky);
+                put_cell(gr * W + gc, q);
             } else if (TILE_OK(x, 4, n_state)) {
                 st_cell(a.dst + x, out);
             }
@@ -577,7 +597,13 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
                     }
                 }
             }
-        });
+        };
+        over(m[3], lox, hix, loy, hiy, [&](int c, int r) { update(Flag<false>(), c, r, c, r, 0, 0); });
+        if (WALLS && !last && edge)   // (the last threads are idle in the cells' last round)
+            ghosts(s + 1, nt - 1 - tid, [&](int c, int r, int cm, int rm) {
+                const int kx = cm >> 16, ky = rm >> 16;
+                if (kx != 2 && ky != 2) update(Flag<true>(), cm & 0xffff, rm & 0xffff, c, r, kx, ky);   // (INFLOW: set at the start)
+            });
         if (!last) __syncthreads();
     }
     if (a.want_rate) {
