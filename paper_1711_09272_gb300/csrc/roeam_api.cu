@@ -120,7 +120,7 @@ struct roeam_grid {
     // Tile kernels (see setup_tile_kernel): whether rk_step uses them, their work list and launch
     bool tile_on = false;
     int4 *d_rects = nullptr;
-    int nrects = 0, rect_threads = 0;
+    int nrects = 0, rect_nx = 0, rect_ny = 0, rect_threads = 0;
     size_t rect_smem = 0;
     unsigned *status = nullptr;
     unsigned *work = nullptr;                            // dynamic unit-scheduling counters (2)
@@ -357,14 +357,16 @@ roeam_status setup_tile_kernel(roeam_grid *g)
         const int nx = (G.ni + bw - 1) / bw, ny = (G.nj + bh - 1) / bh;
         for (int y = 0; y < ny; ++y)
             for (int x = 0; x < nx; ++x) {
-                const int x0 = (int)((long long)x * G.ni / nx), x1 = (int)((long long)(x + 1) * G.ni / nx);
-                const int y0 = (int)((long long)y * G.nj / ny), y1 = (int)((long long)(y + 1) * G.nj / ny);
+                const int x0 = tile_edge(x, G.ni, nx), x1 = tile_edge(x + 1, G.ni, nx);
+                const int y0 = tile_edge(y, G.nj, ny), y1 = tile_edge(y + 1, G.nj, ny);
                 rects.push_back(make_int4(k, x0, y0, (x1 - x0) | ((y1 - y0) << 16)));
                 mw = std::max(mw, x1 - x0);
                 mh = std::max(mh, y1 - y0);
             }
     }
     g->nrects = (int)rects.size();
+    g->rect_nx = (g->hg[0].ni + bw - 1) / bw;
+    g->rect_ny = (g->hg[0].nj + bh - 1) / bh;
     g->rect_smem = tile_bytes<T>(mw + 2 * E, mh + 2 * E, g->muscl, g->curv, walls, stages);
     const int positions = (mw + 2 * E) * (mh + 2 * E);
     g->rect_threads = std::min(tile_threads<T>(), std::max(128, (positions + 31) / 32 * 32));
@@ -475,29 +477,33 @@ roeam_status upload_geometry(roeam_grid *g, const roeam_grid_desc *d)
 }
 
 template <typename T>
+GridCoef<T> make_coef(const GridDev &G)
+{
+    GridCoef<T> c;
+    c.g = T(G.gamma);
+    c.gm1 = T(G.gamma - 1.0);
+    c.gm1i = T(1.0 / (G.gamma - 1.0));
+    c.hgm1 = T(0.5 * (G.gamma - 1.0));
+    // (the classical Roe flux does not use M_ref; its time-step rule is |U| + c: theta = 1)
+    c.mr2 = T(G.scheme == ROEAM_SCHEME_ROE ? 1.0 : G.m_ref * G.m_ref);
+    c.rr_thr = T(1e-5 * G.u_ref);
+    c.eps2 = T(G.eps2);
+    c.dx = T(G.dx);
+    c.dy = T(G.dy);
+    c.V = T(G.dx * G.dy);
+    c.Vi = T(1.0 / (G.dx * G.dy));
+    c.idx = T(1.0 / G.dx);
+    c.idy = T(1.0 / G.dy);
+    for (int s = 0; s < 4; ++s) c.inflow[s] = T(G.inflow[s]);
+    c.harten = T(G.harten);
+    return c;
+}
+
+template <typename T>
 roeam_status upload_coef(roeam_grid *g)
 {
     std::vector<GridCoef<T>> h(g->count);
-    for (int k = 0; k < g->count; ++k) {
-        const GridDev &G = g->hg[k];
-        GridCoef<T> &c = h[k];
-        c.g = T(G.gamma);
-        c.gm1 = T(G.gamma - 1.0);
-        c.gm1i = T(1.0 / (G.gamma - 1.0));
-        c.hgm1 = T(0.5 * (G.gamma - 1.0));
-        // (the classical Roe flux does not use M_ref; its time-step rule is |U| + c: theta = 1)
-        c.mr2 = T(G.scheme == ROEAM_SCHEME_ROE ? 1.0 : G.m_ref * G.m_ref);
-        c.rr_thr = T(1e-5 * G.u_ref);
-        c.eps2 = T(G.eps2);
-        c.dx = T(G.dx);
-        c.dy = T(G.dy);
-        c.V = T(G.dx * G.dy);
-        c.Vi = T(1.0 / (G.dx * G.dy));
-        c.idx = T(1.0 / G.dx);
-        c.idy = T(1.0 / G.dy);
-        for (int s = 0; s < 4; ++s) c.inflow[s] = T(G.inflow[s]);
-        c.harten = T(G.harten);
-    }
+    for (int k = 0; k < g->count; ++k) h[k] = make_coef<T>(g->hg[k]);
     CUDA_TRY(cudaMalloc(&g->d_coef, sizeof(GridCoef<T>) * g->count));
     CUDA_TRY(cudaMemcpy(g->d_coef, h.data(), sizeof(GridCoef<T>) * g->count, cudaMemcpyHostToDevice));
     return ROEAM_OK;
@@ -545,6 +551,15 @@ roeam_status launch_tile_step(roeam_grid *g, cudaStream_t s, long long step, dou
     a.coef = (const GridCoef<T> *)g->d_coef;
     a.tiles = g->d_rects;
     a.ngrids = g->count;
+    if (g->count == 1) {
+        a.g0 = g->hg[0];
+        a.c0 = make_coef<T>(g->hg[0]);
+        a.nx = g->rect_nx;
+        a.wide = a.g0.ni / g->rect_nx;
+        a.wider = a.g0.ni % g->rect_nx;
+        a.high = a.g0.nj / g->rect_ny;
+        a.higher = a.g0.nj % g->rect_ny;
+    }
     a.vdx = (const T *)g->vdx;
     a.vdy = (const T *)g->vdy;
     a.solid = g->solid;

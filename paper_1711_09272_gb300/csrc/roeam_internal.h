@@ -168,6 +168,9 @@ constexpr size_t TILE_SMEM_MAX = 226 * 1024;   // dynamic shared memory a tile m
 
 template <typename T>
 struct TileArgs {
+    GridDev g0;             // the only grid's descriptor and constants, and its rectangles: nx a row,
+    GridCoef<T> c0;         // `wide` x `high` cells, the first `wider` columns and `higher` rows of them one more
+    int nx, wide, wider, high, higher;
     const GridDev *grids;
     const GridCoef<T> *coef;
     const int4 *tiles;      // (grid, first column, first row, width | height << 16)
@@ -186,6 +189,9 @@ struct TileArgs {
     long long n_state, n_vert, n_solid;   // buffer sizes, read by the bounds checks of debug builds
 #endif
 };
+
+// First column of rectangle x of n over ni columns (rows likewise).
+inline int tile_edge(int x, int ni, int n) { return x * (ni / n) + (x < ni % n ? x : ni % n); }
 
 // Shared memory of a tile of W x R positions (the rectangle and its halo): quads of T per position
 // (U, primitives, two fluxes, derived quantities or two slopes, U^n or U^(1) and U^(2)), the Eq. 97 ratios (one row

@@ -49,10 +49,24 @@ template <typename T> __device__ __forceinline__ void copy_value(T *dst, const T
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"((int)sizeof(T)) : "memory");
 }
 
+template <bool ONE, typename T> __device__ __forceinline__ const GridDev &tile_grid(const TileArgs<T> &a, int g)
+{
+    if constexpr (ONE) return a.g0;
+    else return a.grids[g];
+}
+template <bool ONE, typename T> __device__ __forceinline__ decltype(auto) tile_coef(const TileArgs<T> &a, int g)
+{
+    if constexpr (ONE) return (a.c0);
+    else return GridCoef<T>(a.coef[g]);
+}
 template <bool B> struct Flag { static constexpr bool value = B; };
 
-template <typename T, bool MUSCL, bool CURV, bool WALLS, int STAGES>
-__global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<T> a)
+// ONE: a single grid. Its descriptor, its constants (FP32) and its rectangles are kernel arguments, so that
+// the kernel does not begin with a chain of loads and holds none of them in registers: 256^2 Gresho
+// vortex, 50 steps, 607 -> 577 us, 800 x 20 duct, 64 steps, 479 -> 462. (FP64 constants as operands from
+// the constant bank: 64^2 vortex 688 -> 691, from registers 687.)
+template <typename T, bool MUSCL, bool CURV, bool WALLS, int STAGES, bool ONE>
+__global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_constant__ TileArgs<T> a)
 {
     constexpr int H = MUSCL ? 2 : 1;
     constexpr int E = H * STAGES;
@@ -61,11 +75,18 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const TileArgs<
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T red[tile_threads<T>() / 32];
 
-    const int4 tile = __ldg(a.tiles + blockIdx.x);
-    const int g = a.ngrids == 1 ? 0 : tile.x;   // (one grid: its descriptor is loaded beside the tile's)
+    int4 tile;
+    if constexpr (ONE) {
+        const int y = (int)blockIdx.x / a.nx, x = (int)blockIdx.x - y * a.nx;
+        tile = make_int4(0, x * a.wide + min(x, a.wider), y * a.high + min(y, a.higher),
+                         (a.wide + (x < a.wider)) | (a.high + (y < a.higher)) << 16);
+    } else {
+        tile = __ldg(a.tiles + blockIdx.x);
+    }
+    const int g = tile.x;
     const int x0 = tile.y, y0 = tile.z, w = tile.w & 0xffff, h = tile.w >> 16;
-    const GridDev &G = a.grids[g];
-    const GridCoef<T> K = a.coef[g];
+    const GridDev &G = tile_grid<ONE>(a, g);
+    const GridCoef<T> &K = tile_coef<ONE && sizeof(T) == 4>(a, g);
     const int ni = G.ni, nj = G.nj, pitch = G.pitch;
     const int bcW = G.bc[0], bcE = G.bc[1], bcS = G.bc[2], bcN = G.bc[3];
     const bool perx = bcW == BC_PERIODIC, pery = bcS == BC_PERIODIC;
@@ -622,12 +643,15 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS> struct TileVariant {
     static constexpr int STAGES = tile_stages<T>();
     static cudaError_t launch(const TileArgs<T> &a, int ntiles, int threads, size_t smem, cudaStream_t s)
     {
-        return launch_pdl(tile_kernel<T, MUSCL, CURV, WALLS, STAGES>, dim3((unsigned)ntiles), dim3((unsigned)threads), smem, s, a);
+        return launch_pdl(a.ngrids == 1 ? tile_kernel<T, MUSCL, CURV, WALLS, STAGES, true> : tile_kernel<T, MUSCL, CURV, WALLS, STAGES, false>,
+                          dim3((unsigned)ntiles), dim3((unsigned)threads), smem, s, a);
     }
     static cudaError_t prepare(size_t smem)
     {
-        return cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES, true>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES, false>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
 };
 
