@@ -108,29 +108,32 @@ roeam_status validate3(int count, const roeam3_grid_desc *d)
 }
 
 template <typename T>
-roeam_status upload_coef3(roeam3_grid *g, const roeam3_grid_desc *d)
+GridCoef3<T> make_coef3(const GridDev3 &q)
+{
+    GridCoef3<T> c;
+    c.g = T(q.gamma);
+    c.gm1 = T(q.gamma - 1.0);
+    c.gm1i = T(1.0 / (q.gamma - 1.0));
+    c.hgm1 = T(0.5 * (q.gamma - 1.0));
+    c.mr2 = T(q.m_ref * q.m_ref);
+    c.rr_thr = T(1e-5 * q.u_ref);
+    c.eps2 = T(q.eps2);
+    c.ax = T(q.dy * q.dz);
+    c.ay = T(q.dx * q.dz);
+    c.az = T(q.dx * q.dy);
+    c.Vi = T(1.0 / (q.dx * q.dy * q.dz));
+    c.idx = T(1.0 / q.dx);
+    c.idy = T(1.0 / q.dy);
+    c.idz = T(1.0 / q.dz);
+    for (int v = 0; v < MAX_VARS3; ++v) c.inflow[v] = T(q.inflow[v]);
+    return c;
+}
+
+template <typename T>
+roeam_status upload_coef3(roeam3_grid *g)
 {
     std::vector<GridCoef3<T>> h(g->count);
-    for (int k = 0; k < g->count; ++k) {
-        const roeam3_grid_desc &q = d[k];
-        GridCoef3<T> &c = h[k];
-        const double gm = q.p.gamma;
-        c.g = T(gm);
-        c.gm1 = T(gm - 1.0);
-        c.gm1i = T(1.0 / (gm - 1.0));
-        c.hgm1 = T(0.5 * (gm - 1.0));
-        c.mr2 = T(q.p.m_ref * q.p.m_ref);
-        c.rr_thr = T(1e-5 * q.p.u_ref);
-        c.eps2 = T(q.p.eps2);
-        c.ax = T(q.dy * q.dz);
-        c.ay = T(q.dx * q.dz);
-        c.az = T(q.dx * q.dy);
-        c.Vi = T(1.0 / (q.dx * q.dy * q.dz));
-        c.idx = T(1.0 / q.dx);
-        c.idy = T(1.0 / q.dy);
-        c.idz = T(1.0 / q.dz);
-        for (int v = 0; v < MAX_VARS3; ++v) c.inflow[v] = T(q.inflow[v]);
-    }
+    for (int k = 0; k < g->count; ++k) h[k] = make_coef3<T>(g->hg[k]);
     CUDA_TRY3(cudaMalloc(&g->d_coef, sizeof(GridCoef3<T>) * g->count));
     CUDA_TRY3(cudaMemcpy(g->d_coef, h.data(), sizeof(GridCoef3<T>) * g->count, cudaMemcpyHostToDevice));
     return ROEAM_OK;
@@ -216,6 +219,10 @@ StageArgs3<T> base_args3(roeam3_grid *g)
     a.units = g->d_units;
     a.ngrids = g->count;
     a.nunits = g->nunits;
+    if (g->count == 1) {
+        a.g0 = g->hg[0];
+        a.c0 = make_coef3<T>(g->hg[0]);
+    }
     a.status = g->status;
     return a;
 }
@@ -393,7 +400,7 @@ roeam_status roeam3_create_grid(int count, const roeam3_grid_desc *descs, int de
     CREATE3_TRY(cudaMallocHost(&g->h_status, sizeof(unsigned)));
     CREATE3_TRY(cudaMallocHost(&g->h_rate, sizeof(unsigned long long) * count));
 #undef CREATE3_TRY
-    st = g->precision == 32 ? upload_coef3<float>(g, descs) : upload_coef3<double>(g, descs);
+    st = g->precision == 32 ? upload_coef3<float>(g) : upload_coef3<double>(g);
     if (st != ROEAM_OK) return cleanup(st);
     st = g->precision == 32 ? setup_units3<float>(g, num_sms) : setup_units3<double>(g, num_sms);
     if (st != ROEAM_OK) return cleanup(st);

@@ -71,6 +71,8 @@ struct StageArgs3 {
     unsigned long long *rate_wr, *rate_zero;
     T cfl_t, dt_fixed_t;
     unsigned *status;
+    GridDev3 g0;             // the only grid's descriptor and constants
+    GridCoef3<T> c0;
 };
 
 template <typename T>

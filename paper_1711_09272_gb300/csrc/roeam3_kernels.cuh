@@ -529,7 +529,7 @@ template <int NS> struct March3 {
     static constexpr int NV = 5 + NS, TW = tail3(NV), NC = 9 + NS, FIELDS = NC + 3 + NV, TH = threads3<float>();
 };
 
-template <int NS> __device__ __forceinline__ void stage3_march(const StageArgs3<float> &a)
+template <int NS, bool ONE> __device__ __forceinline__ void stage3_march(const StageArgs3<float> &a)
 {
     using M = March3<NS>;
     constexpr int NV = M::NV, TW = M::TW, NC = M::NC, TH = M::TH, ROWS = TH / 32;
@@ -547,8 +547,8 @@ template <int NS> __device__ __forceinline__ void stage3_march(const StageArgs3<
     const int g = a.ngrids == 1 ? 0 : unit.x;
     const int x0 = unit.y & 0xffff, w = unit.y >> 16, y0 = unit.z & 0xffff, h = unit.z >> 16;
     const int k0 = unit.w & 0xffff, k1 = (int)((unsigned)unit.w >> 16);
-    const GridDev3 &G = a.grids[g];
-    const GridCoef3<float> K = a.coef[g];
+    const GridDev3 &G = ONE ? a.g0 : a.grids[g];
+    const GridCoef3<float> K = ONE ? a.c0 : a.coef[g];
     const int nk = G.nk, pitch = G.pitch, bcB = G.bc[4], bcT = G.bc[5];
     int kx, ky;
     const int isrc = resolve_index(x0 - 1 + lane, G.ni, G.bc[0], G.bc[1], kx);
@@ -761,8 +761,16 @@ template <int NS> __device__ __forceinline__ void stage3_march(const StageArgs3<
 template <typename T, int NS>
 __global__ void __launch_bounds__(threads3<T>(), 1) stage3_kernel(const StageArgs3<T> a)
 {
-    if constexpr (sizeof(T) == 4) stage3_march<NS>(a);
+    if constexpr (sizeof(T) == 4) stage3_march<NS, false>(a);
     else stage3_phases<T, NS>(a);
+}
+// FP32 with three scalars, a single grid: its descriptor and constants are kernel arguments, not registers,
+// of which this kernel has none to spare (192^3: 1072 -> 920 us a step). With fewer scalars the
+// constants as operands change nothing or lose 0.7 %, nor does FP64 gain.
+template <int NS>
+__global__ void __launch_bounds__(threads3<float>(), 1) stage3_single(const __grid_constant__ StageArgs3<float> a)
+{
+    stage3_march<NS, true>(a);
 }
 
 // Host float64 layout [nv][nk][nj][ni] per grid <-> the state's quads and tails, blockIdx.y = grid; as
@@ -871,12 +879,19 @@ __global__ void __launch_bounds__(256) totals3_kernel(const GridDev3 *grids, int
 
 // ------------------------------------------------------------------ launchers
 template <typename T, int NS> struct Stage3Variant {
+    static constexpr bool SINGLE = sizeof(T) == 4 && NS == 3;
     static cudaError_t launch(const StageArgs3<T> &a, int threads, size_t smem, cudaStream_t s)
     {
+        if constexpr (SINGLE)
+            if (a.ngrids == 1) return launch_pdl(stage3_single<NS>, dim3((unsigned)a.nunits), dim3((unsigned)threads), smem, s, a);
         return launch_pdl(stage3_kernel<T, NS>, dim3((unsigned)a.nunits), dim3((unsigned)threads), smem, s, a);
     }
     static cudaError_t prepare()
     {
+        if constexpr (SINGLE) {
+            const cudaError_t e = cudaFuncSetAttribute(stage3_single<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX);
+            if (e != cudaSuccess) return e;
+        }
         return cudaFuncSetAttribute(stage3_kernel<T, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX);
     }
     static cudaError_t pack(dim3 grid, const GridDev3 *grids, const GridCoef3<T> *coef, int g_lo, const double *packed,
