@@ -281,7 +281,7 @@ roeam_status roeam_flux_residual_noalloc(roeam_grid *g, int grid_idx, double *re
  * with: 10. Shapes 0-4 cut each grid into warp strips of 32 lanes and segments of 32, 64, 16,
  * 128 and 256 rows and let warps claim units dynamically in the order of the unit table
  * (tallest first); shapes 5-9 are the same heights with a static round robin of units over
- * warps. (Kernels that do not claim units dynamically treat 0-4 as 5-9; a batch too small to
+ * warps. (A batch too small to
  * give every resident warp a unit halves the height, down to 4 rows, and on to 2 rows while the
  * units still fit one round of the resident warps.) Results are bit-identical across shapes. */
 int roeam_tile_config_count(void);

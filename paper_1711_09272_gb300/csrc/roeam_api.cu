@@ -278,7 +278,7 @@ roeam_status setup_tiles(roeam_grid *g, int cfg)
     CUDA_TRY(cudaStreamSynchronize(g->stream));
     g->nblocks = std::max(1, occ * g->num_sms);
     g->eff_ty = ty;
-    g->eff_dyn = tc.dyn && stage_dynamic(g->muscl, g->curv);
+    g->eff_dyn = tc.dyn;
     for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);
     g->graphs.clear();
     return ROEAM_OK;

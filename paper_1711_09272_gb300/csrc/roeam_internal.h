@@ -108,7 +108,7 @@ constexpr int stage_min_blocks()
 {
     return (sizeof(T) != 4 || ABL) ? 1 : (!CURV ? STAGE_MIN_BLOCKS_CART : STAGE_MIN_BLOCKS_CURV);
 }
-// dyn: dynamic unit scheduling (the kernels that support it claim units from a counter after
+// dyn: dynamic unit scheduling (warps claim units from a counter after
 // their first; 0 = static round robin over the unit table).
 struct TileCfg { int tx, ty, nt, dyn; };
 constexpr int NUM_TILE_CFGS = 10;
@@ -116,9 +116,6 @@ constexpr TileCfg TILE_CFGS[NUM_TILE_CFGS] = {
     {32, 32, STAGE_THREADS, 1}, {32, 64, STAGE_THREADS, 1}, {32, 16, STAGE_THREADS, 1}, {32, 128, STAGE_THREADS, 1},
     {32, 256, STAGE_THREADS, 1}, {32, 32, STAGE_THREADS, 0}, {32, 64, STAGE_THREADS, 0}, {32, 16, STAGE_THREADS, 0},
     {32, 128, STAGE_THREADS, 0}, {32, 256, STAGE_THREADS, 0}};
-// Whether a stage-kernel family claims units dynamically when asked to (the reconstructing
-// curvilinear kernels keep the static round robin).
-__host__ __device__ constexpr bool stage_dynamic(int muscl, int curv) { return !(muscl && curv); }
 
 // Stage-kernel families: no walls anywhere in the batch; some WALL side or solid cells; some
 // grid uses an ablation variant of the flux (every face on the scalar path).

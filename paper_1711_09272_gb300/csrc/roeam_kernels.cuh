@@ -968,23 +968,23 @@ template <typename T> __device__ __forceinline__ WC<T> shdn_c(const WC<T> &c, in
     return o;
 }
 
-// Dynamic unit scheduling (StageArgs::work): the unit after u for this warp. DYN = false keeps
-// the static round robin (the reconstructing curvilinear kernels: their units are of equal size
-// on the grids they serve, and the claim's registers made them spill, -16 % on the warped step).
-template <bool DYN, typename T>
+// Dynamic unit scheduling (StageArgs::work): the unit after u for this warp. (Also where units are of
+// equal size: rows near walls take the slower scalar path. 4096^2 warped step 6478 -> 5906 us; it
+// cost this kernel 16 % while the claim's registers made it spill.)
+template <typename T>
 __device__ __forceinline__ int next_unit(const StageArgs<T> &a, int u, int nwarps, int lane)
 {
-    if (!DYN || !a.work) return u + nwarps;
+    if (!a.work) return u + nwarps;
     unsigned n = 0;
     if (lane == 0) n = atomicAdd(a.work, 1u);
     return a.tile_lo + nwarps + (int)__shfl_sync(0xffffffffu, n, 0);
 }
 // A warp that has run out of units counts itself done; the last one resets the counters (every
 // warp's final claim precedes its count, fenced).
-template <bool DYN, typename T>
+template <typename T>
 __device__ __forceinline__ void finish_units(const StageArgs<T> &a, int nwarps, int lane)
 {
-    if (!DYN || !a.work || lane != 0) return;
+    if (!a.work || lane != 0) return;
     __threadfence();
     if (atomicAdd(a.work + 1, 1u) == (unsigned)nwarps - 1u) {
         __threadfence();
@@ -1034,8 +1034,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
     // Each warp takes unit tile_lo + warp first, then (dynamic scheduling) the next unclaimed
     // one, in the order of the unit table (whole-batch launches: by decreasing height), so that
     // warps that drew short units take more of them and the launch ends evenly.
-    constexpr bool DYN = stage_dynamic(MUSCL, CURV);
-    for (int u = a.tile_lo + warp; u < a.tile_hi; u = next_unit<DYN>(a, u, nwarps, lane)) {
+    for (int u = a.tile_lo + warp; u < a.tile_hi; u = next_unit(a, u, nwarps, lane)) {
         const int4 unit = __ldg(a.units + u);   // (grid, first lane's column, j0, j1)
         const int g = unit.x;
         const int i = unit.y + lane;            // this lane's column
@@ -1415,7 +1414,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         }
     }
 
-    finish_units<DYN>(a, nwarps, lane);
+    finish_units(a, nwarps, lane);
 
     if (a.mode == MODE_NORM) {
         // Fixed-order block reduction of the FP64 partials: warp shuffles, then warp 0.
