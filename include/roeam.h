@@ -210,7 +210,7 @@ roeam_status roeam_edge_rows(roeam_grid *g, int grid_idx, int side, int stage, v
  * nj+1) of grid grid_idx, in the state that stage `stage` (0, 1, 2) reads, from src laid out
  * like roeam_edge_rows' output (host or device memory; ordered on the handle's stream and, for
  * host memory, complete on return, so the buffer may be reused at once). A grid
- * with an EXCHANGE side keeps these rows in its own state planes; they start at zero, so each
+ * with an EXCHANGE side keeps these rows in its own state; they start at zero, so each
  * must be set before the stage that reads it. */
 roeam_status roeam_set_halo(roeam_grid *g, int grid_idx, int side, int stage, const void *src);
 
@@ -283,7 +283,10 @@ roeam_status roeam_flux_residual_noalloc(roeam_grid *g, int grid_idx, double *re
  * (tallest first); shapes 5-9 are the same heights with a static round robin of units over
  * warps. (A batch too small to
  * give every resident warp a unit halves the height, down to 4 rows, and on to 2 rows while the
- * units still fit one round of the resident warps.) Results are bit-identical across shapes. */
+ * units still fit one round of the resident warps.) Results are bit-identical across shapes.
+ * Steps of FP64 handles and of FP32 handles of up to about a million cells run in another kernel
+ * (rectangles in shared memory), which has no such shapes: there a shape applies to the residual,
+ * its norms and roeam_rk_stage only. */
 int roeam_tile_config_count(void);
 
 /* Describes tile shape `cfg`: strip width tx, segment height ty (cells) and threads per CTA. */
@@ -303,7 +306,8 @@ roeam_status roeam_set_tile_config(roeam_grid *g, int cfg);
  * allocates a temporary copy of the state when it times. */
 roeam_status roeam_autotune(roeam_grid *g, double cfl, int steps, int *best_cfg, double *ms_per_step);
 
-/* Number of kernels this handle has launched (graph nodes count one each per replay). */
+/* Number of kernels this handle has launched (graph nodes count one each per replay). A step is
+ * three launches, or one for FP32 handles that run in rectangles (see above). */
 unsigned long long roeam_launch_count(const roeam_grid *g);
 
 /* Total cells of grid `grid_idx` (or of the batch with -1), or -1 on a bad argument. */

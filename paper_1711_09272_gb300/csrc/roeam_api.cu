@@ -983,7 +983,7 @@ namespace {
 // the copy-in stream, the computation (the pack, which also takes the time-step rate, nsteps
 // steps with the per-grid unit table, unpack) on the compute stream once the copy has landed, and the device-to-host copy on the
 // copy-out stream once the computation is done. Chunks touch disjoint ranges of the staging
-// buffer, the state planes, the rate slots and the host arrays, so the three streams never
+// buffer, the state, the rate slots and the host arrays, so the three streams never
 // wait for one another except through the chunk's own two events.
 template <typename T, typename H>
 roeam_status pipe_chunk(roeam_grid *g, int chunk, int lo, int hi, int nsteps, double cfl, double dt_fixed,

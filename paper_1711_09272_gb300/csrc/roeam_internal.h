@@ -138,7 +138,7 @@ struct Launchers {
     static cudaError_t stage(const StageArgs<T> &a, int muscl, int curv, int kind, int nblocks, cudaStream_t s);
     // Largest resident CTAs per SM of a stage-kernel variant (for persistent launches).
     static int stage_occupancy(int muscl, int curv, int kind);
-    // Packed float64 [4][nj][ni] per grid <-> pitched working-precision planes.
+    // Packed float64 [4][nj][ni] per grid <-> the state's pitched working-precision cells.
     // (pack reads grid g at packed + G.poff - p_shift; the host-side layout in float64 or float;
     //  with ro it also writes the packed state's rate into ro->rate[g], zeroed by the caller)
     static cudaError_t pack(const GridDev *grids, int g_lo, int g_hi, int max_cells, const double *packed, T *U,

@@ -8,7 +8,7 @@
 //     shared-memory ring of rows that asynchronous copies fill ahead of it, so every cell state
 //     is read from HBM once per stage (plus halo lanes and H+1 warm-up rows per segment);
 //   - neighbour states, detector ratios and fluxes move between lanes with warp shuffles;
-//     a lane reads only its own slots of the ring: no block barrier;
+//     of the ring a lane reads its own slots and, of the vertices, its neighbour's: no block barrier;
 //   - ghost cells come from the boundary conditions on the fly (periodic wrap, wall
 //     mirror, inflow state, zero-gradient outflow), so no separate boundary kernel runs;
 //   - the flux is evaluated in the face frame (normal velocity first), which makes the
@@ -848,8 +848,8 @@ template <typename T> __device__ __forceinline__ T *cell_at(T *base, int c) { re
 // Loading a cell is split in two: issue_group resolves row j (the column is resolved once per unit
 // into isrc / kx) and starts an asynchronous copy of the cell into this lane's slot of the warp's
 // shared-memory ring, RING_AHEAD rows before finish_cell turns the slot into primitives, derived
-// face quantities and flags. Each lane reads only what it copied itself, so waiting for its own
-// copies orders everything: no barrier. Resolution order: an INFLOW side in i gives the inflow
+// face quantities and flags. Each lane reads only cells it copied itself, so waiting for its own
+// copies orders everything: no barrier (a warp barrier for vertices, which the neighbour lane reads). Resolution order: an INFLOW side in i gives the inflow
 // state; otherwise an INFLOW side in j gives it (then mirrored by a WALL side in i); otherwise the
 // source cell, mirrored about the S/N boundary face by a WALL side in j, then about the W/E
 // boundary face by a WALL side in i. (An INFLOW ghost cell resolves to cell 0 of its direction and
@@ -858,7 +858,7 @@ template <typename T> __device__ __forceinline__ T *cell_at(T *base, int c) { re
 // The ring keeps the state rows from the one being finished (j - 1, whose U^(k) the stage epilogue
 // reads back) to the one on its way, and U^n of the rows to be combined: rows in flight hold no
 // registers, and a row has RING_AHEAD iterations to arrive. Measured: with the next row, U^n and
-// U^(k) loaded into registers as four planes per variable (start), the benchmark batch's kernel
+// U^(k) loaded into registers from four planes per variable, the benchmark batch's kernel
 // took 127 registers (16 warps per SM) and 15.2 warp instructions per cell in stage 2; the cell's
 // values together, a quad loaded into registers instead costs 12.4 but waits for each load where
 // the quad is copied (long-scoreboard stalls 0.7 -> 2.4 per instruction, 1 % slower); the ring 12.8
