@@ -295,7 +295,10 @@ roeam_status setup_tiles(roeam_grid *g, int cfg)
 // 512^2 35.6 / 39.5, 700^2 68 / 61; the estimates follow these within about 10 %, so the line lies
 // where both sides cost about the same.
 // FP64 (a stage per CTA): FP64 operations per face and cell, 76 cycles per warp on each of the four
-// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 168 / 277, 1024^2 2313 / 2696).
+// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 158 / 277, 1024^2 2228 / 2696). Counting
+// the rectangles that the even split makes, and full and started passes half and half, and giving the faces
+// a thread each: us per step, first order 100^2 48 -> 39, 128^2 58 -> 51, 256^2 162 -> 158, 800 x 20 58 -> 50;
+// reconstructed 128^2 82 -> 68, 256^2 224 -> 218, 331 x 97 124 -> 118 (32^2 31.8 -> 32.3, 1024^2 3232 -> 3250).
 // EXCHANGE sides (the caller sets ghost rows between stages) and the ablation kernels stay with the
 // strips.
 template <typename T>
@@ -332,11 +335,14 @@ roeam_status setup_tile_kernel(roeam_grid *g)
                     t += 2100 + std::ceil(pairs / 128) * (g->muscl ? 1030 : 750) * slow;
                 }
             } else {
-                const double faces = (double)(w + 1) * h + (double)w * (h + 1);
-                const double pos = (double)(w + 2 * H) * (h + 2 * H), own = (double)w * h;
-                t = 76 * ((g->muscl ? 185 : 133) * std::ceil(faces / 128) + (g->muscl ? 13 : 40) * std::ceil(pos / 128) +
-                          ((g->muscl ? 60 : 10) + 32) * std::ceil(own / 128));
-
+                // (a single grid's rectangles are as large as its even split makes them; a phase's last
+                //  pass counts half its lanes idle: warps spread over the sub-partitions unevenly then)
+                const int W = g->count == 1 ? (max_ni + (max_ni + w - 1) / w - 1) / ((max_ni + w - 1) / w) : w;
+                const int Y = g->count == 1 ? (max_nj + (max_nj + h - 1) / h - 1) / ((max_nj + h - 1) / h) : h;
+                const auto passes = [](double n) { return 0.5 * (std::ceil(n / 128) + n / 128); };
+                const double faces = (double)(W + 1) * Y + (double)W * (Y + 1);
+                t = 76 * ((g->muscl ? 175 : 129) * passes(faces) + (g->muscl ? 13 : 38) * passes((double)(W + 2 * H) * (Y + 2 * H)) +
+                          (g->muscl ? 52 : 16) * passes((double)(W + 2) * (Y + 2)) + 32 * passes((double)W * Y));
             }
             if (t >= best) continue;   // (at least one round)
             double tiles = 0;
@@ -368,8 +374,9 @@ roeam_status setup_tile_kernel(roeam_grid *g)
     g->rect_nx = (g->hg[0].ni + bw - 1) / bw;
     g->rect_ny = (g->hg[0].nj + bh - 1) / bh;
     g->rect_smem = tile_bytes<T>(mw + 2 * E, mh + 2 * E, g->muscl, g->curv, walls, stages);
-    const int positions = (mw + 2 * E) * (mh + 2 * E);
-    g->rect_threads = std::min(tile_threads<T>(), std::max(128, (positions + 31) / 32 * 32));
+    // a thread per position and, in FP64 (whose faces are a list of single ones), per face
+    const int positions = (mw + 2 * E) * (mh + 2 * E), items = stages == 3 ? positions : std::max(positions, 2 * mw * mh + mw + mh);
+    g->rect_threads = std::min(tile_threads<T>(), std::max(128, (items + 31) / 32 * 32));
     // One CTA per SM where that holds them all: with room for a second, the next launch's CTAs (which
     // come early, and wait) pair up on the SMs that are idle now (64^2 FP64 vortex, 20 steps: 855 us,
     // 682 us with the room taken).
