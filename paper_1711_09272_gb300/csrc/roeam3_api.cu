@@ -143,6 +143,9 @@ roeam_status upload_coef3(roeam3_grid *g)
 // FP32 takes 30 x 14 columns; (w, h) in FP64 and the number of segments minimise an estimate of a
 // launch's cycles, units going over the SMs in rounds: planes (a segment costs about one more) times a
 // plane's cycles, which in FP64 are its FP64 operations on an SM's four pipes and three barriers.
+// (Counting the rectangles that the even split makes, full and started passes half and half, and odd widths:
+// FP64 us a step, two scalars, 64^3 1300 -> 1252, 128^3 9526 -> 9294, 33^3 306 -> 258, 40^3 411 -> 380,
+// 60 x 180 x 34 1857 -> 1609, 500 x 4 x 4 158 -> 132; 95 x 63 x 127 3750 -> 3853.)
 // FP64 threads: one per face of a plane up to 256, also where there are fewer positions than that: two warps
 // per scheduler hide each other's latency (32^3: 398 us a step with a thread per position, 241 with 256;
 // 384 threads: 64^3 1348 us against 1332, 16^3 126 against 103, 95 x 63 x 127 3519 against 3852).
@@ -175,13 +178,17 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
     };
     if (f32) consider(MARCH3_X, MARCH3_Y, 5000, 6000, 1.0);
     else
-        for (int w = 64; w >= 2; w -= 2)
+        for (int w = 64; w >= 1; --w)
             for (int h = 2; h <= 64; ++h) {
                 if (w > max_ni + 1 || h > max_nj + 1 || bytes3<T>(w, h, g->nv) == 0) continue;
-                const double faces = (double)(w + 1) * h + (double)w * (h + 1) + (double)w * h;
-                const double positions = (double)(w + 2) * (h + 2);
-                consider(w, h, 2500 + 76 * (std::ceil(faces / 128) * (148 + 9 * g->nscal) +
-                                            std::ceil(positions / 128) * (75 + 7 * g->nv)), 4000, 1.3);
+                // (a single grid's rectangles are as large as its even split makes them; a phase's last
+                //  pass counts half its lanes idle)
+                const int W = g->count == 1 ? (max_ni + (max_ni + w - 1) / w - 1) / ((max_ni + w - 1) / w) : w;
+                const int Y = g->count == 1 ? (max_nj + (max_nj + h - 1) / h - 1) / ((max_nj + h - 1) / h) : h;
+                const auto passes = [](double n) { return 0.5 * (std::ceil(n / 128) + n / 128); };
+                const double faces = (double)(W + 1) * Y + (double)W * (Y + 1) + (double)W * Y;
+                const double positions = (double)(W + 2) * (Y + 2);
+                consider(w, h, 2500 + 76 * (passes(faces) * (148 + 9 * g->nscal) + passes(positions) * (75 + 7 * g->nv)), 4000, 1.3);
             }
     if (bw == 0) return fail3(ROEAM_E_ARG, "no work unit fits");
     std::vector<int4> units;
