@@ -163,6 +163,12 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
     double best = 1e300;
     int bw = 0, bh = 0, bn = 1;
     auto consider = [&](int w, int h, double plane, double segment, double planes_more) {
+        double planes = 0;   // of all rectangles: their cycles over the SMs bound the cost from below
+        for (int q = 0; q < g->count; q += every) {
+            const GridDev3 &G = g->hg[q];
+            planes += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * G.nk;
+        }
+        if (planes * plane / num_sms >= best) return;
         for (int n = 1; n <= std::min(max_nk, 96); ++n) {
             double units = 0;
             int zs = 0;
