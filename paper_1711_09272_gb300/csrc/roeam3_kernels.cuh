@@ -225,7 +225,7 @@ template <int N, typename T> __device__ __forceinline__ void copy_tail(unsigned 
 // thread its own positions), ratios of plane k + 1, fluxes through the west and south faces of plane k
 // and the face above it, one list for all threads. 720 FP64 operations per cell where the marching
 // layout of FP32 took 1700 (8-row tiles, halo rows, segments of 4 planes): 64^3 with two scalars
-// 3306 -> 1332 us a step, 128^3 16.9 -> 9.8 ms.
+// 3306 -> 1252 us a step, 128^3 16.9 -> 9.3 ms.
 template <typename T, int NS> __device__ __forceinline__ void stage3_phases(const StageArgs3<T> &a)
 {
     // Everything of one position lies in one record of shared memory, so that a thread addresses a cell
