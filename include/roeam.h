@@ -285,8 +285,8 @@ roeam_status roeam_flux_residual_noalloc(roeam_grid *g, int grid_idx, double *re
  * give every resident warp a unit halves the height, down to 4 rows, and on to 2 rows while the
  * units still fit one round of the resident warps.) Results are bit-identical across shapes.
  * Steps of FP64 handles and of FP32 handles of up to about a million cells run in another kernel
- * (rectangles in shared memory), which has no such shapes: there a shape applies to the residual,
- * its norms and roeam_rk_stage only. */
+ * (rectangles in shared memory), which has no such shapes (FP64 residuals and norms, too): there a
+ * shape applies to roeam_rk_stage and, in FP32, to the residual and its norms. */
 int roeam_tile_config_count(void);
 
 /* Describes tile shape `cfg`: strip width tx, segment height ty (cells) and threads per CTA. */

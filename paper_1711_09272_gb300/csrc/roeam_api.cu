@@ -120,6 +120,7 @@ struct roeam_grid {
     // Tile kernels (see setup_tile_kernel): whether rk_step uses them, their work list and launch
     bool tile_on = false;
     int4 *d_rects = nullptr;
+    std::vector<int> rect_base;           // first rectangle of each grid
     int nrects = 0, rect_nx = 0, rect_ny = 0, rect_threads = 0;
     size_t rect_smem = 0;
     unsigned *status = nullptr;
@@ -290,10 +291,10 @@ roeam_status setup_tiles(roeam_grid *g, int cfg)
 // (w, h) minimises an estimate of a step's cycles in which CTAs go over the SMs in rounds.
 // FP32 (a whole step per CTA): per stage a latency and the passes its face pairs take over an SM's
 // 128 lanes. Tiles are taken where that beats the strips' three launches of about 6 us each plus
-// their arithmetic. Measured, us per step, tiles / strips: periodic first order 128^2 6.3 / 16.8,
-// 256^2 9.9 / 20.1, 400^2 15.8 / 27.5, 700^2 40.9 / 45.8, 900^2 69 / 52; van Leer 256^2 12.9 / 24.5,
-// 512^2 35.6 / 39.5, 700^2 68 / 61; the estimates follow these within about 10 %, so the line lies
-// where both sides cost about the same.
+// their arithmetic. Measured, us per step, tiles / strips: periodic first order 256^2 9.1 / 20.1,
+// 512^2 26.0 / 31.5, 700^2 39.5 / 45.9, 800^2 51.9 / 51.2, 900^2 67.8 / 51.4; van Leer 256^2 11.4 / 24.5,
+// 512^2 31.7 / 37.6, 600^2 45.3 / 42.0, 700^2 61 / 55; warped van Leer 384^2 33.6 / 44.5, 512^2 53.1 / 52.2; the
+// estimates follow these within about 10 %, so the line lies where both sides cost about the same.
 // FP64 (a stage per CTA): FP64 operations per face and cell, 76 cycles per warp on each of the four
 // sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 158 / 277, 1024^2 2228 / 2696). Counting
 // the rectangles that the even split makes, and full and started passes half and half, and giving the faces
@@ -358,8 +359,10 @@ roeam_status setup_tile_kernel(roeam_grid *g)
     }
     std::vector<int4> rects;
     int mw = 0, mh = 0;
+    g->rect_base.clear();
     for (int k = 0; k < g->count; ++k) {
         const GridDev &G = g->hg[k];
+        g->rect_base.push_back((int)rects.size());
         const int nx = (G.ni + bw - 1) / bw, ny = (G.nj + bh - 1) / bh;
         for (int y = 0; y < ny; ++y)
             for (int x = 0; x < nx; ++x) {
@@ -371,6 +374,7 @@ roeam_status setup_tile_kernel(roeam_grid *g)
             }
     }
     g->nrects = (int)rects.size();
+    g->rect_base.push_back(g->nrects);
     g->rect_nx = (g->hg[0].ni + bw - 1) / bw;
     g->rect_ny = (g->hg[0].nj + bh - 1) / bh;
     g->rect_smem = tile_bytes<T>(mw + 2 * E, mh + 2 * E, g->muscl, g->curv, walls, stages);
@@ -549,8 +553,7 @@ unsigned long long *rate_slot(roeam_grid *g, long long step)
 // One SSP-RK3 step through the tile kernels. `state` is the buffer holding U^n; a whole-step launch
 // (FP32) leaves U^(n+1) in `other`, stage launches (FP64) update `state` in place.
 template <typename T>
-roeam_status launch_tile_step(roeam_grid *g, cudaStream_t s, long long step, double cfl, double dt_fixed, void *state,
-                              void *other)
+TileArgs<T> tile_args(roeam_grid *g)
 {
     TileArgs<T> a;
     std::memset(&a, 0, sizeof(a));
@@ -570,16 +573,24 @@ roeam_status launch_tile_step(roeam_grid *g, cudaStream_t s, long long step, dou
     a.vdx = (const T *)g->vdx;
     a.vdy = (const T *)g->vdy;
     a.solid = g->solid;
-    a.rate_rd = rate_slot(g, step);
-    a.rate_wr = rate_slot(g, step + 1);
-    a.cfl_t = T(cfl);
-    a.dt_fixed_t = T(dt_fixed);
     a.status = g->status;
 #ifdef ROEAM_DEBUG
     a.n_state = g->total_elems;
     a.n_vert = g->total_vert;
     a.n_solid = g->total_solid;
 #endif
+    return a;
+}
+
+template <typename T>
+roeam_status launch_tile_step(roeam_grid *g, cudaStream_t s, long long step, double cfl, double dt_fixed, void *state,
+                              void *other)
+{
+    TileArgs<T> a = tile_args<T>(g);
+    a.rate_rd = rate_slot(g, step);
+    a.rate_wr = rate_slot(g, step + 1);
+    a.cfl_t = T(cfl);
+    a.dt_fixed_t = T(dt_fixed);
     T *U = (T *)state, *A = (T *)other, *B = (T *)g->B;
     const auto run = [&]() {
         return TileLaunchers<T>::step(a, g->muscl, g->curv, g->kind == KIND_WALLS, g->nrects, g->rect_threads,
@@ -816,9 +827,48 @@ roeam_status do_get_state_device(roeam_grid *g, int idx, double *out, cudaStream
     return order_before(g, cs);
 }
 
+// FP64 residuals and norms run in the tile kernel where the steps do (the whole-step kernel of FP32 has no
+// such form): 256^2 reconstructed 165 us in strips, 73 in tiles. (At wall faces the two round differently.)
+template <typename T>
+bool tile_residual(const roeam_grid *g) { return g->tile_on && tile_stages<T>() == 1; }
+
+// The residual of grid idx (all grids with -1) into `dst` (the state's layout, `shift` elements lower).
+template <typename T>
+roeam_status launch_tile_residual(roeam_grid *g, int idx, void *dst, long long shift)
+{
+    TileArgs<T> a = tile_args<T>(g);
+    a.residual = 1;
+    a.dt_fixed_t = T(1);   // (no time step is read)
+    a.src = a.un = (const T *)g->U;
+    a.dst = (T *)dst;
+    a.dst_shift = shift;
+    const int lo = idx >= 0 ? g->rect_base[idx] : 0, hi = idx >= 0 ? g->rect_base[idx + 1] : g->nrects;
+    a.tiles += lo;
+    CUDA_TRY(TileLaunchers<T>::step(a, g->muscl, g->curv, g->kind == KIND_WALLS, hi - lo, g->rect_threads, g->rect_smem, g->stream));
+    return ROEAM_OK;
+}
+
+roeam_status read_norm(roeam_grid *g, int idx, int kind, int nb, int launches, double out[4])
+{
+    CUDA_TRY(launch_reduce_partials(g->partials, nb, 8, g->red_out, g->stream));
+    g->launches += launches;
+    CUDA_TRY(cudaMemcpyAsync(g->h_red, g->red_out, sizeof(double) * 8, cudaMemcpyDeviceToHost, g->stream));
+    CUDA_TRY(cudaStreamSynchronize(g->stream));
+    const double nf = g->hg[idx].nfluid > 0 ? g->hg[idx].nfluid : 1.0;
+    for (int k = 0; k < 4; ++k) out[k] = kind == ROEAM_NORM_L2 ? std::sqrt(g->h_red[k] / nf) : g->h_red[4 + k];
+    return ROEAM_OK;
+}
+
 template <typename T>
 roeam_status do_residual(roeam_grid *g, int idx, double *out)
 {
+    if (tile_residual<T>(g)) {
+        roeam_status st = launch_tile_residual<T>(g, idx, g->A, 0);
+        if (st != ROEAM_OK) return st;
+        g->launches += 1;
+        if (out) return do_get<T>(g, idx, g->A, out);
+        return ROEAM_OK;
+    }
     StageArgs<T> a = base_args<T>(g);
     a.mode = MODE_RESIDUAL;
     a.src = (const T *)g->U;
@@ -834,6 +884,14 @@ roeam_status do_residual(roeam_grid *g, int idx, double *out)
 template <typename T>
 roeam_status do_norm(roeam_grid *g, int idx, int kind, double out[4])
 {
+    if (tile_residual<T>(g) && g->stage_next == 0 && g->part_next == 0) {   // (A is free)
+        const long long n = (long long)g->hg[idx].ni * g->hg[idx].nj;
+        const int nb = (int)std::min<long long>(std::min<long long>((n + 255) / 256, g->partial_rows), 1024);
+        roeam_status st = launch_tile_residual<T>(g, idx, g->A, 0);
+        if (st != ROEAM_OK) return st;
+        CUDA_TRY(TileLaunchers<T>::norms(g->d_grids, idx, (const T *)g->A, g->partials, nb, g->stream));
+        return read_norm(g, idx, kind, nb, 3, out);
+    }
     StageArgs<T> a = base_args<T>(g);
     a.mode = MODE_NORM;
     a.work = nullptr;   // static units: each block's partials cover the same cells every call
@@ -846,13 +904,7 @@ roeam_status do_norm(roeam_grid *g, int idx, int kind, double out[4])
     const int nb = std::min(g->nblocks, std::min(g->partial_rows, a.tile_hi - a.tile_lo));
     CUDA_TRY(cudaMemsetAsync(g->partials, 0, sizeof(double) * 8 * g->partial_rows, g->stream));
     CUDA_TRY(Launchers<T>::stage(a, g->muscl, g->curv, g->kind, nb, g->stream));
-    CUDA_TRY(launch_reduce_partials(g->partials, nb, 8, g->red_out, g->stream));
-    g->launches += 2;
-    CUDA_TRY(cudaMemcpyAsync(g->h_red, g->red_out, sizeof(double) * 8, cudaMemcpyDeviceToHost, g->stream));
-    CUDA_TRY(cudaStreamSynchronize(g->stream));
-    const double nf = g->hg[idx].nfluid > 0 ? g->hg[idx].nfluid : 1.0;
-    for (int k = 0; k < 4; ++k) out[k] = kind == ROEAM_NORM_L2 ? std::sqrt(g->h_red[k] / nf) : g->h_red[4 + k];
-    return ROEAM_OK;
+    return read_norm(g, idx, kind, nb, 2, out);
 }
 
 template <typename T>
@@ -1888,19 +1940,24 @@ roeam_status do_residual_noalloc(roeam_grid *g, int idx, double *out)
     // G.poff (float64 copy); the shifts place both at the start of their scratch regions.
     T *region_t = (T *)scratch;
     double *region_d = (double *)((unsigned char *)scratch + bytes_t);
-    StageArgs<T> a = base_args<T>(g);
-    a.mode = MODE_RESIDUAL;
-    a.src = (const T *)g->U;
-    a.un = (const T *)g->U;
-    a.dst = region_t;
-    a.dst_shift = G.off;
+    if (tile_residual<T>(g)) {
+        st = launch_tile_residual<T>(g, idx, region_t, G.off);
+        if (st != ROEAM_OK) return st;
+    } else {
+        StageArgs<T> a = base_args<T>(g);
+        a.mode = MODE_RESIDUAL;
+        a.src = (const T *)g->U;
+        a.un = (const T *)g->U;
+        a.dst = region_t;
+        a.dst_shift = G.off;
 #ifdef ROEAM_DEBUG
-    a.n_dst = 4 * G.plane;
+        a.n_dst = 4 * G.plane;
 #endif
-    a.units = g->d_units_grid;
-    a.tile_lo = g->h_tile_base[idx];
-    a.tile_hi = g->h_tile_base[idx + 1];
-    CUDA_TRY(Launchers<T>::stage(a, g->muscl, g->curv, g->kind, g->nblocks, g->stream));
+        a.units = g->d_units_grid;
+        a.tile_lo = g->h_tile_base[idx];
+        a.tile_hi = g->h_tile_base[idx + 1];
+        CUDA_TRY(Launchers<T>::stage(a, g->muscl, g->curv, g->kind, g->nblocks, g->stream));
+    }
     CUDA_TRY(Launchers<T>::unpack(g->d_grids, idx, idx + 1, G.ni * G.nj, region_t, region_d, g->stream, G.off,
                                   G.poff));
     g->launches += 2;

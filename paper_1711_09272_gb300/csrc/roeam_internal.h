@@ -177,6 +177,8 @@ struct TileArgs {
     const T *vdx, *vdy;
     const uint8_t *solid;
     T alpha, beta;          // STAGES = 1
+    int residual;           // STAGES = 1: write the residual of `src` to `dst` instead of a stage's result,
+    long long dst_shift;    // cell x of it at dst + x - dst_shift
     int want_rate;
     const unsigned long long *rate_rd;
     unsigned long long *rate_wr, *rate_zero;
@@ -207,6 +209,9 @@ struct TileLaunchers {
     static cudaError_t step(const TileArgs<T> &a, int muscl, int curv, int walls, int ntiles, int threads, size_t smem,
                             cudaStream_t s);
     static cudaError_t prepare(int muscl, int curv, int walls);
+    // FP64 sums of squares [k] and maxima of magnitudes [4 + k] over grid idx of a residual R, one row of
+    // eight per block.
+    static cudaError_t norms(const GridDev *grids, int idx, const T *R, double *partials, int nblocks, cudaStream_t s);
 };
 
 // The ablation-variant stage kernels, instantiated in their own translation units.

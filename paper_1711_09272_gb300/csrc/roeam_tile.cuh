@@ -583,6 +583,14 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
                 cg.Xx = K.dy; cg.Xy = T(0); cg.Yx = T(0); cg.Yy = K.dx; cg.V = K.V;
             }
             const T sc = CURV ? rcp(cg.V) : cy;
+            if (STAGES == 1 && a.residual) {
+                for (int k = 0; k < 4; ++k) {
+                    const T D = CURV ? (fw[k] - fe[k] + fs[k]) - fn[k] : vfma(fw[k] - fe[k], rxy, fs[k]) - fn[k];
+                    out[k] = solid ? T(0) : D * sc;
+                }
+                if (TILE_OK(x, 4, n_state)) st_cell(a.dst + (x - a.dst_shift), out);
+                return;
+            }
             for (int k = 0; k < 4; ++k) {
                 T D = CURV ? (fw[k] - fe[k] + fs[k]) - fn[k] : vfma(fw[k] - fe[k], rxy, fs[k]) - fn[k];
                 if (solid) D = T(0);
@@ -638,6 +646,40 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
     }
 }
 
+// Sums and maxima of a residual in a fixed order: warp shuffles, then the block's warps.
+template <typename T>
+__global__ void __launch_bounds__(256) norms_kernel(const GridDev *grids, int idx, const T *__restrict__ R, double *partials)
+{
+    __shared__ double wred[8][8];
+    const GridDev &G = grids[idx];
+    const unsigned ni = (unsigned)G.ni, n = ni * (unsigned)G.nj, pitch = (unsigned)G.pitch;
+    const T *const base = R + G.off;
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (unsigned q = blockIdx.x * 256u + threadIdx.x; q < n; q += gridDim.x * 256u) {
+        const unsigned j = q / ni, i = q - j * ni;
+        T r[4];
+        ld_cell(base + 4 * ((long long)j * pitch + i), r);
+        for (int k = 0; k < 4; ++k) {
+            const double x = (double)r[k];
+            v[k] = fma(x, x, v[k]);
+            v[4 + k] = fmax(v[4 + k], fabs(x));
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1)
+        for (int k = 0; k < 8; ++k) {
+            const double x = __shfl_xor_sync(0xffffffffu, v[k], o);
+            v[k] = k < 4 ? v[k] + x : fmax(v[k], x);
+        }
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 8; ++k) wred[threadIdx.x >> 5][k] = v[k];
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double r = 0.0;
+        for (int w = 0; w < 8; ++w) r = threadIdx.x < 4 ? r + wred[w][threadIdx.x] : fmax(r, wred[w][threadIdx.x]);
+        partials[(size_t)blockIdx.x * 8 + threadIdx.x] = r;
+    }
+}
+
 // ------------------------------------------------------------------ launchers
 template <typename T, bool MUSCL, bool CURV, bool WALLS> struct TileVariant {
     static constexpr int STAGES = tile_stages<T>();
@@ -666,6 +708,13 @@ cudaError_t TileLaunchers<T>::step(const TileArgs<T> &a, int muscl, int curv, in
                                    size_t smem, cudaStream_t s)
 {
     ROEAM_TILE_DISPATCH(launch(a, ntiles, threads, smem, s))
+}
+
+template <typename T>
+cudaError_t TileLaunchers<T>::norms(const GridDev *grids, int idx, const T *R, double *partials, int nblocks, cudaStream_t s)
+{
+    norms_kernel<T><<<nblocks, 256, 0, s>>>(grids, idx, R, partials);
+    return cudaGetLastError();
 }
 
 // Allows the kernel the most shared memory that a launch may ask for (the attribute belongs to the
