@@ -282,7 +282,7 @@ template <typename T, int NS> __device__ __forceinline__ void stage3_phases(cons
     if (a.rate_zero && blockIdx.x == 0)
         for (int q = tid; q < a.ngrids; q += nt) a.rate_zero[q] = 0ull;
     T dt = T(0);
-    if (stage_mode) dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_value<T>(__ldg(a.rate_rd + g));
+    if (stage_mode) dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_at<T>(a.rate_rd + g);
 
     // starts the copies of plane k (to k1 at most) and, in the same group, of U^n of plane k - 2
     auto issue = [&](int k) {
@@ -571,7 +571,7 @@ template <int NS, bool ONE> __device__ __forceinline__ void stage3_march(const S
     if (a.rate_zero && blockIdx.x == 0)
         for (int i = tid; i < a.ngrids; i += TH) a.rate_zero[i] = 0ull;
     float dt = 0.f;
-    if (stage_mode) dt = a.dt_fixed_t > 0.f ? a.dt_fixed_t : a.cfl_t / rate_value<float>(__ldg(a.rate_rd + g));
+    if (stage_mode) dt = a.dt_fixed_t > 0.f ? a.dt_fixed_t : a.cfl_t / rate_at<float>(a.rate_rd + g);
 
     // starts the copies of plane k (to k1 at most) and, in the same group, of U^n of plane k - 2
     auto issue = [&](int k) {
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(256) unpack3_kernel(const GridDev3 *grids, int
             if (q < n) {
                 const unsigned jk = q / ni, i = q - jk * ni;
                 const long long c = (long long)jk * G.pitch + i;
-                ld_cell(quads + 4 * c, v[e]);
+                ld_own(quads + 4 * c, v[e]);
                 ld_tail<TW>(tails + TW * c, t[e]);
             }
         }

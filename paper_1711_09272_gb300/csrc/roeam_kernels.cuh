@@ -31,6 +31,10 @@ __device__ __forceinline__ int clampi(int a, int lo, int hi) { return a < lo ? l
 // waits before it touches anything else (and before it can end, so that completion stays in order).
 // pdl_trigger() lets the next launch start so early. Back-to-back small kernels: 4.1 us each in a
 // stream without it, 1.3 us with it.
+// What a launch writes is therefore not read-only for the lifetime of the next one: states, rates and
+// packed arrays are read by ordinary loads or asynchronous copies, which come after pdl_wait() and see
+// those writes. The non-coherent path (__ldg, const __restrict__ parameters) promises neither; it is for
+// unit tables and masks, which no kernel writes.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -498,6 +502,11 @@ __device__ __forceinline__ unsigned long long rate_bits(double r) { return (unsi
 template <typename T> __device__ __forceinline__ T rate_value(unsigned long long b);
 template <> __device__ __forceinline__ float rate_value<float>(unsigned long long b) { return __uint_as_float((unsigned)b); }
 template <> __device__ __forceinline__ double rate_value<double>(unsigned long long b) { return __longlong_as_double((long long)b); }
+// The rate in a slot that the launch before this one raised, to be read after pdl_wait().
+template <typename T> __device__ __forceinline__ T rate_at(const unsigned long long *slot)
+{
+    return rate_value<T>(*(const volatile unsigned long long *)slot);
+}
 
 // Largest of a warp's non-negative rates, through the bit patterns (redux: one instruction per word).
 __device__ __forceinline__ float warp_rate_max(float r)
@@ -812,17 +821,6 @@ template <typename T> struct GridRegs {
 
 // A cell's four conserved values lie together in the state buffers, so a cell is one 128-bit
 // access with one address (two in FP64).
-__device__ __forceinline__ void ld_cell(const float *p, float q[4])
-{
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-    q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
-}
-__device__ __forceinline__ void ld_cell(const double *p, double q[4])
-{
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(p)), b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-    q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
-}
-// The same through ordinary loads (shared memory, or a buffer that the kernel also writes).
 __device__ __forceinline__ void ld_own(const float *p, float q[4])
 {
     const float4 v = *reinterpret_cast<const float4 *>(p);
@@ -1077,7 +1075,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         T dt = T(0);
         if (a.mode == MODE_STAGE) {
             if (a.dt_fixed_t > T(0)) dt = a.dt_fixed_t;
-            else dt = a.cfl_t / rate_value<T>(__ldg(a.rate_rd + g));
+            else dt = a.cfl_t / rate_at<T>(a.rate_rd + g);
         }
 
         WC<T> Wn[NW];
@@ -1466,7 +1464,7 @@ template <int NT, typename T> __device__ __forceinline__ T block_max(T v, T *red
 constexpr int IO_PER = 4;
 
 template <typename T, typename H, bool RATE, bool CURV>
-__global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_lo, const H *__restrict__ packed,
+__global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_lo, const H *packed,
                                                    T *__restrict__ U, long long p_shift, RateOut<T> ro)
 {
     __shared__ T red[8];
@@ -1474,7 +1472,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_l
     const int g = g_lo + blockIdx.y;
     const GridDev &G = grids[g];
     const unsigned ni = (unsigned)G.ni, n = ni * (unsigned)G.nj, stride = gridDim.x * 256u;
-    const H *__restrict__ src = packed + (G.poff - p_shift);
+    const H *src = packed + (G.poff - p_shift);
     T *__restrict__ dst = U + G.off;
     const unsigned pitch = (unsigned)G.pitch;
     pdl_wait();
@@ -1518,13 +1516,13 @@ __global__ void __launch_bounds__(256) pack_kernel(const GridDev *grids, int g_l
 }
 
 template <typename T, typename H>
-__global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g_lo, const T *__restrict__ U,
+__global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g_lo, const T *U,
                                                      H *__restrict__ packed, long long u_shift, long long p_shift)
 {
     pdl_trigger();
     const GridDev &G = grids[g_lo + blockIdx.y];
     const unsigned ni = (unsigned)G.ni, n = ni * (unsigned)G.nj, stride = gridDim.x * 256u;
-    const T *__restrict__ src = U + (G.off - u_shift);
+    const T *src = U + (G.off - u_shift);
     H *__restrict__ dst = packed + (G.poff - p_shift);
     const unsigned pitch = (unsigned)G.pitch;
     pdl_wait();
@@ -1535,7 +1533,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const GridDev *grids, int g
             const unsigned q = q0 + e * stride;
             if (q < n) {
                 const unsigned j = q / ni, i = q - j * ni;
-                ld_cell(src + 4ull * (j * pitch + i), v[e]);
+                ld_own(src + 4ull * (j * pitch + i), v[e]);
             }
         }
 #pragma unroll
@@ -1588,7 +1586,7 @@ __global__ void __launch_bounds__(256) totals_kernel(const GridDev *grids, const
             V = G.dx * G.dy;
         }
         T q4[4];
-        ld_cell(U + G.off + 4 * ((long long)j * G.pitch + i), q4);
+        ld_own(U + G.off + 4 * ((long long)j * G.pitch + i), q4);
         for (int k = 0; k < 4; ++k) s[k] = fma(V, (double)q4[k], s[k]);
     }
     for (int o = 16; o > 0; o >>= 1)

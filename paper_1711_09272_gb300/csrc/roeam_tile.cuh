@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
             mirror_vel(q.u, q.v, nx, ny);
         }
     };
-    const T dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_value<T>(__ldg(a.rate_rd + g));
+    const T dt = a.dt_fixed_t > T(0) ? a.dt_fixed_t : a.cfl_t / rate_at<T>(a.rate_rd + g);
     const T rxy = K.dy / K.dx, cy = T(0.5) * K.dx * K.Vi;   // Cartesian residual weights
     copies_wait<0>();
     // (each thread turns the cells that it copied itself into primitives: no barrier in between, but for
@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(256) norms_kernel(const GridDev *grids, int id
     for (unsigned q = blockIdx.x * 256u + threadIdx.x; q < n; q += gridDim.x * 256u) {
         const unsigned j = q / ni, i = q - j * ni;
         T r[4];
-        ld_cell(base + 4 * ((long long)j * pitch + i), r);
+        ld_own(base + 4 * ((long long)j * pitch + i), r);
         for (int k = 0; k < 4; ++k) {
             const double x = (double)r[k];
             v[k] = fma(x, x, v[k]);
