@@ -195,7 +195,8 @@ __device__ __forceinline__ double sqrt1(double x)
     const double s = x * y, e = fma(-s, y, 1.0);
     return fma(s * e, fma(0.375, e, 0.5), s);
 }
-__device__ __forceinline__ double sqrt0(double x) { return dbits(x) > 0 ? sqrt1(x) : 0.0; }
+// (A subnormal, whose seed is infinite, counts as zero: |q|^2 / c^2 of a cell at rest but for 1e-155 c.)
+__device__ __forceinline__ double sqrt0(double x) { return __double2hiint(x) >= 0x00100000 ? sqrt1(x) : 0.0; }
 __device__ __forceinline__ V2 rcp(V2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
 __device__ __forceinline__ V2 rsq(V2 x) { return mk2(rsq(x.v.x), rsq(x.v.y)); }
 __device__ __forceinline__ V2 sqrt1(V2 x) { return x * rsq(x); }
@@ -559,9 +560,10 @@ template <typename T> __device__ __forceinline__ T ratio_P(T r0, T p0, T r1, T p
 template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V b);
 template <> __device__ __forceinline__ double limiter<double>(bool vanleer, double a, double b)
 {
-    // (sign tests on the bit patterns)
-    const bool keep = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && ((dbits(a) << 1) != 0);
-    const double m = vanleer ? (a + a) * (b * rcp(a + b)) : copysign(imin(fabs(a), fabs(b)), a);
+    // (sign tests on the bit patterns; a sum below the normal range has no reciprocal and no slope)
+    const double s = a + b;
+    const bool keep = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && (!vanleer || (__double2hiint(s) & 0x7ff00000) != 0);
+    const double m = vanleer ? (a + a) * (b * rcp(s)) : copysign(imin(fabs(a), fabs(b)), a);
     return keep ? m : 0.0;
 }
 
