@@ -1614,6 +1614,14 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS, bool ABL = false> struc
     {
         // (the rings, and the norm accumulators)
         const size_t smem = NT / 32 * ring_bytes<T, CURV, WALLS>() + (a.mode == MODE_NORM ? 8 * NT * sizeof(double) : 0);
+        // FP64 starts early only where every resident warp has a unit: the one-warp CTAs of a smaller grid
+        // would wait beside those still running and then share a sub-partition's FP64 pipe with each other
+        // while others idle. Three stages back to back, early / not: 64^2 244 / 140 us, 128^2 261 / 140, 256^2
+        // van Leer 564 / 486 (256^2 first order, nearly full, 267 / 273; full, as 1024^2, the same).
+        if (sizeof(T) == 8 && a.tile_hi - a.tile_lo < nblocks * (NT / 32)) {
+            stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL><<<nblocks, NT, smem, s>>>(a);
+            return cudaGetLastError();
+        }
         return launch_pdl(stage_kernel<T, MUSCL, CURV, WALLS, NT, ABL>, dim3(nblocks), dim3(NT), smem, s, a);
     }
     static int occupancy()
