@@ -285,21 +285,45 @@ roeam_status setup_tiles(roeam_grid *g, int cfg)
     return ROEAM_OK;
 }
 
+// Estimate of an FP32 step in strips, in cycles: the latency of three launches (a few rows each, longer on
+// the scalar path near walls), that of claiming where there are more units than warps, and the row
+// iterations of all units (one more than its rows each), those near walls counted dearer. Fitted to 224
+// measured steps (28 sizes and batches of 8 to a million cells, eight kernels; root mean square error 12 %):
+// periodic first order is 11 us plus 1.06 ns an iteration, and 8 us where units are claimed.
+double strip_step_cycles(const roeam_grid *g)
+{
+    const bool walls = g->kind == KIND_WALLS;
+    const int H = g->muscl ? 2 : 1;
+    double rows = 0;
+    for (const GridDev &G : g->hg) {
+        const int *bc = G.bc;
+        const double x = std::min(1.0, ((bc[0] == ROEAM_BC_WALL) + (bc[1] == ROEAM_BC_WALL)) / (double)G.ntx);
+        const double y = std::min(1.0, ((bc[2] == ROEAM_BC_WALL) + (bc[3] == ROEAM_BC_WALL)) * (H + 1) / (double)G.nj);
+        rows += (double)G.ntx * (G.nj + G.nty) * (1.0 + (g->muscl ? 1.1 : 0.35) * (x + y - x * y));
+    }
+    const double launches = (g->muscl ? 29000.0 : 23000.0) * (g->curv ? 1.12 : 1.0) * (walls ? (g->muscl ? 1.95 : 1.5) : 1.0);
+    const double row = (g->muscl ? 3.2 : 2.2) + (g->curv ? 1.1 : 0.0) + (walls ? (g->curv ? 0.4 : (g->muscl ? 1.0 : 0.8)) : 0.0);
+    return launches + (g->total_tiles > g->nblocks ? 16000.0 : 0.0) + row * rows;
+}
+
 // Whether roeam_rk_step runs this handle through the tile kernels, and their rectangles.
 //
 // Every grid is cut into rectangles of at most w x h cells of nearly equal size, one CTA each, and
 // (w, h) minimises an estimate of a step's cycles in which CTAs go over the SMs in rounds.
 // FP32 (a whole step per CTA): per stage a latency and the passes its face pairs take over an SM's
-// 128 lanes. Tiles are taken where that beats the strips' three launches of about 6 us each plus
-// their arithmetic. Measured, us per step, tiles / strips: periodic first order 256^2 9.1 / 20.1,
-// 512^2 26.0 / 31.5, 700^2 39.5 / 45.9, 800^2 51.9 / 51.2, 900^2 67.8 / 51.4; van Leer 256^2 11.4 / 24.5,
-// 512^2 31.7 / 37.6, 600^2 45.3 / 42.0, 700^2 61 / 55; warped van Leer 384^2 33.6 / 44.5, 512^2 53.1 / 52.2; the
-// estimates follow these within about 10 %, so the line lies where both sides cost about the same.
+// 128 lanes. Tiles are taken where that beats the estimate of the strips (strip_step_cycles): both follow
+// the measured times within about 12 %, so the line lies where both sides cost about the same. Measured,
+// us per step, tiles / strips: first order 256^2 9.3 / 14.8, 512^2 26.1 / 26.1, 700^2 39.6 / 44.4, 900^2
+// 68 / 46, 300 grids of 32^2 29 / 46, 152 of 64^2 53 / 59, 40 of 150^2 74 / 58, 50000 x 4 45 / 28, 4 x 50000
+// 48 / 73; van Leer 256^2 11.6 / 19.0, 512^2 31.9 / 30.2, 700^2 61 / 55, 300 of 32^2 50 / 56, 1000 of 9 x 8
+// 43 / 34; minmod in a box of walls 512^2 47 / 46, 300 of 32^2 56 / 109; warped van Leer with walls and solid
+// cells 300 of 32^2 66 / 145, 600 of 24^2 64 / 117, 16 of 256 x 200 154 / 140.
 // FP64 (a stage per CTA): FP64 operations per face and cell, 76 cycles per warp on each of the four
-// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 158 / 277, 1024^2 2228 / 2696). Counting
-// the rectangles that the even split makes, and full and started passes half and half, and giving the faces
-// a thread each: us per step, first order 100^2 48 -> 39, 128^2 58 -> 51, 256^2 162 -> 158, 800 x 20 58 -> 50;
-// reconstructed 128^2 82 -> 68, 256^2 224 -> 218, 331 x 97 124 -> 118 (32^2 31.8 -> 32.3, 1024^2 3232 -> 3250).
+// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 158 / 277, 1024^2 2228 / 2696; 64 grids of
+// 100 x 80 1151 / 2056, 300 of 32^2 665 / 1485). Counting the rectangles that the even split makes, and full
+// and started passes half and half, and giving the faces a thread each: us per step, first order 100^2 48 ->
+// 39, 128^2 58 -> 51, 256^2 162 -> 158, 800 x 20 58 -> 50; reconstructed 128^2 82 -> 68, 256^2 224 -> 218,
+// 331 x 97 124 -> 118 (32^2 31.8 -> 32.3, 1024^2 3232 -> 3250).
 // EXCHANGE sides (the caller sets ghost rows between stages) and the ablation kernels stay with the
 // strips.
 template <typename T>
@@ -354,8 +378,7 @@ roeam_status setup_tile_kernel(roeam_grid *g)
         }
     if (bw == 0) return ROEAM_OK;
     if (stages == 3) {
-        const double strips = 36000.0 + cells * (g->muscl ? 0.18 : 0.1) * (g->curv ? 1.35 : (walls ? 1.1 : 1.0));
-        if (best + 2500.0 > strips) return ROEAM_OK;
+        if (best > strip_step_cycles(g)) return ROEAM_OK;
     }
     std::vector<int4> rects;
     int mw = 0, mh = 0;
