@@ -851,7 +851,7 @@ roeam_status do_get_state_device(roeam_grid *g, int idx, double *out, cudaStream
 }
 
 // FP64 residuals and norms run in the tile kernel where the steps do (the whole-step kernel of FP32 has no
-// such form): 256^2 reconstructed 165 us in strips, 73 in tiles. (At wall faces the two round differently.)
+// such form): 256^2 reconstructed 165 us in strips, 73 in tiles.
 template <typename T>
 bool tile_residual(const roeam_grid *g) { return g->tile_on && tile_stages<T>() == 1; }
 

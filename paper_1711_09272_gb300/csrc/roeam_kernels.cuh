@@ -712,9 +712,12 @@ __device__ __forceinline__ void face_scalar(const Face<T> &f, const GridCoef<T> 
         if (pos) for (int k = 0; k < 4; ++k) { WL[k] = rL[k]; WR[k] = rR[k]; }
     }
     FS<T> L, R;
-    if (!MUSCL && (f.A.fl | f.B.fl) == 0) {
-        L = {f.A.r, vfma(f.nx, f.A.u, f.ny * f.A.v), vfma(f.nx, f.A.v, -(f.ny * f.A.u)), f.A.p, f.A.c2, f.A.H, f.A.sr, f.A.Mq};
-        R = {f.B.r, vfma(f.nx, f.B.u, f.ny * f.B.v), vfma(f.nx, f.B.v, -(f.ny * f.B.u)), f.B.p, f.B.c2, f.B.H, f.B.sr, f.B.Mq};
+    if constexpr (!MUSCL) {
+        // (a wall's mirrored side has the fluid cell's derived quantities, as in the tile kernel: a step gives
+        //  the same bits whichever kernel runs it)
+        const WC<T> &a = f.A.fl ? f.B : f.A, &b = f.A.fl || !f.B.fl ? f.B : f.A;
+        L = {WL[0], vfma(f.nx, WL[1], f.ny * WL[2]), vfma(f.nx, WL[2], -(f.ny * WL[1])), WL[3], a.c2, a.H, a.sr, a.Mq};
+        R = {WR[0], vfma(f.nx, WR[1], f.ny * WR[2]), vfma(f.nx, WR[2], -(f.ny * WR[1])), WR[3], b.c2, b.H, b.sr, b.Mq};
     } else {
         L = side_rot(WL[0], WL[1], WL[2], WL[3], f.nx, f.ny, K);
         R = side_rot(WR[0], WR[1], WR[2], WR[3], f.nx, f.ny, K);
