@@ -298,7 +298,9 @@ roeam_status roeam_set_tile_config(roeam_grid *g, int cfg);
 
 /* Autotuner: times `steps` SSP-RK3 steps at `cfl` with every tile shape on the current
  * state (best of two timings; shapes that give the same units and schedule are timed once),
- * restores the state after each trial, and keeps the fastest shape. best_cfg (nullable)
+ * restores the state after each trial, and keeps the fastest shape. The trials run the kernels
+ * that shapes apply to, also on handles whose steps run in rectangles (see above): there the
+ * figures are those of three roeam_rk_stage launches, and steps stay as they are. best_cfg (nullable)
  * receives it; ms_per_step (nullable, roeam_tile_config_count() doubles) the measured time
  * per step of each shape. The result is kept for the process: a later call on any handle
  * with the same workload (device, kernel family, every grid's sizes, boundary kinds and

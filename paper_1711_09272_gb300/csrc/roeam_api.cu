@@ -1575,7 +1575,13 @@ roeam_status roeam_autotune(roeam_grid *g, double cfl, int steps, int *best_cfg,
         }
         return setup_tiles(g, best);
     };
+    // the trials run the strips also where steps run in rectangles: those have no shapes
+    const bool tile_on = g->tile_on;
+    g->tile_on = false;
     st = run();
+    g->tile_on = tile_on;
+    for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);   // (of a trial that failed)
+    g->graphs.clear();
     cudaStreamSynchronize(g->stream);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
