@@ -1284,6 +1284,7 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
     if (st != ROEAM_OK) return cleanup(st);
     st = g->precision == 32 ? setup_tile_kernel<float>(g) : setup_tile_kernel<double>(g);
     if (st != ROEAM_OK) return cleanup(st);
+    g->rate_clean = g->tile_on;   // (every slot is zero)
     // Load the module that holds the allocation-free residual's scratch array now (CUDA loads
     // modules lazily, and committing the array is an allocation), so that a caller which makes
     // its handles at start-up has the array before it stops allocating.
