@@ -1684,6 +1684,7 @@ roeam_status roeam_edge_rows(roeam_grid *g, int grid_idx, int side, int stage, v
     CUDA_TRY(g->precision == 32
                  ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, false, g->stream)
                  : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, false, g->stream));
+    g->launches += 1;
     CUDA_TRY(cudaMemcpyAsync(dst, g->rows, g->esize * n, cudaMemcpyDefault, g->stream));
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type != cudaMemoryTypeDevice) {
@@ -1710,6 +1711,7 @@ roeam_status roeam_set_halo(roeam_grid *g, int grid_idx, int side, int stage, co
     CUDA_TRY(g->precision == 32
                  ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, true, g->stream)
                  : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, true, g->stream));
+    g->launches += 1;
     // a host source (page-locked memory copies asynchronously) may be reused once this returns
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, src) != cudaSuccess || at.type != cudaMemoryTypeDevice) {
