@@ -62,7 +62,8 @@ struct Range {
 struct TuneResult { int best; double ms[NUM_TILE_CFGS]; };
 std::mutex g_tune_mu;
 std::map<std::string, TuneResult> g_tune_cache;
-constexpr size_t MAX_GRAPHS = 8; // captured graphs kept per handle (one per (cfl, dt_fixed) pair)
+constexpr size_t MAX_GRAPHS = 8; // (cfl, dt_fixed) pairs whose captured graphs a handle keeps (one each, or one
+                                 // per buffer that U^n may be in)
 
 struct GraphKey {
     double cfl, dt_fixed;
@@ -707,7 +708,7 @@ roeam_status rk_steps(roeam_grid *g, double cfl, double dt_fixed, int nsteps)
     if (left >= GRAPH_STEPS) {
         GraphKey key{cfl, dt_fixed, g->U};
         auto it = g->graphs.find(key);
-        if (it == g->graphs.end() && g->graphs.size() >= MAX_GRAPHS) {
+        if (it == g->graphs.end() && g->graphs.size() >= MAX_GRAPHS * (swaps ? 2 : 1)) {
             // keep the cache small: a caller that varies dt_fixed call by call rebuilds graphs
             CUDA_TRY(cudaStreamSynchronize(g->stream));
             for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);

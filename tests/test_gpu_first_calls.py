@@ -18,7 +18,10 @@ def recorded(fn):
     with profile(activities=kinds) as prof:
         fn()
         torch.cuda.synchronize()
-    return [e.name for e in prof.events()]
+    names = [e.name for e in prof.events()]
+    if not any("kernel" in n for n in names):
+        pytest.skip("the profiler records no GPU work here")
+    return names
 
 
 @pytest.mark.parametrize("prec", [64, 32])
