@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "roeam.h"
@@ -162,6 +163,18 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
     const int every = 1 + (g->count - 1) / 16;   // (a sample of a large batch's grids)
     double best = 1e300;
     int bw = 0, bh = 0, bn = 1;
+    // Numbers of segments and the planes of the longest one; of equal planes the fewest segments. (Beyond 96 in
+    // steps of a sixteenth: needles along z need more, FP32 1 x 1 x 4000 259 us a step with 96 segments, 177 with
+    // 152; FP64 1342 and 906.)
+    std::vector<std::pair<int, int>> cuts;
+    for (int n = 1; n <= max_nk; n += n < 96 ? 1 : n / 16) {
+        int zs = 0;
+        for (int q = 0; q < g->count; q += every) {
+            const int nk = g->hg[q].nk, sn = std::min(n, nk);
+            zs = std::max(zs, (nk + sn - 1) / sn);
+        }
+        if (cuts.empty() || zs < cuts.back().second) cuts.emplace_back(n, zs);
+    }
     auto consider = [&](int w, int h, double plane, double segment, double planes_more) {
         double planes = 0;   // of all rectangles: their cycles over the SMs bound the cost from below
         for (int q = 0; q < g->count; q += every) {
@@ -169,26 +182,21 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
             planes += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * G.nk;
         }
         if (planes * plane / num_sms >= best) return;
-        // (beyond 96 segments in steps of a sixteenth: needles along z need more, FP32 1 x 1 x 4000 259 us a
-        //  step with 96 segments, 177 with 152; FP64 1342 and 906)
-        for (int n = 1; n <= max_nk; n += n < 96 ? 1 : n / 16) {
+        for (const auto &c : cuts) {
             double units = 0;
-            int zs = 0;
             for (int q = 0; q < g->count; q += every) {
                 const GridDev3 &G = g->hg[q];
-                const int sn = std::min(n, G.nk);
-                units += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * sn;
-                zs = std::max(zs, (G.nk + sn - 1) / sn);
+                units += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * std::min(c.first, G.nk);
             }
-            const double cost = std::ceil(units / num_sms) * (plane * (zs + planes_more) + segment);
-            if (cost < best * 0.999) { best = cost; bw = w; bh = h; bn = n; }
+            const double cost = std::ceil(units / num_sms) * (plane * (c.second + planes_more) + segment);
+            if (cost < best * 0.999) { best = cost; bw = w; bh = h; bn = c.first; }
         }
     };
     if (f32) consider(MARCH3_X, MARCH3_Y, 5000, 6000, 1.0);
     else
-        for (int w = 64; w >= 1; --w)
-            for (int h = 2; h <= 64; ++h) {
-                if (w > max_ni + 1 || h > max_nj + 1 || bytes3<T>(w, h, g->nv) == 0) continue;
+        for (int w = std::min(64, max_ni + 1); w >= 1; --w)
+            for (int h = 2; h <= std::min(64, max_nj + 1); ++h) {
+                if (bytes3<T>(w, h, g->nv) == 0) break;
                 // (a single grid's rectangles are as large as its even split makes them; a phase's last
                 //  pass counts half its lanes idle)
                 const int W = g->count == 1 ? (max_ni + (max_ni + w - 1) / w - 1) / ((max_ni + w - 1) / w) : w;

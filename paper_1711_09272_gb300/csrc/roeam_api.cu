@@ -113,7 +113,6 @@ struct roeam_grid {
     void *U = nullptr, *A = nullptr, *B = nullptr;      // U^n (in place), stage buffers
     void *vdx = nullptr, *vdy = nullptr;
     uint8_t *solid = nullptr;
-    void *rows = nullptr;            // two rows of the widest grid (roeam_edge_rows, roeam_set_halo)
     int stage_next = 0;              // next stage of a step run stage by stage (roeam_rk_stage)
     double *staging = nullptr;
     unsigned long long *rate = nullptr;                  // RATE_SLOTS x count slots (see rate_slot)
@@ -345,59 +344,90 @@ roeam_status setup_tile_kernel(roeam_grid *g)
     }
     if (stages == 3 && cells > 1.5e6) return ROEAM_OK;   // (strips win well below this)
     const double slow = g->curv ? 1.28 : (walls ? 1.18 : 1.0);
-    const int every = 1 + (g->count - 1) / 256;           // (a sample of a large batch's grids)
-    double best = 1e300;
-    int bw = 0, bh = 0;
-    for (int w = 64; w >= 4; --w)   // (of equal estimates the widest: 32 x 14 runs the 256^2 Gresho step in
-        for (int h = 2; h <= 64; ++h) {   // 13.0 us, 16 x 32 in 14.3)
-            if (w > max_ni + 3 || h > max_nj + 1) continue;
-            const size_t smem = tile_bytes<T>(w + 2 * E, h + 2 * E, g->muscl, g->curv, walls, stages);
-            if (smem > TILE_SMEM_MAX) continue;
-            double t = 0;
-            if (stages == 3) {
-                for (int s = 0; s < stages; ++s) {
-                    const int e = H * (stages - 1 - s);
-                    const double pairs = (double)(w + 2 * e + 1) * (h + 2 * e + 1);
-                    t += 2100 + std::ceil(pairs / 128) * (g->muscl ? 1030 : 750) * slow;
-                }
-            } else {
-                // (a single grid's rectangles are as large as its even split makes them; a phase's last
-                //  pass counts half its lanes idle: warps spread over the sub-partitions unevenly then)
-                const int W = g->count == 1 ? (max_ni + (max_ni + w - 1) / w - 1) / ((max_ni + w - 1) / w) : w;
-                const int Y = g->count == 1 ? (max_nj + (max_nj + h - 1) / h - 1) / ((max_nj + h - 1) / h) : h;
-                const auto passes = [](double n) { return 0.5 * (std::ceil(n / 128) + n / 128); };
-                const double faces = (double)(W + 1) * Y + (double)W * (Y + 1);
-                t = 76 * ((g->muscl ? 175 : 129) * passes(faces) + (g->muscl ? 13 : 38) * passes((double)(W + 2 * H) * (Y + 2 * H)) +
-                          (g->muscl ? 52 : 16) * passes((double)(W + 2) * (Y + 2)) + 32 * passes((double)W * Y));
+    const int every = 1 + (g->count - 1) / 128;           // (a sample of a large batch's grids)
+    double sampled = 0, grids = 0;                        // (they bound the rectangles' number from below)
+    for (int k = 0; k < g->count; k += every) {
+        sampled += (double)every * g->hg[k].ni * g->hg[k].nj;
+        grids += every;
+    }
+    // cycles of one rectangle (0: does not fit)
+    const auto cycles = [&](int w, int h) {
+        if (tile_bytes<T>(w + 2 * E, h + 2 * E, g->muscl, g->curv, walls, stages) > TILE_SMEM_MAX) return 0.0;
+        double t = 0;
+        if (stages == 3) {
+            for (int s = 0; s < stages; ++s) {
+                const int e = H * (stages - 1 - s);
+                const double pairs = (double)(w + 2 * e + 1) * (h + 2 * e + 1);
+                t += 2100 + std::ceil(pairs / 128) * (g->muscl ? 1030 : 750) * slow;
             }
-            if (t >= best) continue;   // (at least one round)
-            double tiles = 0;
-            for (int k = 0; k < g->count; k += every)
-                tiles += (double)every * ((g->hg[k].ni + w - 1) / w) * ((g->hg[k].nj + h - 1) / h);
-            const double cost = std::ceil(tiles / g->num_sms) * t;
+            return t;
+        }
+        // (a single grid's rectangles are as large as its even split makes them; a phase's last
+        //  pass counts half its lanes idle: warps spread over the sub-partitions unevenly then)
+        const int W = g->count == 1 ? (max_ni + (max_ni + w - 1) / w - 1) / ((max_ni + w - 1) / w) : w;
+        const int Y = g->count == 1 ? (max_nj + (max_nj + h - 1) / h - 1) / ((max_nj + h - 1) / h) : h;
+        const auto passes = [](double n) { return 0.5 * (std::ceil(n / 128) + n / 128); };
+        const double faces = (double)(W + 1) * Y + (double)W * (Y + 1);
+        return 76 * ((g->muscl ? 175 : 129) * passes(faces) + (g->muscl ? 13 : 38) * passes((double)(W + 2 * H) * (Y + 2 * H)) +
+                     (g->muscl ? 52 : 16) * passes((double)(W + 2) * (Y + 2)) + 32 * passes((double)W * Y));
+    };
+    // rectangles of the sampled grids along x for each width, along y for each height
+    const int most_w = std::min(64, max_ni + 3), most_h = std::min(64, max_nj + 1), samples = (g->count + every - 1) / every;
+    std::vector<double> across((size_t)(most_w + 1) * samples), up((size_t)(most_h + 1) * samples);
+    for (int w = 4; w <= most_w; ++w)
+        for (int q = 0; q < samples; ++q) across[(size_t)w * samples + q] = (g->hg[q * every].ni + w - 1) / w;
+    for (int h = 2; h <= most_h; ++h)
+        for (int q = 0; q < samples; ++q) up[(size_t)h * samples + q] = (g->hg[q * every].nj + h - 1) / h;
+    const auto cost_of = [&](int w, int h, double t) {
+        const double *x = &across[(size_t)w * samples], *y = &up[(size_t)h * samples];
+        double tiles = 0;
+        for (int q = 0; q < samples; ++q) tiles += x[q] * y[q];
+        return std::ceil(every * tiles / g->num_sms) * t;
+    };
+    // A coarse look first: what its best beats by the lower bound alone need not be counted.
+    double limit = 1e300, best = 1e300;
+    for (int w = 8; w <= most_w; w += 8)
+        for (int h = 4; h <= most_h; h += 4) {
+            const double t = cycles(w, h);
+            if (t == 0) break;
+            if (std::ceil(std::max(grids, sampled / (w * h)) / g->num_sms) * t < limit) limit = std::min(limit, cost_of(w, h, t));
+        }
+    int bw = 0, bh = 0;
+    for (int w = most_w; w >= 4; --w)   // (of equal estimates the widest: 32 x 14 runs the 256^2 Gresho step in
+        for (int h = 2; h <= most_h; ++h) {   // 13.0 us, 16 x 32 in 14.3)
+            const double t = cycles(w, h);
+            if (t == 0) break;
+            const double least = std::ceil(std::max(grids, sampled / (w * h)) / g->num_sms) * t;
+            if (least > limit || least >= best) continue;
+            const double cost = cost_of(w, h, t);
             if (cost < best * 0.999) { best = cost; bw = w; bh = h; }
         }
     if (bw == 0) return ROEAM_OK;
     if (stages == 3) {
         if (best > strip_step_cycles(g)) return ROEAM_OK;
     }
-    std::vector<int4> rects;
+    std::vector<int4> rects;   // (a single grid's are computed from rect_nx and rect_ny)
     int mw = 0, mh = 0;
     g->rect_base.clear();
+    g->nrects = 0;
     for (int k = 0; k < g->count; ++k) {
         const GridDev &G = g->hg[k];
-        g->rect_base.push_back((int)rects.size());
         const int nx = (G.ni + bw - 1) / bw, ny = (G.nj + bh - 1) / bh;
-        for (int y = 0; y < ny; ++y)
-            for (int x = 0; x < nx; ++x) {
-                const int x0 = tile_edge(x, G.ni, nx), x1 = tile_edge(x + 1, G.ni, nx);
-                const int y0 = tile_edge(y, G.nj, ny), y1 = tile_edge(y + 1, G.nj, ny);
-                rects.push_back(make_int4(k, x0, y0, (x1 - x0) | ((y1 - y0) << 16)));
-                mw = std::max(mw, x1 - x0);
-                mh = std::max(mh, y1 - y0);
+        g->rect_base.push_back(g->nrects);
+        g->nrects += nx * ny;
+        const int wide = G.ni / nx, wider = G.ni % nx, high = G.nj / ny, higher = G.nj % ny;
+        mw = std::max(mw, wide + (wider > 0));
+        mh = std::max(mh, high + (higher > 0));
+        for (int y = 0, y0 = 0; y < ny && g->count > 1; ++y) {
+            const int h = high + (y < higher);
+            for (int x = 0, x0 = 0; x < nx; ++x) {
+                const int w = wide + (x < wider);
+                rects.push_back(make_int4(k, x0, y0, w | h << 16));
+                x0 += w;
             }
+            y0 += h;
+        }
     }
-    g->nrects = (int)rects.size();
     g->rect_base.push_back(g->nrects);
     g->rect_nx = (g->hg[0].ni + bw - 1) / bw;
     g->rect_ny = (g->hg[0].nj + bh - 1) / bh;
@@ -409,9 +439,11 @@ roeam_status setup_tile_kernel(roeam_grid *g)
     // come early, and wait) pair up on the SMs that are idle now (64^2 FP64 vortex, 20 steps: 855 us,
     // 682 us with the room taken).
     if (g->nrects <= g->num_sms) g->rect_smem = std::max(g->rect_smem, (size_t)115 * 1024);
-    CUDA_TRY(TileLaunchers<T>::prepare(g->muscl, g->curv, walls));
-    CUDA_TRY(cudaMalloc(&g->d_rects, sizeof(int4) * rects.size()));
-    CUDA_TRY(cudaMemcpy(g->d_rects, rects.data(), sizeof(int4) * rects.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(TileLaunchers<T>::prepare(g->muscl, g->curv, walls, g->count == 1));
+    if (g->count > 1) {
+        CUDA_TRY(cudaMalloc(&g->d_rects, sizeof(int4) * rects.size()));
+        CUDA_TRY(cudaMemcpy(g->d_rects, rects.data(), sizeof(int4) * rects.size(), cudaMemcpyHostToDevice));
+    }
     g->tile_on = true;
     return ROEAM_OK;
 }
@@ -867,7 +899,7 @@ roeam_status launch_tile_residual(roeam_grid *g, int idx, void *dst, long long s
     a.dst = (T *)dst;
     a.dst_shift = shift;
     const int lo = idx >= 0 ? g->rect_base[idx] : 0, hi = idx >= 0 ? g->rect_base[idx + 1] : g->nrects;
-    a.tiles += lo;
+    if (a.tiles) a.tiles += lo;
     CUDA_TRY(TileLaunchers<T>::step(a, g->muscl, g->curv, g->kind == KIND_WALLS, hi - lo, g->rect_threads, g->rect_smem, g->stream));
     return ROEAM_OK;
 }
@@ -1157,11 +1189,9 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
     g->state_set.assign(count, 0);
     long long off = 0, voff = 0, soff = 0, poff = 0;
     bool any_solid = false;
-    int max_ni = 0;
     for (int k = 0; k < count; ++k) {
         const roeam_grid_desc &q = descs[k];
         GridDev &G = g->hg[k];
-        max_ni = std::max(max_ni, q.ni);
         std::memset(&G, 0, sizeof(G));
         G.ni = q.ni;
         G.nj = q.nj;
@@ -1265,7 +1295,6 @@ roeam_status roeam_create_grid(int count, const roeam_grid_desc *descs, int devi
         CREATE_TRY(cudaMemcpy(g->solid, hs.data(), hs.size(), cudaMemcpyHostToDevice));
     }
     CREATE_TRY(cudaMalloc(&g->staging, sizeof(double) * (size_t)g->total_packed));
-    CREATE_TRY(cudaMalloc(&g->rows, g->esize * 8 * (size_t)max_ni));
     CREATE_TRY(cudaMalloc(&g->rate, sizeof(unsigned long long) * RATE_SLOTS * count));
     CREATE_TRY(cudaMemset(g->rate, 0, sizeof(unsigned long long) * RATE_SLOTS * count));
     CREATE_TRY(cudaMalloc(&g->status, sizeof(unsigned)));
@@ -1317,7 +1346,6 @@ void roeam_destroy_grid(roeam_grid *g)
     cudaFree(g->vdy);
     cudaFree(g->solid);
     cudaFree(g->staging);
-    cudaFree(g->rows);
     cudaFree(g->rate);
     cudaFree(g->status);
     cudaFree(g->work);
@@ -1680,13 +1708,14 @@ roeam_status roeam_edge_rows(roeam_grid *g, int grid_idx, int side, int stage, v
     CUDA_TRY(cudaSetDevice(g->device));
     const GridDev &G = g->hg[grid_idx];
     const int r0 = side == 2 ? 0 : G.nj - 2;
-    // (gathered on the device, then one copy to wherever dst lives)
+    // (gathered on the device, in the staging buffer, which holds at least four rows; then one copy to wherever
+    //  dst lives)
     const long long n = 8ll * G.ni;
     CUDA_TRY(g->precision == 32
-                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, false, g->stream)
-                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, false, g->stream));
+                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->staging, false, g->stream)
+                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, g->staging, false, g->stream));
     g->launches += 1;
-    CUDA_TRY(cudaMemcpyAsync(dst, g->rows, g->esize * n, cudaMemcpyDefault, g->stream));
+    CUDA_TRY(cudaMemcpyAsync(dst, g->staging, g->esize * n, cudaMemcpyDefault, g->stream));
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type != cudaMemoryTypeDevice) {
         cudaGetLastError();
@@ -1708,10 +1737,10 @@ roeam_status roeam_set_halo(roeam_grid *g, int grid_idx, int side, int stage, co
     CUDA_TRY(cudaSetDevice(g->device));
     const int r0 = side == 2 ? -2 : G.nj;
     const long long n = 8ll * G.ni;
-    CUDA_TRY(cudaMemcpyAsync(g->rows, src, g->esize * n, cudaMemcpyDefault, g->stream));
+    CUDA_TRY(cudaMemcpyAsync(g->staging, src, g->esize * n, cudaMemcpyDefault, g->stream));
     CUDA_TRY(g->precision == 32
-                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->rows, true, g->stream)
-                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (double *)g->rows, true, g->stream));
+                 ? Launchers<float>::rows((float *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, (float *)g->staging, true, g->stream)
+                 : Launchers<double>::rows((double *)stage_source(g, stage), G.off, G.pitch, G.ni, r0, g->staging, true, g->stream));
     g->launches += 1;
     // a host source (page-locked memory copies asynchronously) may be reused once this returns
     cudaPointerAttributes at;

@@ -189,9 +189,6 @@ struct TileArgs {
 #endif
 };
 
-// First column of rectangle x of n over ni columns (rows likewise).
-inline int tile_edge(int x, int ni, int n) { return x * (ni / n) + (x < ni % n ? x : ni % n); }
-
 // Shared memory of a tile of W x R positions (the rectangle and its halo): quads of T per position
 // (U, primitives, two fluxes, derived quantities or two slopes, U^n or U^(1) and U^(2)), the Eq. 97 ratios (one row
 // more: the pair list's unused faces past the last row read it), vertices, column and row maps,
@@ -208,7 +205,7 @@ template <typename T>
 struct TileLaunchers {
     static cudaError_t step(const TileArgs<T> &a, int muscl, int curv, int walls, int ntiles, int threads, size_t smem,
                             cudaStream_t s);
-    static cudaError_t prepare(int muscl, int curv, int walls);
+    static cudaError_t prepare(int muscl, int curv, int walls, bool one);   // (one: a single grid)
     // FP64 sums of squares [k] and maxima of magnitudes [4 + k] over grid idx of a residual R, one row of
     // eight per block.
     static cudaError_t norms(const GridDev *grids, int idx, const T *R, double *partials, int nblocks, cudaStream_t s);

@@ -691,12 +691,10 @@ template <typename T, bool MUSCL, bool CURV, bool WALLS> struct TileVariant {
         return launch_pdl(a.ngrids == 1 ? tile_kernel<T, MUSCL, CURV, WALLS, STAGES, true> : tile_kernel<T, MUSCL, CURV, WALLS, STAGES, false>,
                           dim3((unsigned)ntiles), dim3((unsigned)threads), smem, s, a);
     }
-    static cudaError_t prepare(size_t smem)
+    static cudaError_t prepare(bool one, size_t smem)
     {
-        const cudaError_t e = cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return e != cudaSuccess ? e : cudaFuncSetAttribute(tile_kernel<T, MUSCL, CURV, WALLS, STAGES, false>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaFuncSetAttribute(one ? tile_kernel<T, MUSCL, CURV, WALLS, STAGES, true> : tile_kernel<T, MUSCL, CURV, WALLS, STAGES, false>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
 };
 
@@ -723,9 +721,9 @@ cudaError_t TileLaunchers<T>::norms(const GridDev *grids, int idx, const T *R, d
 // Allows the kernel the most shared memory that a launch may ask for (the attribute belongs to the
 // device, so every handle asks for the same).
 template <typename T>
-cudaError_t TileLaunchers<T>::prepare(int muscl, int curv, int walls)
+cudaError_t TileLaunchers<T>::prepare(int muscl, int curv, int walls, bool one)
 {
-    ROEAM_TILE_DISPATCH(prepare(TILE_SMEM_MAX))
+    ROEAM_TILE_DISPATCH(prepare(one, TILE_SMEM_MAX))
 }
 
 }  // namespace roeam

@@ -20,9 +20,9 @@ def test_trials_run_what_the_shapes_apply_to(prec):
         q.set_state(U, 0)
         n0 = b.launches
         best, ms = b.autotune(0.4, steps)
-        distinct = len(set(ms))
         assert ms[best] == ms.min()
-        assert b.launches - n0 == distinct * 2 * (1 + steps) * 3
+        # (every shape ends up at two rows here: two layouts, claiming and static, each timed twice)
+        assert b.launches - n0 == 2 * 2 * (1 + steps) * 3
         for n in (1, 9, 2):
             n0 = b.launches
             db, dq = (x.step(cfl=0.4, nsteps=n, want_dt=True) for x in (b, q))
