@@ -116,6 +116,9 @@ struct roeam_grid {
     int stage_next = 0;              // next stage of a step run stage by stage (roeam_rk_stage)
     double *staging = nullptr;
     unsigned long long *rate = nullptr;                  // RATE_SLOTS x count slots (see rate_slot)
+#ifdef ROEAM_DEBUG
+    long long debug_limit[3] = {-1, -1, -1};   // (roeam_debug_limit)
+#endif
     bool rate_clean = false;        // the next step's output slot is already zero (a tile step ran last)
     // Tile kernels (see setup_tile_kernel): whether rk_step uses them, their work list and launch
     bool tile_on = false;
@@ -577,6 +580,20 @@ roeam_status upload_coef(roeam_grid *g)
 }
 
 // Stage-kernel arguments common to every mode.
+#ifdef ROEAM_DEBUG
+// Elements of a buffer that the kernels' bounds checks allow (0 source, 1 U^n, 2 destination): all of them,
+// or what roeam_debug_limit set.
+long long debug_size(const roeam_grid *g, int buffer, long long n) { return g->debug_limit[buffer] >= 0 ? g->debug_limit[buffer] : n; }
+template <typename A> void debug_sizes(const roeam_grid *g, A &a)
+{
+    a.n_state = debug_size(g, 0, g->total_elems);
+    a.n_un = debug_size(g, 1, g->total_elems);
+    a.n_dst = debug_size(g, 2, g->total_elems);
+    a.n_vert = g->total_vert;
+    a.n_solid = g->total_solid;
+}
+#endif
+
 template <typename T>
 StageArgs<T> base_args(roeam_grid *g)
 {
@@ -594,9 +611,7 @@ StageArgs<T> base_args(roeam_grid *g)
     a.status = g->status;
     a.work = g->eff_dyn ? g->work : nullptr;
 #ifdef ROEAM_DEBUG
-    a.n_state = a.n_dst = g->total_elems;
-    a.n_vert = g->total_vert;
-    a.n_solid = g->total_solid;
+    debug_sizes(g, a);
 #endif
     return a;
 }
@@ -631,9 +646,7 @@ TileArgs<T> tile_args(roeam_grid *g)
     a.solid = g->solid;
     a.status = g->status;
 #ifdef ROEAM_DEBUG
-    a.n_state = g->total_elems;
-    a.n_vert = g->total_vert;
-    a.n_solid = g->total_solid;
+    debug_sizes(g, a);
 #endif
     return a;
 }
@@ -888,11 +901,17 @@ roeam_status do_get_state_device(roeam_grid *g, int idx, double *out, cudaStream
 template <typename T>
 bool tile_residual(const roeam_grid *g) { return g->tile_on && tile_stages<T>() == 1; }
 
-// The residual of grid idx (all grids with -1) into `dst` (the state's layout, `shift` elements lower).
+// The residual of grid idx (all grids with -1) into `dst` (the state's layout, `shift` elements lower; room for
+// `room` elements, or the state's with 0).
 template <typename T>
-roeam_status launch_tile_residual(roeam_grid *g, int idx, void *dst, long long shift)
+roeam_status launch_tile_residual(roeam_grid *g, int idx, void *dst, long long shift, long long room = 0)
 {
     TileArgs<T> a = tile_args<T>(g);
+#ifdef ROEAM_DEBUG
+    if (room) a.n_dst = debug_size(g, 2, room);
+#else
+    (void)room;
+#endif
     a.residual = 1;
     a.dt_fixed_t = T(1);   // (no time step is read)
     a.src = a.un = (const T *)g->U;
@@ -1631,6 +1650,17 @@ roeam_status roeam_autotune(roeam_grid *g, double cfl, int steps, int *best_cfg,
     return st;
 }
 
+#ifdef ROEAM_DEBUG
+// Test hook of bounds-checked builds: the checks of buffer 0 (source), 1 (U^n) or 2 (destination) allow only its
+// first n elements (-1: all again). What they refuse is skipped although it lies in the buffer.
+extern "C" void roeam_debug_limit(roeam_grid *g, int buffer, long long n)
+{
+    g->debug_limit[buffer] = n;
+    for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);
+    g->graphs.clear();
+}
+#endif
+
 unsigned long long roeam_launch_count(const roeam_grid *g) { return g ? g->launches : 0ull; }
 
 long long roeam_cell_count(const roeam_grid *g, int grid_idx)
@@ -2003,7 +2033,7 @@ roeam_status do_residual_noalloc(roeam_grid *g, int idx, double *out)
     T *region_t = (T *)scratch;
     double *region_d = (double *)((unsigned char *)scratch + bytes_t);
     if (tile_residual<T>(g)) {
-        st = launch_tile_residual<T>(g, idx, region_t, G.off);
+        st = launch_tile_residual<T>(g, idx, region_t, G.off, 4 * G.plane);
         if (st != ROEAM_OK) return st;
     } else {
         StageArgs<T> a = base_args<T>(g);
@@ -2013,7 +2043,7 @@ roeam_status do_residual_noalloc(roeam_grid *g, int idx, double *out)
         a.dst = region_t;
         a.dst_shift = G.off;
 #ifdef ROEAM_DEBUG
-        a.n_dst = 4 * G.plane;
+        a.n_dst = debug_size(g, 2, 4 * G.plane);
 #endif
         a.units = g->d_units_grid;
         a.tile_lo = g->h_tile_base[idx];

@@ -77,9 +77,9 @@ struct StageArgs {
     // both, so that the next launch on the handle's stream starts from zero.
     unsigned *work;
 #ifdef ROEAM_DEBUG
-    // buffer sizes (elements of each state buffer and of dst, of each vertex plane buffer; bytes of
+    // buffer sizes (elements of src, un and dst, of each vertex plane buffer; bytes of
     // the solid masks), read by the bounds checks of debug builds
-    long long n_state, n_dst, n_vert, n_solid;
+    long long n_state, n_un, n_dst, n_vert, n_solid;
 #endif
 };
 
@@ -185,7 +185,7 @@ struct TileArgs {
     T cfl_t, dt_fixed_t;
     unsigned *status;
 #ifdef ROEAM_DEBUG
-    long long n_state, n_vert, n_solid;   // buffer sizes, read by the bounds checks of debug builds
+    long long n_state, n_un, n_dst, n_vert, n_solid;   // buffer sizes, read by the bounds checks of debug builds
 #endif
 };
 

@@ -1058,7 +1058,7 @@ __global__ void __launch_bounds__(NT, (stage_min_blocks<T, MUSCL, CURV, ABL>()))
         else { R.vdx = R.vdy = nullptr; R.vpitch = 0; }
 #ifdef ROEAM_DEBUG
         R.dbg.lo[DB_SRC] = (const unsigned char *)a.src; R.dbg.bytes[DB_SRC] = sizeof(T) * a.n_state;
-        R.dbg.lo[DB_UN] = (const unsigned char *)a.un; R.dbg.bytes[DB_UN] = sizeof(T) * a.n_state;
+        R.dbg.lo[DB_UN] = (const unsigned char *)a.un; R.dbg.bytes[DB_UN] = sizeof(T) * a.n_un;
         R.dbg.lo[DB_DST] = (const unsigned char *)a.dst; R.dbg.bytes[DB_DST] = sizeof(T) * a.n_dst;
         R.dbg.lo[DB_VDX] = (const unsigned char *)a.vdx; R.dbg.bytes[DB_VDX] = sizeof(T) * a.n_vert;
         R.dbg.lo[DB_VDY] = (const unsigned char *)a.vdy; R.dbg.bytes[DB_VDY] = sizeof(T) * a.n_vert;

@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
             const bool own = !ghost && c >= E && c < E + w && r >= E && r < E + h;   // (others also update halo cells)
             const long long x = G.off + 4 * ((long long)(jy0 + r) * pitch + (ix0 + c));
             if (STAGES == 1) {
-                if (alpha != T(0)) ld_own(a.un + x, un);
+                if (alpha != T(0) && TILE_OK(x, 4, n_un)) ld_own(a.un + x, un);
                 else for (int k = 0; k < 4; ++k) un[k] = uk[k];
             } else if (WALLS) {
                 ld_own(U + 4 * at, un);
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
                     const T D = CURV ? (fw[k] - fe[k] + fs[k]) - fn[k] : vfma(fw[k] - fe[k], rxy, fs[k]) - fn[k];
                     out[k] = solid ? T(0) : D * sc;
                 }
-                if (TILE_OK(x, 4, n_state)) st_cell(a.dst + (x - a.dst_shift), out);
+                if (TILE_OK(x - a.dst_shift, 4, n_dst)) st_cell(a.dst + (x - a.dst_shift), out);
                 return;
             }
             for (int k = 0; k < 4; ++k) {
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
                 prims(out, q);
                 if constexpr (WALLS && ghost) mirror_ghost(q, gc, gr, c, kx, ky);
                 put_cell(gr * W + gc, q);
-            } else if (TILE_OK(x, 4, n_state)) {
+            } else if (TILE_OK(x, 4, n_dst)) {
                 st_cell(a.dst + x, out);
             }
             if (own && !solid) {
