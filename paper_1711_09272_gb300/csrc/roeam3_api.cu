@@ -119,10 +119,6 @@ GridCoef3<T> make_coef3(const GridDev3 &q)
     c.mr2 = T(q.m_ref * q.m_ref);
     c.rr_thr = T(1e-5 * q.u_ref);
     c.eps2 = T(q.eps2);
-    c.ax = T(q.dy * q.dz);
-    c.ay = T(q.dx * q.dz);
-    c.az = T(q.dx * q.dy);
-    c.Vi = T(1.0 / (q.dx * q.dy * q.dz));
     c.idx = T(1.0 / q.dx);
     c.idy = T(1.0 / q.dy);
     c.idz = T(1.0 / q.dz);

@@ -29,7 +29,6 @@ struct GridDev3 {
 template <typename T>
 struct GridCoef3 {
     T g, gm1, gm1i, hgm1, mr2, rr_thr, eps2;
-    T ax, ay, az, Vi;            // face areas dy dz, dx dz, dx dy; 1 / (dx dy dz)
     T idx, idy, idz;             // 1/dx, 1/dy, 1/dz
     T inflow[MAX_VARS3];
 };

@@ -131,12 +131,7 @@ template <typename T> __device__ __forceinline__ bool lt(T a, T b) { return a < 
 __device__ __forceinline__ bool ge(double a, double b) { return dbits(a) >= dbits(b); }   // (b >= 0)
 template <typename T> __device__ __forceinline__ bool gt(T a, T b) { return a > b; }
 template <typename T> __device__ __forceinline__ bool ge(T a, T b) { return a >= b; }
-template <typename T> __device__ __forceinline__ bool eq(T a, T b) { return a == b; }
-__device__ __forceinline__ B2 lt(V2 a, V2 b) { return {a.v.x < b.v.x, a.v.y < b.v.y}; }
-__device__ __forceinline__ B2 gt(V2 a, V2 b) { return {a.v.x > b.v.x, a.v.y > b.v.y}; }
 __device__ __forceinline__ B2 ge(V2 a, V2 b) { return {a.v.x >= b.v.x, a.v.y >= b.v.y}; }
-__device__ __forceinline__ B2 eq(V2 a, V2 b) { return {a.v.x == b.v.x, a.v.y == b.v.y}; }
-__device__ __forceinline__ B2 operator&&(B2 a, B2 b) { return {a.x && b.x, a.y && b.y}; }
 template <typename T> __device__ __forceinline__ T sel(bool m, T a, T b) { return m ? a : b; }
 __device__ __forceinline__ V2 sel(B2 m, V2 a, V2 b) { return mk2(m.x ? a.v.x : b.v.x, m.y ? a.v.y : b.v.y); }
 
@@ -207,12 +202,6 @@ __device__ __forceinline__ float vcopysign(float a, float b) { return copysignf(
 __device__ __forceinline__ double vcopysign(double a, double b) { return copysign(a, b); }
 __device__ __forceinline__ V2 vcopysign(V2 a, V2 b) { return mk2(copysignf(a.v.x, b.v.x), copysignf(a.v.y, b.v.y)); }
 
-// sgn with sgn(0) = 0.
-template <typename V> __device__ __forceinline__ V sgnv(V a)
-{
-    const V z = splat<V>(0);
-    return sel(gt(a, z), splat<V>(1), sel(lt(a, z), splat<V>(-1), z));
-}
 template <typename V> __device__ __forceinline__ V pow8(V a) { V a2 = a * a, a4 = a2 * a2; return a4 * a4; }
 
 // Eq. 98: f(phi) = min(phi sqrt(4 + (1 - phi^2)^2) / (1 + phi^2), 1). f(1) = 1 and f = 1 for every

@@ -43,12 +43,6 @@ __device__ __forceinline__ bool tile_ok(long long i, int n, long long size, unsi
 #define TILE_OK(i, n, size) true
 #endif
 
-// Asynchronous copy of one value into shared memory.
-template <typename T> __device__ __forceinline__ void copy_value(T *dst, const T *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"((int)sizeof(T)) : "memory");
-}
-
 template <bool ONE, typename T> __device__ __forceinline__ const GridDev &tile_grid(const TileArgs<T> &a, int g)
 {
     if constexpr (ONE) return a.g0;
@@ -121,14 +115,13 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
     // outside the grid), or the vertex column; [1] the position its cells' values come from (its own but
     // for ghost cells) and their kind (resolve_index) in bits 16 and up. Divisions happen here once, not per position and phase: `recip` holds
     // 2^32 / n + 1 for the width n of every rectangle that a phase covers.
-    __shared__ unsigned recip[4 * STAGES + 2];
-    if (tid < 4 * STAGES + 2) {
-        int n = tid == 4 * STAGES ? W + 1 : W;
-        if (tid < 4 * STAGES) {
+    __shared__ unsigned recip[3 * STAGES + 2];
+    if (tid < 3 * STAGES + 2) {
+        int n = tid == 3 * STAGES ? W + 1 : W;
+        if (tid < 3 * STAGES) {
             int lox, hix, loy, hiy;
-            margin(tid >> 2, lox, hix, loy, hiy);
-            const int p = tid & 3;   // cells with ghosts, ratios, face pairs (or west faces), cells
-            n = hix - lox + (p == 0 ? 2 * H : (p == 1 ? 2 : (p == 2 ? 1 : 0)));
+            margin(tid / 3, lox, hix, loy, hiy);
+            n = hix - lox + 2 - tid % 3;   // ratios, face pairs (or west faces), cells
         }
         recip[tid] = 0xffffffffu / (unsigned)n + 1u;
     }
@@ -161,15 +154,16 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
 
     // vertices do not depend on the launches before this one
     if constexpr (CURV)
-        over(recip[4 * STAGES], 0, W + 1, 0, R + 1, [&](int c, int r) {
+        over(recip[3 * STAGES], 0, W + 1, 0, R + 1, [&](int c, int r) {
             // (a periodic seam's last vertex column repeats the first)
             int i = ix0 + c, j = jy0 + r;
             i = perx && (i < 0 || i > ni) ? CM[2 * c] : clampi(i, 0, ni);
             j = pery && (j < 0 || j > nj) ? RM[2 * r] : clampi(j, 0, nj);
             const long long b = G.voff + (long long)j * G.vpitch + i;
             if (TILE_OK(b, 1, n_vert)) {
-                copy_value(VV + 2 * (r * (W + 1) + c), a.vdx + b);
-                copy_value(VV + 2 * (r * (W + 1) + c) + 1, a.vdy + b);
+                const unsigned d = (unsigned)__cvta_generic_to_shared(VV + 2 * (r * (W + 1) + c));
+                copy_word(d, a.vdx + b);
+                copy_word(d + (unsigned)sizeof(T), a.vdy + b);
             }
         });
     auto vtx = [&](int c, int r, T &x, T &y) { x = VV[2 * (r * (W + 1) + c)]; y = VV[2 * (r * (W + 1) + c) + 1]; };
@@ -197,7 +191,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
         for (int q = tid; q < a.ngrids; q += nt) a.rate_zero[q] = 0ull;
     {
         const unsigned dst = (unsigned)__cvta_generic_to_shared(U);
-        over(recip[4 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
+        over(recip[3 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
             const int i = CM[2 * c], j = RM[2 * r];
             const long long x = G.off + 4 * ((long long)j * pitch + i);
             if ((i | j) >= 0 && TILE_OK(x, 4, n_state))
@@ -206,7 +200,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
         copies_commit();
     }
     if constexpr (WALLS) {
-        const unsigned mw = recip[4 * STAGES + 1];
+        const unsigned mw = recip[3 * STAGES + 1];
         const bool mask = G.soff >= 0;
 #pragma unroll 4
         for (int at = tid; at < P; at += nt) {
@@ -257,7 +251,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
     // (each thread turns the cells that it copied itself into primitives: no barrier in between, but for
     //  the vertices that mirrors at curved walls need)
     if constexpr (CURV && WALLS) __syncthreads();
-    over(recip[4 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
+    over(recip[3 * STAGES + 1], 0, W, 0, R, [&](int c, int r) {
         if ((CM[2 * c] | RM[2 * r]) >= 0) {
             T raw[4];
             WC<T> q;
@@ -281,7 +275,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
     for (int s = 0; s < STAGES; ++s) {
         int lox, hix, loy, hiy;
         margin(s, lox, hix, loy, hiy);
-        const unsigned *const m = recip + 4 * s;
+        const unsigned *const m = recip + 3 * s;
         const T alpha = STAGES == 1 ? a.alpha : (s == 0 ? T(0) : (s == 1 ? T(0.75) : T(1.0 / 3.0)));
         const T beta = STAGES == 1 ? a.beta : (s == 0 ? T(1) : (s == 1 ? T(0.25) : T(2.0 / 3.0)));
         const bool last = s == STAGES - 1;
@@ -327,7 +321,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
         // ---- cells: Eq. 97 ratios of the west and south faces (1 at solid sides), limited slopes
         // (at first order the ratios of the outermost column's west and row's south faces read outside
         //  the stage's cells, but inside shared memory, and are not used)
-        over(m[1], lox - 1, hix + 1, loy - 1, hiy + 1, [&](int c, int r) {
+        over(m[0], lox - 1, hix + 1, loy - 1, hiy + 1, [&](int c, int r) {
             const int at = r * W + c;
             T q[4], qw[4], qs[4];
             ld_own(A1 + 4 * at, q);
@@ -443,7 +437,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
             face_scalar<T, MUSCL>(f, K, eps1, xi_form, vanleer, F);
         };
         if constexpr (PAIRS) {
-            over(m[2], lox, hix + 1, loy, hiy + 1, [&](int c, int r) {
+            over(m[1], lox, hix + 1, loy, hiy + 1, [&](int c, int r) {
                 const int at = r * W + c;
                 V2 s1 = mk2(1.f, 1.f);
                 if (use_s1) s1 = detector_of(mk2(detector_min(at, 1), detector_min(at, W)));
@@ -496,7 +490,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
         } else {
             // west faces, then south faces, one list: every lane has a face
             const int wx = hix + 1 - lox, hx = hiy - loy, nx_ = wx * hx, wyy = hix - lox, ny_ = wyy * (hiy + 1 - loy);
-            const unsigned mx = m[2], my = m[3];
+            const unsigned mx = m[1], my = m[2];
             for (int idx = tid; idx < nx_ + ny_; idx += nt) {
                 const bool isx = idx < nx_;
                 const int k = isx ? idx : idx - nx_, wd = isx ? wx : wyy;
@@ -630,7 +624,7 @@ __global__ void __launch_bounds__(tile_threads<T>()) tile_kernel(const __grid_co
                 }
             }
         };
-        over(m[3], lox, hix, loy, hiy, [&](int c, int r) { update(Flag<false>(), c, r, c, r, 0, 0); });
+        over(m[2], lox, hix, loy, hiy, [&](int c, int r) { update(Flag<false>(), c, r, c, r, 0, 0); });
         if (WALLS && !last && edge)   // (the last threads are idle in the cells' last round)
             ghosts(s + 1, nt - 1 - tid, [&](int c, int r, int cm, int rm) {
                 const int kx = cm >> 16, ky = rm >> 16;
