@@ -284,9 +284,10 @@ roeam_status roeam_flux_residual_noalloc(roeam_grid *g, int grid_idx, double *re
  * warps. (A batch too small to
  * give every resident warp a unit halves the height, down to 4 rows, and on to 2 rows while the
  * units still fit one round of the resident warps.) Results are bit-identical across shapes.
- * Steps of FP64 handles and of FP32 handles of up to about a million cells run in another kernel
- * (rectangles in shared memory), which has no such shapes (FP64 residuals and norms, too): there a
- * shape applies to roeam_rk_stage and, in FP32, to the residual and its norms. */
+ * Steps of FP64 handles, and of FP32 handles too small to fill the chip with strips (a single grid of
+ * up to about 700 x 700 cells, batches of small grids), run in another kernel (rectangles in shared
+ * memory), which has no such shapes (FP64 residuals and norms, too): there a shape applies to
+ * roeam_rk_stage, roeam_step_host and, in FP32, to the residual and its norms. Results are the same bits. */
 int roeam_tile_config_count(void);
 
 /* Describes tile shape `cfg`: strip width tx, segment height ty (cells) and threads per CTA. */

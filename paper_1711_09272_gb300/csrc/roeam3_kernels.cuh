@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(threads3<T>(), 1) stage3_kernel(const StageArg
     else stage3_phases<T, NS>(a);
 }
 // FP32 with three scalars, a single grid: its descriptor and constants are kernel arguments, not registers,
-// of which this kernel has none to spare (192^3: 1072 -> 920 us a step). With fewer scalars the
+// of which this kernel has none to spare (192^3: 1073 -> 931 us a step). With fewer scalars the
 // constants as operands change nothing or lose 0.7 %, nor does FP64 gain.
 template <int NS>
 __global__ void __launch_bounds__(threads3<float>(), 1) stage3_single(const __grid_constant__ StageArgs3<float> a)

@@ -322,7 +322,7 @@ double strip_step_cycles(const roeam_grid *g)
 // 43 / 34; minmod in a box of walls 512^2 47 / 46, 300 of 32^2 56 / 109; warped van Leer with walls and solid
 // cells 300 of 32^2 66 / 145, 600 of 24^2 64 / 117, 16 of 256 x 200 154 / 140.
 // FP64 (a stage per CTA): FP64 operations per face and cell, 76 cycles per warp on each of the four
-// sub-partitions. Tiles win at every size (64^2 33 / 139, 256^2 158 / 277, 1024^2 2228 / 2696; 64 grids of
+// sub-partitions. Tiles win at every size (64^2 32 / 134, 256^2 158 / 267, 1024^2 2224 / 2604; 64 grids of
 // 100 x 80 1151 / 2056, 300 of 32^2 665 / 1485). Counting the rectangles that the even split makes, and full
 // and started passes half and half, and giving the faces a thread each: us per step, first order 100^2 48 ->
 // 39, 128^2 58 -> 51, 256^2 162 -> 158, 800 x 20 58 -> 50; reconstructed 128^2 82 -> 68, 256^2 224 -> 218,

@@ -12,15 +12,15 @@
 // rectangle in the three stages, recomputing what its neighbours also compute, so no CTA waits
 // for another and U^(1), U^(2) never leave shared memory. What bounds a step is then latency and, on
 // the larger grids, instruction issue: of 7 us for a 16 x 6 rectangle, 0.8 are descriptors and maps,
-// 0.5 the load, and a stage takes 0.2 ratios, 0.7 fluxes, 0.5 update. The strips take 17 to 25 us a step
-// on these grids whatever their size (three launches of a few serial row iterations each): 256^2 van
-// Leer 24.5 -> 11.4 us a step, 400^2 corner 32 -> 19, 800 x 20 duct 25 -> 7.0 (7.9 with ghost cells in a
-// phase of their own).
+// 0.5 the load, and a stage takes 0.2 ratios, 0.7 fluxes, 0.5 update. The strips take 11 to 29 us a step
+// on these grids whatever their size (three launches of a few serial row iterations each). Strips and
+// tiles, us a step: 256^2 van Leer 19.0, 11.6, 400^2 corner 25.6, 18.4, 800 x 20 duct 18.1, 7.1 (7.9 with
+// ghost cells in a phase of their own).
 // STAGES = 1 (FP64): one stage per launch. FP64 kernels are bound by the FP64 pipe, so recomputed
 // halos cost time; the phases evaluate each face once per CTA and keep all lanes busy where the
 // strips of a small grid evaluated three rows of faces per two rows of cells. The fluxes take 75 % of
 // a stage and run at the pipe's rate (133 operations per first-order face, about 190 reconstructed).
-// 64^2 139 -> 33 us a step, 256^2 first order 277 -> 158, van Leer 496 -> 238, 1024^2 2696 -> 2227.
+// Strips and tiles, us a step: 64^2 134, 32, 256^2 first order 267, 158, van Leer 483, 234, 1024^2 2604, 2224.
 //
 // In directions that are not periodic the halo ends H cells outside the grid; in periodic ones the
 // halo cells are cells of the other side, which evolve like their originals.
