@@ -1698,7 +1698,10 @@ static cudaError_t launch_pack(const GridDev *grids, int g_lo, int g_hi, int max
                                cudaStream_t s, long long p_shift, const RateOut<T> *ro)
 {
     if (g_hi <= g_lo) return cudaSuccess;
-    const dim3 grid(io_blocks(max_cells, g_hi - g_lo), g_hi - g_lo);
+    // (FP64 rates: a cell per thread up to two blocks per SM; four in a row keep a few SMs busy, and loads queued
+    //  back to back crowd on them: 64^2 19.3 -> 6.8 us, 256^2 46 -> 16, 400^2 52 -> 33)
+    const int bx = io_blocks(max_cells, g_hi - g_lo), most = 304 / (g_hi - g_lo), spread = (max_cells + 255) / 256;
+    const dim3 grid(sizeof(T) == 4 || !ro || bx >= most ? bx : (spread < most ? spread : most), g_hi - g_lo);
     if (!ro) return launch_pdl(pack_kernel<T, H, false, false>, grid, dim3(256), 0, s, grids, g_lo, packed, U, p_shift, RateOut<T>());
     return launch_pdl(ro->curv ? pack_kernel<T, H, true, true> : pack_kernel<T, H, true, false>, grid, dim3(256), 0, s, grids,
                       g_lo, packed, U, p_shift, *ro);
