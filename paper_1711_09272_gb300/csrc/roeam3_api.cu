@@ -156,7 +156,8 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
         max_nk = std::max(max_nk, G.nk);
     }
     const bool f32 = sizeof(T) == 4;
-    const int every = 1 + (g->count - 1) / 16;   // (a sample of a large batch's grids)
+    constexpr int SAMPLES = 16;   // (of a large batch's grids)
+    const int every = 1 + (g->count - 1) / SAMPLES, samples = (g->count + every - 1) / every;
     double best = 1e300;
     int bw = 0, bh = 0, bn = 1;
     // Numbers of segments and the planes of the longest one; of equal planes the fewest segments. (Beyond 96 in
@@ -172,18 +173,17 @@ roeam_status setup_units3(roeam3_grid *g, int num_sms)
         if (cuts.empty() || zs < cuts.back().second) cuts.emplace_back(n, zs);
     }
     auto consider = [&](int w, int h, double plane, double segment, double planes_more) {
-        double planes = 0;   // of all rectangles: their cycles over the SMs bound the cost from below
-        for (int q = 0; q < g->count; q += every) {
-            const GridDev3 &G = g->hg[q];
-            planes += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * G.nk;
+        double columns[SAMPLES];   // rectangles of a plane of each sampled grid
+        double planes = 0;         // of all rectangles: their cycles over the SMs bound the cost from below
+        for (int q = 0; q < samples; ++q) {
+            const GridDev3 &G = g->hg[q * every];
+            columns[q] = (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h);
+            planes += columns[q] * G.nk;
         }
         if (planes * plane / num_sms >= best) return;
         for (const auto &c : cuts) {
             double units = 0;
-            for (int q = 0; q < g->count; q += every) {
-                const GridDev3 &G = g->hg[q];
-                units += (double)every * ((G.ni + w - 1) / w) * ((G.nj + h - 1) / h) * std::min(c.first, G.nk);
-            }
+            for (int q = 0; q < samples; ++q) units += columns[q] * std::min(c.first, g->hg[q * every].nk);
             const double cost = std::ceil(units / num_sms) * (plane * (c.second + planes_more) + segment);
             if (cost < best * 0.999) { best = cost; bw = w; bh = h; bn = c.first; }
         }
